@@ -1549,20 +1549,6 @@ cudaError_t adjoint_step(dvm_ctx *c, AdjWork &w, const T *f, const T *part, cons
     return cudaGetLastError();
 }
 
-// Adds a state in the public layout [cell][comp][p] (a linear objective's
-// dJ/dF^N) to lambda in the padded device layout (interior cells only; the
-// pads stay 0).
-template <typename T>
-__global__ void k_adj_seed(Grid2D g, const T *pub, T *lam)
-{
-    const long k = blockIdx.x;            // one block per cell, threads over (comp, p)
-    const int e = blockIdx.y * blockDim.x + threadIdx.x;
-    if (e >= 2 * g.nv) return;
-    const int comp = e >= g.nv, p = e - comp * g.nv;
-    const long d = ebase<T>(g, comp, p) + pcell(g, k) * Vec<T>::W;
-    lam[d] += pub[k * 2L * g.nv + e];
-}
-
 // The adjoint sweep for J = [with_drag] F_x(F^N) + <seed, F^N>: the drag
 // objective seeds lambda^N through the wall stress and the fusion transpose,
 // a linear functional adds its dJ/dF^N = seed (public layout, host or
@@ -1850,15 +1836,20 @@ int drag_adjoint_t(dvm_ctx *c, int nsteps, int K, double *J, double *gTw, double
             k_adj_fuseT<T><<<dim3((unsigned)w.ncv, nba(2L * c->nvp, 256)), 256, 0, c->stream>>>(a, lamA,
                                                                                               (T *)nullptr);
     }
-    // the public-layout staging buffer of the seed and of lambda^0
-    if ((seed || lam0) && !c->d_pub) AC(cudaMalloc(&c->d_pub, c->state_elems * c->elem));
+    // the public-layout staging buffer of a seed or a lambda^0 that the
+    // layout kernels cannot use in place
+    const bool seed_direct = seed && seed_dev && direct_access(c, seed);
+    const bool lam0_direct = lam0 && lam0_dev && direct_access(c, lam0);
+    if (((seed && !seed_direct) || (lam0 && !lam0_direct)) && !c->d_pub)
+        AC(cudaMalloc(&c->d_pub, c->state_elems * c->elem));
     if (seed) {
         // a linear functional of F^N as the step leaves it (members of a
-        // merged control volume hold its value; no fusion transpose)
-        AC(cudaMemcpyAsync(c->d_pub, seed, c->state_elems * c->elem,
-                           seed_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, c->stream));
-        k_adj_seed<T><<<dim3((unsigned)c->nc, nba(2L * c->nv, 256)), 256, 0, c->stream>>>(grid2d(c),
-                                                                                         (const T *)c->d_pub, lamA);
+        // merged control volume hold its value; no fusion transpose): its
+        // gradient is added to lambda (interior cells; the pads stay 0)
+        if (!seed_direct)
+            AC(cudaMemcpyAsync(c->d_pub, seed, c->state_elems * c->elem,
+                               seed_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, c->stream));
+        AC(add_state(c, seed_direct ? seed : c->d_pub, lamA));
     }
     // reverse sweep, segment by segment: recompute the segment onto the tape
     // (each step writes the next tape buffer) unless the forward run kept it,
@@ -1958,9 +1949,10 @@ int drag_adjoint_t(dvm_ctx *c, int nsteps, int K, double *J, double *gTw, double
     }
     if (lam0) {
         // dJ/dF^0 in the public layout
-        AC(unpack2d(c, w.lam[lin], c->d_pub));
-        AC(cudaMemcpyAsync(lam0, c->d_pub, c->state_elems * c->elem,
-                           lam0_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, c->stream));
+        AC(unpack_state(c, w.lam[lin], lam0_direct ? lam0 : c->d_pub));
+        if (!lam0_direct)
+            AC(cudaMemcpyAsync(lam0, c->d_pub, c->state_elems * c->elem,
+                               lam0_dev ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, c->stream));
     }
     if (gprim0) {
         if (!c->have_prim0) { set_error("dvm_drag_adjoint: gprim0 needs a state set by dvm_init_maxwellian"); return DVM_ERR_STATE; }

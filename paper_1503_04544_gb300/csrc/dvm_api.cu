@@ -171,8 +171,6 @@ static cudaError_t st_ghost(dvm_ctx *c, int side, const double *d, int n)
 static cudaError_t st_halo(dvm_ctx *c, int buf) { return c->dim == 2 ? halo2d(c, buf) : halo3d(c, buf); }
 static cudaError_t st_zero_solid(dvm_ctx *c) { return c->dim == 2 ? zero_solid2d(c) : zero_solid3d(c); }
 static cudaError_t st_partials(dvm_ctx *c) { return c->dim == 2 ? partials_from_state2d(c) : partials_from_state3d(c); }
-static cudaError_t st_pack(dvm_ctx *c, const void *pub, void *dev) { return c->dim == 2 ? pack2d(c, pub, dev) : pack3d(c, pub, dev); }
-static cudaError_t st_unpack(dvm_ctx *c, const void *dev, void *pub) { return c->dim == 2 ? unpack2d(c, dev, pub) : unpack3d(c, dev, pub); }
 namespace dvm {
 cudaError_t shakhov3d(dvm_ctx *c);   // the Shakhov term of the 3D step (dvm_shakhov3d.cu)
 }
@@ -715,15 +713,22 @@ static int ensure_pub(dvm_ctx *c)
     return DVM_OK;
 }
 
+// A device array on this context's device is converted in place; a host array
+// (or one a kernel here cannot read) passes through the staging buffer.
+
 int dvm_set_state(dvm_ctx *c, const void *f, size_t bytes, int on_device)
 {
     if (!c || !f) { set_error("null"); return DVM_ERR_ARG; }
     if (split_step_open(c, "dvm_set_state")) return DVM_ERR_STATE;
     if (bytes != c->state_elems * c->elem) { set_error("state size mismatch"); return DVM_ERR_ARG; }
-    int rc = ensure_pub(c);
-    if (rc != DVM_OK) return rc;
-    CK(cudaMemcpyAsync(c->d_pub, f, bytes, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, c->stream));
-    CK(st_pack(c, c->d_pub, c->f[c->cur]));
+    if (on_device && direct_access(c, f)) {
+        CK(pack_state(c, f, c->f[c->cur]));
+    } else {
+        int rc = ensure_pub(c);
+        if (rc != DVM_OK) return rc;
+        CK(cudaMemcpyAsync(c->d_pub, f, bytes, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, c->stream));
+        CK(pack_state(c, c->d_pub, c->f[c->cur]));
+    }
     c->have_prim0 = false;
     CK(st_zero_solid(c));
     CK(st_halo(c, c->cur));
@@ -739,10 +744,14 @@ int dvm_get_state(dvm_ctx *c, void *f, size_t bytes, int on_device)
 {
     if (!c || !f) { set_error("null"); return DVM_ERR_ARG; }
     if (bytes != c->state_elems * c->elem) { set_error("state size mismatch"); return DVM_ERR_ARG; }
-    int rc = ensure_pub(c);
-    if (rc != DVM_OK) return rc;
-    CK(st_unpack(c, c->f[c->cur], c->d_pub));
-    CK(cudaMemcpyAsync(f, c->d_pub, bytes, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, c->stream));
+    if (on_device && direct_access(c, f)) {
+        CK(unpack_state(c, c->f[c->cur], f));
+    } else {
+        int rc = ensure_pub(c);
+        if (rc != DVM_OK) return rc;
+        CK(unpack_state(c, c->f[c->cur], c->d_pub));
+        CK(cudaMemcpyAsync(f, c->d_pub, bytes, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyDeviceToHost, c->stream));
+    }
     CK(cudaStreamSynchronize(c->stream));
     return DVM_OK;
 }

@@ -234,8 +234,11 @@ cudaError_t fusion2d(dvm_ctx *c, void *f, void *part);          // Eq. FusionDD 
 cudaError_t mass2d(dvm_ctx *c, double *d_scratch, double *d_out);
 cudaError_t moments_out2d(dvm_ctx *c, double *d_out);
 cudaError_t ghost2d(dvm_ctx *c, int side, const double *d_prim, int nside);
-cudaError_t pack2d(dvm_ctx *c, const void *pub, void *dev);      // public -> device layout
-cudaError_t unpack2d(dvm_ctx *c, const void *dev, void *pub);    // device -> public layout
+// public and device layout (dvm_layout.cu)
+cudaError_t pack_state(dvm_ctx *c, const void *pub, void *dev);      // public -> device
+cudaError_t unpack_state(dvm_ctx *c, const void *dev, void *pub);    // device -> public
+cudaError_t add_state(dvm_ctx *c, const void *pub, void *dev);       // dev += public
+bool direct_access(const dvm_ctx *c, const void *p);                 // a caller's array usable in place
 cudaError_t zero_solid2d(dvm_ctx *c);                            // both state buffers
 cudaError_t halo2d(dvm_ctx *c, int buf);                         // periodic / zero-gradient padding
 cudaError_t members2d(dvm_ctx *c, bool moving);                  // control-volume records
@@ -264,8 +267,6 @@ cudaError_t step3d(dvm_ctx *c);
 cudaError_t mass3d(dvm_ctx *c, double *d_scratch, double *d_out);
 cudaError_t moments_out3d(dvm_ctx *c, double *d_out);
 cudaError_t ghost3d(dvm_ctx *c, int side, const double *d_prim, int nside);
-cudaError_t pack3d(dvm_ctx *c, const void *pub, void *dev);
-cudaError_t unpack3d(dvm_ctx *c, const void *dev, void *pub);
 cudaError_t zero_solid3d(dvm_ctx *c);
 cudaError_t halo3d(dvm_ctx *c, int buf);
 size_t vtab3_bytes(const dvm_ctx *c);

@@ -1566,16 +1566,15 @@ __global__ void k_ghost(Grid2D g, const double *prim, int side, int nside, T *f0
 
 // Padding of periodic and zero-gradient sides from the interior of a state
 // buffer (both layers, every group and component).
+// One thread copies one group's vector of one component.
 template <typename T>
 __global__ void k_halo(Grid2D g, T *f)
 {
-    constexpr int W = Vec<T>::W;
+    using V = typename Vec<T>::type;
     const long per = 2L * (g.nx + g.ny);      // padding cells of one layer (cross arms)
     const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= 2 * per * 2 * g.nvp) return;
+    if (t >= 2 * per * 2 * g.ngrp) return;
     const long hc = t % (2 * per);            // padding cell: layer, side, position
-    const long rest = t / (2 * per);
-    const int comp = (int)(rest % 2), p = (int)(rest / 2);
     const int layer = (int)(hc / per) + 1;
     long pos = hc % per;
     int side, q;
@@ -1590,22 +1589,8 @@ __global__ void k_halo(Grid2D g, T *f)
     else if (side == 1) { di = g.nx - 1 + layer; dj = q; si = kind == DVM_BC_PERIODIC ? layer - 1 : g.nx - 1; sj = q; }
     else if (side == 2) { di = q; dj = -layer; si = q; sj = kind == DVM_BC_PERIODIC ? g.ny - layer : 0; }
     else { di = q; dj = g.ny - 1 + layer; si = q; sj = kind == DVM_BC_PERIODIC ? layer - 1 : g.ny - 1; }
-    const long base = ((long)(p / W) * 2 + comp) * g.slab * W + (p % W);
-    f[base + nbr(g, di, dj) * W] = f[base + nbr(g, si, sj) * W];
-}
-
-// Conversion between the public layout [cell][comp][p] and the device layout.
-template <typename T>
-__global__ void k_pack(Grid2D g, const T *src, T *dst, int to_dev)
-{
-    const long k = blockIdx.x;            // one block per cell, threads over (comp, p)
-    const int e = blockIdx.y * blockDim.x + threadIdx.x;
-    if (e >= 2 * g.nv) return;
-    const int comp = e >= g.nv, p = e - comp * g.nv;
-    const long t = k * 2L * g.nv + e;
-    const long d = ebase<T>(g, comp, p) + pcell(g, k) * Vec<T>::W;
-    if (to_dev) dst[d] = src[t];
-    else dst[t] = src[d];
+    V *const slab = reinterpret_cast<V *>(f) + t / (2 * per) * g.slab;   // (group, component)
+    slab[nbr(g, di, dj)] = slab[nbr(g, si, sj)];
 }
 
 // Zero the state of every solid cell (they belong to no control volume): one
@@ -2134,17 +2119,6 @@ cudaError_t ghost2d(dvm_ctx *c, int side, const double *d_prim, int nside)
     return cudaGetLastError();
 }
 
-cudaError_t pack2d(dvm_ctx *c, const void *pub, void *dev)
-{
-    Grid2D g = grid2d(c);
-    dim3 grid((unsigned)(c->nx * c->ny), nblk(2 * c->nv, 256));
-    if (c->prec == DVM_FP32)
-        k_pack<float><<<grid, 256, 0, c->stream>>>(g, (const float *)pub, (float *)dev, 1);
-    else
-        k_pack<double><<<grid, 256, 0, c->stream>>>(g, (const double *)pub, (double *)dev, 1);
-    return cudaGetLastError();
-}
-
 cudaError_t zero_solid2d(dvm_ctx *c)
 {
     Grid2D g = grid2d(c);
@@ -2161,20 +2135,9 @@ cudaError_t zero_solid2d(dvm_ctx *c)
 cudaError_t halo2d(dvm_ctx *c, int buf)
 {
     Grid2D g = grid2d(c);
-    const long n = 2 * 2L * (c->nx + c->ny) * 2 * c->nvp;
+    const long n = 2 * 2L * (c->nx + c->ny) * 2 * c->ngrp;
     if (c->prec == DVM_FP32) k_halo<float><<<nblk(n, 256), 256, 0, c->stream>>>(g, (float *)c->f[buf]);
     else k_halo<double><<<nblk(n, 256), 256, 0, c->stream>>>(g, (double *)c->f[buf]);
-    return cudaGetLastError();
-}
-
-cudaError_t unpack2d(dvm_ctx *c, const void *dev, void *pub)
-{
-    Grid2D g = grid2d(c);
-    dim3 grid((unsigned)(c->nx * c->ny), nblk(2 * c->nv, 256));
-    if (c->prec == DVM_FP32)
-        k_pack<float><<<grid, 256, 0, c->stream>>>(g, (const float *)dev, (float *)pub, 0);
-    else
-        k_pack<double><<<grid, 256, 0, c->stream>>>(g, (const double *)dev, (double *)pub, 0);
     return cudaGetLastError();
 }
 
