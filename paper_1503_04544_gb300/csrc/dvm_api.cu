@@ -349,20 +349,18 @@ int dvm_create(const dvm_grid *grid, const dvm_vgrid *vg, const dvm_physics *ph,
         }
         c->S = S;
     } else {
-        // one resident block per SM (tiles of 32 x 11 cells in FP32, 32 x 8 in
-        // FP64, columns of 4 cells): the smallest split count giving at least
-        // four waves on 152 SMs with a last wave at least 95% full, else the
-        // best-filled count up to 24
-        const long slots = 152;
-        const int rows = precision == DVM_FP32 ? 11 : 8;
-        const long blocks = (long)((c->nx + 31) / 32) * ((c->ny + rows - 1) / rows) * ((c->nz + 3) / 4);
+        // one resident block per SM; a block's prologue (per-cell data,
+        // pipeline fill) is worth about 12 groups, and blocks near the
+        // obstacle take longer, so half a block beyond the average is left
+        // for the tail: FP64 40^3 x 12^3 (70 blocks, 864 groups): S = 2, one
+        // full wave, 10.6 ms a launch; 3: 11.4; 5: 9.5; 8: 7.7
+        const double blocks = bulk3_blocks(c);
         int best = 1;
-        double best_eff = 0;
+        double least = -1;
         for (int S = 1; S <= 24 && S <= c->ngrp; ++S) {
-            const long nb = blocks * S, waves = (nb + slots - 1) / slots;
-            const double eff = (double)nb / ((double)slots * waves);
-            if (waves >= 4 && eff >= 0.95) { best = S; break; }
-            if (eff > best_eff + 1e-9) { best_eff = eff; best = S; }
+            const double per_sm = blocks * S / 152;
+            const double cost = std::fmax(std::ceil(per_sm), per_sm + 0.5) * ((c->ngrp + S - 1) / S + 12);
+            if (least < 0 || cost < least) { least = cost; best = S; }
         }
         c->S = best;
     }
@@ -885,10 +883,11 @@ int dvm_load(dvm_ctx *c, const char *path)
     bool ok = std::fread(&h, sizeof(h), 1, fp) == 1 && std::memcmp(h.magic, kCkptMagic, 8) == 0 &&
               h.version == kCkptVersion;
     // the checkpoint must come from a context of the same problem
-    ok = ok && h.dim == c->dim && h.precision == c->prec && h.scheme == c->scheme && h.S == c->S &&
+    // (the number of velocity splits may differ: it only groups the sums)
+    ok = ok && h.dim == c->dim && h.precision == c->prec && h.scheme == c->scheme && h.S >= 1 && h.S <= c->ngrp &&
          h.nx == c->nx && h.ny == c->ny && h.nz == c->nz && h.nvx == c->nvx && h.nvy == c->nvy &&
          h.nvz == c->nvz && h.shape == c->body.shape && h.movable == c->body.movable && h.dt == c->dt &&
-         h.tau0 == c->tau0 && h.state_bytes == c->state_elems * c->elem && h.part_bytes == part_bytes(c) &&
+         h.tau0 == c->tau0 && h.state_bytes == c->state_elems * c->elem && h.part_bytes == part_bytes(c) / c->S * h.S &&
          h.body_bytes == sizeof(dvm::BodyDev) && (h.time_scheme == DVM_EXPLICIT || h.time_scheme == DVM_IMEX) &&
          h.model == c->model && h.problem == mine;
     if (ok) {
@@ -914,7 +913,22 @@ int dvm_load(dvm_ctx *c, const char *path)
     }
     int rc = dvm_set_state(c, state.data(), state.size(), 0);
     if (rc != DVM_OK) return rc;
-    // the saved partial sums, not ones recomputed from the state
+    // the saved partial sums, not ones recomputed from the state; those of
+    // another split count fill this context's first slots (a slot holds
+    // nothing but a summand of the cell's moments), any more are added to them
+    if (h.S != c->S) {
+        const size_t slot = part_bytes(c) / c->S;
+        std::vector<char> mine_parts(part_bytes(c), 0);
+        std::memcpy(mine_parts.data(), part.data(), slot * (h.S < c->S ? h.S : c->S));
+        for (int q = c->S; q < h.S; ++q)
+            for (size_t n = 0; n < slot; n += c->elem) {
+                char *d = mine_parts.data() + (q % c->S) * slot + n;
+                const char *s = part.data() + q * slot + n;
+                if (c->elem == 4) *reinterpret_cast<float *>(d) += *reinterpret_cast<const float *>(s);
+                else *reinterpret_cast<double *>(d) += *reinterpret_cast<const double *>(s);
+            }
+        part.swap(mine_parts);
+    }
     CK(cudaMemcpyAsync(c->part[c->cur], part.data(), part.size(), cudaMemcpyHostToDevice, c->stream));
     c->need_fusion = h.need_fusion != 0;
     c->steps_done = h.steps_done;

@@ -185,6 +185,16 @@ __device__ __forceinline__ float minmod3(float a, float b)
     return xorsign(fmaxf(min_xorsign_abs(a, b), 0.f), a);
 }
 
+// The bits of |x|.  Written as an instruction of its own: the compiler turns
+// the masked bit pattern of a double into fabs, which runs on the FP64 pipe
+// (8 of the 34 FP64 operations a velocity of the 3D update took).
+__device__ __forceinline__ unsigned long long magnitude_bits(double x)
+{
+    unsigned long long m;
+    asm("and.b64 %0, %1, 0x7FFFFFFFFFFFFFFF;" : "=l"(m) : "l"(__double_as_longlong(x)));
+    return m;
+}
+
 // The same for FP64 with integer operations on the bit patterns: the
 // magnitudes of IEEE-754 doubles order as their bits without the sign, and
 // the result is one of the arguments or zero, so it is exact (a zero result
@@ -193,8 +203,7 @@ __device__ __forceinline__ float minmod3(float a, float b)
 __device__ __forceinline__ double minmod3(double a, double b)
 {
     const long long ia = __double_as_longlong(a), ib = __double_as_longlong(b);
-    const unsigned long long ma = (unsigned long long)ia & 0x7FFFFFFFFFFFFFFFull;
-    const unsigned long long mb = (unsigned long long)ib & 0x7FFFFFFFFFFFFFFFull;
+    const unsigned long long ma = magnitude_bits(a), mb = magnitude_bits(b);
     const long long r = ma <= mb ? ia : ib;
     return (ia ^ ib) < 0 ? 0.0 : __longlong_as_double(r);
 }
@@ -221,6 +230,73 @@ __device__ __forceinline__ void minmod_mag_pair(float b, float a, float c, float
 {
     mo = fmaxf(min_xorsign_abs(b, a), 0.f);
     mi = fmaxf(min_xorsign_abs(a, c), 0.f);
+}
+
+// ---- lanes of a velocity group: the arithmetic of the bulk kernels on the
+// units the state precision has, a pair of FP32 velocities (f32x2) or one
+// FP64 velocity; a group is two units in both precisions.
+template <typename T> struct Lanes;
+template <> struct Lanes<float> { using P = F2; static constexpr int N = 2; };
+template <> struct Lanes<double> { using P = double; static constexpr int N = 1; };
+
+__device__ __forceinline__ double add2(double a, double b) { return a + b; }
+__device__ __forceinline__ double sub2(double a, double b) { return a - b; }
+__device__ __forceinline__ double mul2(double a, double b) { return a * b; }
+__device__ __forceinline__ double fma2(double a, double b, double c) { return fma(a, b, c); }
+
+// The two units of a group's vector at p (shared or global memory).
+__device__ __forceinline__ void ld_units(const float4 *p, F2 (&r)[2])
+{
+    const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(p);
+    r[0].v = v.x;
+    r[1].v = v.y;
+}
+__device__ __forceinline__ void ld_units(const double2 *p, double (&r)[2])
+{
+    const double2 v = *p;
+    r[0] = v.x;
+    r[1] = v.y;
+}
+// One unit of the vector at p.
+__device__ __forceinline__ F2 ld_unit(const float4 *p, int h)
+{
+    F2 r;
+    r.v = reinterpret_cast<const unsigned long long *>(p)[h];
+    return r;
+}
+__device__ __forceinline__ double ld_unit(const double2 *p, int h) { return reinterpret_cast<const double *>(p)[h]; }
+
+// minmod(b, a) of every lane, with its sign.
+__device__ __forceinline__ F2 minmod2(F2 b, F2 a)
+{
+    float b0, b1, a0, a1;
+    f2_get(b, b0, b1);
+    f2_get(a, a0, a1);
+    return f2(minmod3(b0, a0), minmod3(b1, a1));
+}
+__device__ __forceinline__ double minmod2(double b, double a) { return minmod3(b, a); }
+
+// minmod(b, a) - minmod(a, c): the two limiter values of an axis.  FP32: both
+// carry the sign of a where they are not zero, so the difference is that of
+// the magnitudes with the sign of a (five min/max/bit operations per lane).
+__device__ __forceinline__ double minmod_diff(double b, double a, double c) { return minmod3(b, a) - minmod3(a, c); }
+
+// wo minmod(b, a) - wi minmod(a, c) with face weights wo, wi >= 0.
+__device__ __forceinline__ double minmod_diff(double b, double a, double c, double wo, double nwi)
+{
+    return fma(nwi, minmod3(a, c), wo * minmod3(b, a));
+}
+__device__ __forceinline__ float minmod_diff(float b, float a, float c)
+{
+    float o, i;
+    minmod_mag_pair(b, a, c, o, i);
+    return xorsign(o - i, a);
+}
+__device__ __forceinline__ float minmod_diff(float b, float a, float c, float wo, float nwi)
+{
+    float o, i;
+    minmod_mag_pair(b, a, c, o, i);
+    return xorsign(fmaf(nwi, i, wo * o), a);
 }
 
 // 2^x by the hardware approximation (relative error a few ulp; results below
@@ -279,6 +355,39 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity)
     for (long it = 0; it < kWaitLimit; ++it)
         if (mbar_try_wait(bar, parity)) return true;
     return false;
+}
+
+// The same with the fast path first and the outcome or-ed into bad (1 after
+// a timeout), for loops that wait often: one poll and a branch when the phase
+// has completed.  bar: shared-memory address.
+__device__ __forceinline__ void mbar_wait_or(uint32_t bar, uint32_t parity, uint32_t &bad)
+{
+    static_assert(kWaitLimit == 1L << 20, "the poll limit below");
+    asm volatile(
+        "{\n\t.reg .pred p;\n\t.reg .u32 n;\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "@p bra DONE;\n\t"
+        "mov.u32 n, 1048576;\n\t"
+        "POLL:\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "@p bra DONE;\n\t"
+        "sub.u32 n, n, 1;\n\t"
+        "setp.ne.u32 p, n, 0;\n\t"
+        "@p bra POLL;\n\t"
+        "mov.u32 %0, 1;\n\t"
+        "DONE:\n\t}"
+        : "+r"(bad)
+        : "r"(bar), "r"(parity)
+        : "memory");
+}
+
+// Arrival on an mbarrier by the lanes with on != 0, without a branch.
+__device__ __forceinline__ void mbar_arrive_if(uint32_t bar, uint32_t on)
+{
+    asm volatile(
+        "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %1, 0;\n\t"
+        "@p mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}" ::"r"(bar), "r"(on)
+        : "memory");
 }
 
 __device__ __forceinline__ void tma_load_3d(void *dst, const CUtensorMap *map, uint64_t *bar, int x, int y, int z)

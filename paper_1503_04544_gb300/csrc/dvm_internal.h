@@ -271,6 +271,8 @@ cudaError_t zero_solid3d(dvm_ctx *c);
 cudaError_t halo3d(dvm_ctx *c, int buf);
 size_t vtab3_bytes(const dvm_ctx *c);
 int make_tensor_maps3d(dvm_ctx *c);                // TMA descriptors of f[0], f[1] (3D)
+void tile3d(const dvm_ctx *c, int *tx, int *ty);   // tile of the 3D bulk kernel
+int bulk3_blocks(const dvm_ctx *c);                // its blocks for one velocity split
 size_t cvinfo3_bytes();
 
 // Limiter-branch words of the 2D MUSCL step (recorded for the adjoint): one

@@ -26,14 +26,12 @@
 
 #include <cstdio>
 #include <string>
+#include <type_traits>
 
 #include "dvm_device.cuh"
 
 namespace dvm {
 namespace {
-
-constexpr int kCoef3 = 6;            // per-cell coefficients of the bulk kernel
-constexpr int kCoef3S = 11;          // the same with the Shakhov model's five
 
 template <typename T> struct alignas(2 * sizeof(T)) VX3 { T vx, nux; };
 template <typename T> struct alignas(4 * sizeof(T)) VYZ3 { T vy, vz, nuy, nuz; };
@@ -66,12 +64,6 @@ __device__ __forceinline__ long pidx3(const Grid3D &g, int p, int pc)
     return ((long)grp * g.slab + pc) * g.W + (p - grp * g.W);
 }
 
-// Padded index of public velocity p = (p3 nvy + p2) nvx + p1.
-__device__ __forceinline__ int padded3(const Grid3D &g, int p)
-{
-    const int r = p / g.nvx;
-    return r * g.nvxp + (p - r * g.nvx);
-}
 
 // Padding cells that mirror interior cell (i, j, k) on periodic and
 // zero-gradient sides (two per axis at most); -1 where unused.
@@ -102,10 +94,6 @@ __device__ __forceinline__ void mirrors3(const Grid3D &g, int i, int j, int k, i
     }
 }
 
-__device__ __forceinline__ bool near_side3(const Grid3D &g, int i, int j, int k)
-{
-    return i < 2 || i >= g.nx - 2 || j < 2 || j >= g.ny - 2 || k < 2 || k >= g.nz - 2;
-}
 
 // Primitive variables from the sums s0 = sum F, s1..3 = sum v F,
 // s4 = sum |v|^2/2 F (Eq. MacroscopicTD; T from E = rho|u|^2/2 + 3/2 rho T).
@@ -144,6 +132,7 @@ __device__ __forceinline__ T norm3(T tmp)
 template <typename T> struct Bulk3Args {
     Grid3D g;
     int S, nzc;
+    int tx, ty;               // tile of cells (tile3d)
     int Sin;                  // partial-sum slots of pin (S, or 1 for summed moments of a velocity split)
     const T *fin;
     T *fout;
@@ -159,30 +148,40 @@ template <typename T> struct Bulk3Args {
 };
 
 constexpr int kZc3 = 4;                           // z-planes per block column
-constexpr int kRing3 = 8;                         // shared-memory planes in flight
-constexpr int kPlaneX = 32 + 4;                   // tile width plus a two-cell halo
+constexpr int kPlanes3 = kZc3 + 3;                // planes of a column: two upwind, the cells, one downwind
 
-// Tile rows of the bulk kernel (one consumer warp each): 11 in FP32, so that
-// with the producer warp the block's 12 warps put 3 on each SM sub-partition
-// and a thread may hold up to 168 registers (it uses about 160, without
-// spills; 12 rows would cap it at 128); 8 in FP64 (shared memory of the
-// per-cell state).
-template <typename T> __host__ __device__ constexpr int rows3() { return sizeof(T) == 4 ? 11 : 8; }
-template <typename T> __host__ __device__ constexpr int plane_cells3() { return kPlaneX * (rows3<T>() + 4); }
-// Ring slot stride in 16-byte cells: every slot is the destination of a
+// Warps of the bulk kernel's block.  FP32: 16, the most that leave a thread
+// 128 registers.  FP64: 8 (shared memory of the per-cell data; the kernel is
+// bound by the FP64 pipe).
+template <typename T> __host__ __device__ constexpr int warps3() { return sizeof(T) == 4 ? 16 : 8; }
+// Ring slot stride in 16-byte cells: the most cells of a plane, tile and
+// two-cell halo (tile3d keeps to it).  Every slot is the destination of a
 // tensor copy and starts on a 128-byte boundary.
-template <typename T> __host__ __device__ constexpr int plane_stride3() { return (plane_cells3<T>() * 16 + 127) / 128 * 8; }
+template <typename T> __host__ __device__ constexpr int plane_stride3() { return sizeof(T) == 4 ? 816 : 448; }
 
-// Velocity tables staged in shared memory by the bulk kernel: all of v_x and
-// up to kVyzStage (v_y, v_z) pairs (more are read from global memory).
-constexpr int kVyzStage = 512;
+// Ring slots: the planes of a whole group, so that plane o of every group has
+// its own slot; the Shakhov variant has room for five.
+template <bool SHAK> __host__ __device__ constexpr int ring3() { return SHAK?5:kPlanes3; }
+
+// Per-cell values of the bulk kernel in shared memory.  FP32: c0, c1, c2, r
+// (one vector), uy, uz, and the Shakhov model's k q.  FP64: the values of
+// MxSlot for the Maxwellian's recurrence along v_x.
+constexpr int kMxBlocks = 4;         // restarts of the recurrence along a v_x row
+enum MxSlot { kMxUy = 0, kMxUz, kMxC2, kMxOmr, kMxQ, kMxM, kMxR = kMxM + kMxBlocks, kMxCount = kMxR + kMxBlocks };
+template <typename T, bool SHAK> __host__ __device__ constexpr int ncoef3()
+{
+    return sizeof(T) == 8 ? kMxCount : (SHAK ? 9 : 6);
+}
+// Compensated sums in FP32 (sum, compensation), plain in FP64.
+template <typename T> __host__ __device__ constexpr int nsum3() { return sizeof(T) == 4 ? 10 : 5; }
 
 template <typename T, bool SHAK>
 size_t bulk3_smem()
 {
-    const int ncoef = SHAK ? kCoef3S : kCoef3;
-    return (size_t)kRing3 * plane_stride3<T>() * 16 + (size_t)kZc3 * (ncoef + 10) * 32 * rows3<T>() * sizeof(T) +
-           2 * kRing3 * sizeof(uint64_t) + (size_t)kMaxAxisNv * sizeof(VX3<T>) + (size_t)kVyzStage * sizeof(VYZ3<T>);
+    return (size_t)ring3<SHAK>() * plane_stride3<T>() * 16 +
+           (size_t)kZc3 * (ncoef3<T, SHAK>() + nsum3<T>()) * 32 * warps3<T>() * sizeof(T) +
+           32 * warps3<T>() * sizeof(uint32_t) +
+           (size_t)(kMaxAxisNv / Vec<T>::W) * (4 * 16 + 8) + 2 * ring3<SHAK>() * sizeof(uint64_t);
 }
 
 __device__ __forceinline__ void tma_load_4d(void *dst, const CUtensorMap *map, uint64_t *bar, int x, int y, int z, int w)
@@ -194,67 +193,85 @@ __device__ __forceinline__ void tma_load_4d(void *dst, const CUtensorMap *map, u
         : "memory");
 }
 
-// Flux difference along one axis in units of the Courant number on a full gas
-// cell (Eq. eq-schema3D), with the neighbours taken on the upwind side:
-// a = F - F_up plus the limited reconstructions of the outgoing and incoming
-// faces; ko, ki are (1 - nu)/2 where the face stencil is all gas, else 0.
-template <typename T, bool MUSCL>
-__device__ __forceinline__ T dflux(T f, T u1, T u2, T d1, T ko, T ki)
-{
-    const T a = f - u1;
-    if (!MUSCL) return a;
-    T mo, mi;
-    minmod_pair(d1 - f, a, u1 - u2, mo, mi);
-    return fma(-ki, mi, fma(ko, mo, a));
-}
-
 // 2^x in the state precision: the hardware approximation in FP32.
 __device__ __forceinline__ float exp2_state(float x) { return ex2_fast(x); }
 __device__ __forceinline__ double exp2_state(double x) { return exp2(x); }
 
+// Lane l of a unit.
+__device__ __forceinline__ float unit_lane(F2 x, int l) { float a, b; f2_get(x, a, b); return l ? b : a; }
+__device__ __forceinline__ double unit_lane(double x, int) { return x; }
+
 // Bulk update of every gas cell that is a control volume on its own.
 //
-// Block = a tile of 32 x R cells in (x, y) and a column of kZc3 cells in z
-// (blockIdx.z = split * nzc + column), R consumer warps (one per tile row)
-// and one producer warp.  For each velocity group of its split the producer
-// streams the kZc3 + 4 planes of the column (tile plus a two-cell halo, one
-// TMA load each) into a ring of kRing3 shared-memory stages, refilling a stage
-// once every consumer warp has released it.  The consumers march up the
-// column: x/y neighbours come from the plane's stage; along z the cell values,
-// their differences and the face value at z + 1/2 (the z - 1/2 face of the
-// next cell) roll through registers.  Every wait is bounded and records
-// kErrTimeout instead of blocking.  The neighbours of a group are taken on its
-// upwind side (uniform within a group along y and z, and along x except for
-// the group that contains v_x = 0).  Moments of the new state are summed per
-// cell in registers over 8 groups, then folded into compensated sums in
-// shared memory.
+// Block = a tile of a.tx x a.ty cells in (x, y), taken row by row by the
+// threads (tile3d), and a column of kZc3 cells in z (blockIdx.z = split * nzc + column); R warps.  For
+// each velocity group of its split the planes of the column (tile plus a
+// two-cell halo, one TMA load each) stream through a ring of shared-memory
+// slots in upwind order of v_z.  Thread 0 refills the slot that its warp
+// released two planes ago, once every warp has released it (a producer warp
+// of its own would take the 17th warp's registers from all: 96 a thread and
+// spills).  Every wait is bounded and records kErrTimeout instead of blocking.
+//
+// A thread marches its column downwind: along z the centre, the upwind
+// difference and the limited slope of the upwind face roll through registers,
+// so that each face is formed once and the group needs two upwind planes and
+// one downwind plane beside its cells; x and y neighbours come from the
+// plane's slot, on the group's upwind side.  The arithmetic runs on units of
+// the group (pairs of FP32 velocities, f32x2).  Warps whose 32 cells all have
+// the limiter on every face take the path without face weights, the others
+// (near the obstacle) the one with weights; a group whose v_x changes sign
+// within a unit goes velocity by velocity.  The weighted path has to be nearly
+// as fast: one slow warp holds up its whole block at the ring.
+//
+// Moments: v_y and v_z are uniform in a row of groups, so a cell sums F,
+// v_x F and v_x^2 F over the row and forms the five moments once per row,
+// into compensated sums in shared memory.
+//
+// FP64: the Maxwellian along the row by the recurrence M(v + dv) = M R,
+// R(v + dv) = R Q, restarted every 8 velocities (16 from 33 velocities per
+// axis on) from per-cell values of the v_x factor, times the row's factor of
+// v_y and v_z (one exp2 a row): two FP64 multiplications a velocity instead of
+// an exp2.  Relative error below 30 ulp (130 for 33 and more velocities).
+//
+// FP32 is bound by issue slots (70 warp instructions a velocity and 32 cells,
+// 24 of them on the half-rate ALU pipe) and by waits for planes; FP64 by the
+// FP64 pipe (two lanes a clock; 26 operations a velocity).  The form before
+// this one (a thread per column in fixed z order, both z faces' planes read,
+// exp2 per velocity, velocity by velocity moments) took, a launch: FP32 64^3 x
+// 20^3 9.72 ms, now 7.2; 96^3 x 20^3 30.6, now 23.4; Shakhov 45 x 50 x 37 x
+// (14, 15, 13) 2.13, now 1.53; FP64 40^3 x 12^3 20.8, now 7.7.
+//
 // With SHAK (the Shakhov model, FP32) the cells relax towards F_S = M [1 +
 // k c.q (|c|^2/T - 5)], k = (1 - Pr) / (5 rho T^2), with the heat flux q of
 // the cell at t^n from k_heatflux3: |c|^2/T from the Maxwellian's base-2
-// exponent and k c.q linear in v, four operations per velocity.
+// exponent and k c.q linear in v.
 template <typename T, bool MUSCL, bool SHAK>
-__global__ void __launch_bounds__(32 * (rows3<T>() + 1), 1)
+__global__ void __launch_bounds__(32 * warps3<T>(), 1)
     k_bulk3(Bulk3Args<T> a, const __grid_constant__ CUtensorMap tmap)
 {
     static_assert(!SHAK || sizeof(T) == 4, "the Shakhov variant of the bulk kernel is FP32");
-    constexpr int W = Vec<T>::W, ZC = kZc3, R = rows3<T>(), NT = 32 * R, NP = ZC + 4;
-    constexpr int NCO = SHAK ? kCoef3S : kCoef3;
-    constexpr int PC = plane_stride3<T>(), PB = plane_cells3<T>() * 16;
-    static_assert((PC * 16) % 128 == 0, "tensor-copy destinations start on 128-byte boundaries");
     using V = typename Vec<T>::type;
+    using P = typename Lanes<T>::P;
+    constexpr int W = Vec<T>::W, LN = Lanes<T>::N, ZC = kZc3, R = warps3<T>(), NT = 32 * R, NP = kPlanes3;
+    constexpr int RING = ring3<SHAK>(), NCO = ncoef3<T, SHAK>(), NSUM = nsum3<T>();
+    constexpr int PC = plane_stride3<T>();
+    constexpr bool F64 = sizeof(T) == 8;
+    static_assert((PC * 16) % 128 == 0, "tensor-copy destinations start on 128-byte boundaries");
     extern __shared__ __align__(128) unsigned char sm3[];
-    V *ring = reinterpret_cast<V *>(sm3);
-    T *coef = reinterpret_cast<T *>(sm3 + kRing3 * PC * 16);        // [ZC][NCO][NT]
-    T *ksum = coef + ZC * NCO * NT;                                  // [ZC][5][2][NT]
-    uint64_t *full = reinterpret_cast<uint64_t *>(ksum + ZC * 10 * NT);
-    uint64_t *empty = full + kRing3;
-    VX3<T> *svx = reinterpret_cast<VX3<T> *>(empty + kRing3);          // [kMaxAxisNv]
-    VYZ3<T> *svyz = reinterpret_cast<VYZ3<T> *>(svx + kMaxAxisNv);       // [kVyzStage]
+    V *const ring = reinterpret_cast<V *>(sm3);
+    T *const coef = reinterpret_cast<T *>(sm3 + RING * PC * 16);    // FP32 [ZC][NT][4], then [ZC][NCO - 4][NT]; FP64 [ZC][NCO][NT]
+    T *const ksum = coef + ZC * NCO * NT;                           // [ZC][NSUM][NT]
+    V *const vtab = reinterpret_cast<V *>(ksum + ZC * NSUM * NT);   // [nxg][4]: v_x, v_x^2, -nu_x, (1 - nu_x)/2
+    int *const xsg = reinterpret_cast<int *>(vtab + 4 * (kMaxAxisNv / W));   // [nxg][2] sign of v_x in each unit (0: mixed)
+    uint64_t *const full = reinterpret_cast<uint64_t *>(xsg + 2 * (kMaxAxisNv / W));
+    uint64_t *const empty = full + RING;
+    uint32_t *const cellw = reinterpret_cast<uint32_t *>(empty + RING) + threadIdx.x;  // flags of the thread's cells
     const Grid3D &g = a.g;
-    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * 32 + tx;
-    const bool producer = ty == R;
-    const int i0 = blockIdx.x * 32, j0 = blockIdx.y * R;
-    const int i = i0 + tx, j = j0 + ty;
+    const int tid = threadIdx.x, px = a.tx + 4;          // px: cells of a plane's row
+    const bool intile = tid < a.tx * a.ty;
+    const int ly = intile ? tid / a.tx : 0, lx = intile ? tid - ly * a.tx : 0;
+    const int i0 = blockIdx.x * a.tx, j0 = blockIdx.y * a.ty;
+    const int i = i0 + lx, j = j0 + ly;
     const int zc = blockIdx.z % a.nzc, split = blockIdx.z / a.nzc;
     const int z0 = zc * ZC;
     const long nc = (long)g.nx * g.ny * g.nz;
@@ -262,321 +279,466 @@ __global__ void __launch_bounds__(32 * (rows3<T>() + 1), 1)
     const int g0 = split * gps, g1 = min(g0 + gps, g.ngrp);
     const int ngr = max(g1 - g0, 0);
     const int total = ngr * NP;
-    const bool inij = !producer && i < g.nx && j < g.ny;
-    const int sz = (g.nx + 4) * (g.ny + 4);
+    const bool inij = intile && i < g.nx && j < g.ny;
+    // first group with v_z >= 0
+    int gpos = 0;
+    while (gpos < g.nvz && a.vyz[gpos * g.nvy].vz < T(0)) ++gpos;
+    gpos *= g.nxg * g.nvy;
+    // load of plane n of the split, counted over its groups: plane o of a
+    // group in upwind order (padded plane indices)
+    const auto load_plane = [&](int n) {
+        const int gi = n / NP, o = n - gi * NP, grp = g0 + gi, slot = RING == NP ? o : n % RING;
+        mbar_expect_tx(&full[slot], (uint32_t)(px * (a.ty + 4) * 16));
+        tma_load_4d(ring + slot * PC, &tmap, &full[slot], i0 * W, j0, grp >= gpos ? z0 + o : z0 + ZC + 3 - o, grp);
+    };
+    // velocities between restarts of the FP64 recurrence
+    const int rec = g.nvx <= 8 * kMxBlocks ? 8 : 16;
 
     if (tid == 0) {
-        for (int st = 0; st < kRing3; ++st) {
+        for (int st = 0; st < RING; ++st) {
             mbar_init(&full[st], 1);
             mbar_init(&empty[st], R);
         }
         mbar_fence_init();
+        for (int n = 0; n < RING && n < total; ++n) load_plane(n);
     }
-    // the velocity tables of the groups, staged once per block
-    const int nyz = g.nvy * g.nvz;
-    const bool stage_yz = nyz <= kVyzStage;
-    for (int q = tid; q < g.nvxp; q += blockDim.x * blockDim.y) svx[q] = a.vxt[q];
-    if (stage_yz)
-        for (int q = tid; q < nyz; q += blockDim.x * blockDim.y) svyz[q] = a.vyz[q];
-    const VX3<T> *vxtab = svx;
-    const VYZ3<T> *vyztab = stage_yz ? svyz : a.vyz;
+    // the v_x rows of the groups, staged once per block
+    for (int q = tid; q < g.nxg; q += NT) {
+        T *const t = reinterpret_cast<T *>(vtab + 4 * q);
+        int s[2];
+        for (int h = 0; h < 2; ++h) {
+            bool pos = true, neg = true;
+            for (int l = 0; l < LN; ++l) {
+                const int e = h * LN + l;
+                const VX3<T> cx = a.vxt[q * W + e];
+                t[e] = cx.vx;
+                t[W + e] = cx.vx * cx.vx;
+                t[2 * W + e] = -cx.nux;
+                t[3 * W + e] = T(0.5) * (T(1) - cx.nux);
+                pos = pos && cx.vx >= T(0);
+                neg = neg && cx.vx <= T(0);
+            }
+            s[h] = pos ? 1 : (neg ? -1 : 0);
+        }
+        xsg[2 * q] = s[0];
+        xsg[2 * q + 1] = s[1];
+    }
     // per-cell data of the column: flags, and for plain cells the
     // equilibrium in the form log2 M(v) = c0 + vx (c1 - c2 vx) - c2 dyz(v)
-    uint32_t plainm = 0, zerom = 0, mirm = 0, masks = 0;   // masks: byte t = limiter mask of cell t
-    static_assert(ZC <= 4, "one mask byte per column cell");
-    if (!producer) {
-#pragma unroll
-        for (int t = 0; t < ZC; ++t) {
-            const int k = z0 + t;
-            const bool in = inij && k < g.nz;
-            const long cell = ((long)k * g.ny + j) * g.nx + i;
-            const uint16_t fl = in ? a.flags[cell] : 0;
-            T *cz = coef + t * NCO * NT + tid;
-            if (fl & kPlain) {
-                plainm |= 1u << t;
-                T s[5];
-                gather_partials3(a.pin, a.Sin, nc, cell, s);
-                T rho, ux, uy, uz, tmp;
-                if (!primitives3<T>(pick<T>(g.dv_f, g.dv), s, rho, ux, uy, uz, tmp)) atomicExch(&a.err[kErrNonphys], 1);
-                cz[5 * NT] = pick<T>(g.dt_tau0_f, g.dt_tau0) * rho;
-                if (a.eqp) {
-                    // conservative equilibrium (Sec. 3.1): tau from the direct
-                    // density, the Maxwellian from the Newton parameters
-                    rho = a.eqp[cell]; ux = a.eqp[nc + cell]; uy = a.eqp[2 * nc + cell];
-                    uz = a.eqp[3 * nc + cell]; tmp = a.eqp[4 * nc + cell];
+    // bit t: cell t of the column is plain, bit 4 + t: to be zeroed, bits 8 +
+    // 6 t: its face mask (in shared memory: registers are short)
+    uint32_t word = 0, fullm = 0;
+    static_assert(ZC <= 4, "the flag word");
+    T *const cq = coef + (F64 ? 0 : 4 * ZC * NT);
+    constexpr int NCQ = F64 ? NCO : NCO - 4;
+#pragma unroll 1
+    for (int t = 0; t < ZC; ++t) {
+        const int k = z0 + t;
+        const bool in = inij && k < g.nz;
+        const long cell = ((long)k * g.ny + j) * g.nx + i;
+        const uint16_t fl = in ? a.flags[cell] : 0;
+        T *const cz = cq + t * NCQ * NT + tid;
+        if (fl & kPlain) {
+            word |= 1u << t;
+            T s[5];
+            gather_partials3(a.pin, a.Sin, nc, cell, s);
+            T rho, ux, uy, uz, tmp;
+            if (!primitives3<T>(pick<T>(g.dv_f, g.dv), s, rho, ux, uy, uz, tmp)) atomicExch(&a.err[kErrNonphys], 1);
+            const T r = pick<T>(g.dt_tau0_f, g.dt_tau0) * rho;
+            if (a.eqp) {
+                // conservative equilibrium (Sec. 3.1): tau from the direct
+                // density, the Maxwellian from the Newton parameters
+                rho = a.eqp[cell]; ux = a.eqp[nc + cell]; uy = a.eqp[2 * nc + cell];
+                uz = a.eqp[3 * nc + cell]; tmp = a.eqp[4 * nc + cell];
+            }
+            const T c2 = T(kLog2e) / (T(2) * tmp);
+            if constexpr (F64) {
+                const T dv = T(g.dvx), A = r * rho * norm3(tmp);
+                cz[kMxUy * NT] = uy;
+                cz[kMxUz * NT] = uz;
+                cz[kMxC2 * NT] = c2;
+                cz[kMxOmr * NT] = T(1) - r;
+                cz[kMxQ * NT] = exp2(T(-2) * c2 * dv * dv);
+                for (int b = 0; b * rec < g.nvxp; ++b) {
+                    const T dx = T(g.vxmin) + T(b * rec) * dv - ux;
+                    cz[(kMxM + b) * NT] = A * exp2(-c2 * dx * dx);
+                    cz[(kMxR + b) * NT] = exp2(-c2 * (T(2) * dx * dv + dv * dv));
                 }
-                const T c2 = T(kLog2e) / (T(2) * tmp);
-                cz[0] = log2(rho * norm3(tmp)) - c2 * ux * ux;
-                cz[NT] = T(2) * c2 * ux;
-                cz[2 * NT] = c2;
-                cz[3 * NT] = uy;
-                cz[4 * NT] = uz;
+            } else {
+                T *const cv = coef + (t * NT + tid) * 4;
+                cv[0] = log2(rho * norm3(tmp)) - c2 * ux * ux;
+                cv[1] = T(2) * c2 * ux;
+                cv[2] = c2;
+                cv[3] = r;
+                cz[0] = uy;
+                cz[NT] = uz;
                 if constexpr (SHAK) {
-                    // k q, -k u.q and 2 log2(A) / log2(e) - 5
                     const T kk = a.pr1 / (T(5) * rho * tmp * tmp);
-                    const T kqx = kk * a.qh[cell], kqy = kk * a.qh[nc + cell], kqz = kk * a.qh[2 * nc + cell];
-                    cz[6 * NT] = kqx;
-                    cz[7 * NT] = kqy;
-                    cz[8 * NT] = kqz;
-                    cz[9 * NT] = -(kqx * ux + kqy * uy + kqz * uz);
-                    cz[10 * NT] = T(2.0 / kLog2e) * log2(rho * norm3(tmp)) - T(5);
+                    cz[2 * NT] = kk * a.qh[cell];
+                    cz[3 * NT] = kk * a.qh[nc + cell];
+                    cz[4 * NT] = kk * a.qh[2 * nc + cell];
                 }
             }
-            if (fl & kZero) zerom |= 1u << t;
-            masks |= (uint32_t)((fl >> kMaskShift3) & 0x3F) << (8 * t);
-            if (in && near_side3(g, i, j, k)) mirm |= 1u << t;
-#pragma unroll
-            for (int m = 0; m < 10; ++m) ksum[(t * 10 + m) * NT + tid] = T(0);
         }
+        if (fl & kZero) word |= 16u << t;
+        const uint32_t mk = (fl >> kMaskShift3) & 0x3F;
+        word |= mk << (8 + 6 * t);
+        // every lane of the warp outside the grid, or plain with the
+        // limiter on all six faces
+        if (__all_sync(0xffffffffu, !in || ((fl & kPlain) && (!MUSCL || mk == 0x3F)))) fullm |= 1u << t;
+        for (int m = 0; m < NSUM; ++m) ksum[(t * NSUM + m) * NT + tid] = T(0);
     }
+    *cellw = word;
     __syncthreads();
 
-    if (producer) {
-        if (tx == 0) {
-            for (int s = 0; s < total; ++s) {
-                const int slot = s % kRing3;
-                if (s >= kRing3 && !mbar_wait(&empty[slot], (uint32_t)(((s / kRing3) - 1) & 1)))
-                    atomicExch(&a.err[kErrTimeout], 1);
-                mbar_expect_tx(&full[slot], PB);
-                const int gi = s / NP, o = s - gi * NP;
-                // plane z0 - 2 + o of the column, padded index z0 + o
-                tma_load_4d(ring + slot * PC, &tmap, &full[slot], i0 * W, j0, z0 + o, g0 + gi);
-            }
-            // every issued copy has landed before the block exits
-            for (int s = max(total - kRing3, 0); s < total; ++s)
-                mbar_wait(&full[s % kRing3], (uint32_t)((s / kRing3) & 1));
-        }
-        return;
-    }
-
-    const int c0 = (ty + 2) * kPlaneX + tx + 2;
+    const int c0 = (ly + 2) * px + lx + 2;
+    const int sz = (g.nx + 4) * (g.ny + 4);
     const int pc0 = inij ? nbr3(g, i, j, z0) : 0;
-    auto wait_full = [&](int s) -> const V * {
-        const int slot = s % kRing3;
-        if (!mbar_wait(&full[slot], (uint32_t)((s / kRing3) & 1))) atomicExch(&a.err[kErrTimeout], 1);
-        return ring + slot * PC;
+    // padding mirrors of the thread's cells along x and y: offset of the first
+    // one (0: none); on zero-gradient sides, where it is one cell, a second
+    // one twice as far
+    int mx = 0, my = 0;
+    const int row = g.nx + 4;
+    if (inij) {
+        if (g.bc[0] == DVM_BC_PERIODIC) mx = i < 2 ? g.nx : (i >= g.nx - 2 ? -g.nx : 0);
+        else if (i == 0 && g.bc[0] == DVM_BC_ZEROGRAD) mx = -1;
+        else if (i == g.nx - 1 && g.bc[1] == DVM_BC_ZEROGRAD) mx = 1;
+        if (g.bc[2] == DVM_BC_PERIODIC) my = j < 2 ? g.ny * row : (j >= g.ny - 2 ? -g.ny * row : 0);
+        else if (j == 0 && g.bc[2] == DVM_BC_ZEROGRAD) my = -row;
+        else if (j == g.ny - 1 && g.bc[3] == DVM_BC_ZEROGRAD) my = row;
+    }
+    const bool zside = z0 < 2 || z0 + ZC > g.nz - 2;
+    const bool xside = __any_sync(0xffffffffu, mx != 0), yside = __any_sync(0xffffffffu, my != 0);
+
+    // slot and phase of plane o of group gi: with a slot for every plane of a
+    // group, plane o is always in slot o
+    const uint32_t full0 = smem_u32(full), empty0 = smem_u32(empty), lane0 = (tid & 31) == 0;
+    const bool warp0 = tid < 32;
+    uint32_t bad = 0;               // a wait timed out
+    const auto slot_of = [](int gi, int o) { return RING == NP ? o : (gi * NP + o) % RING; };
+    const auto wait_full = [&](int gi, int o) {
+        const uint32_t phase = RING == NP ? gi & 1 : ((gi * NP + o) / RING) & 1;
+        mbar_wait_or(full0 + 8 * slot_of(gi, o), phase, bad);
     };
-    auto release = [&](int s) {
+    const auto release = [&](int gi, int o) {
         __syncwarp();
-        if (tx == 0) mbar_arrive(&empty[s % kRing3]);
+        mbar_arrive_if(empty0 + 8 * slot_of(gi, o), lane0);
+        if (warp0 && lane0) {
+            // the plane this warp released two planes ago, RING planes on
+            const int n = gi * NP + o - 2;
+            if (n >= 0 && n + RING < total) {
+                const int slot = RING == NP ? (o + NP - 2) % NP : n % RING;
+                mbar_wait_or(empty0 + 8 * slot, (uint32_t)((n / RING) & 1), bad);
+                load_plane(n + RING);
+            }
+        }
+    };
+    // store of a cell's vector and of its padding mirrors
+    const auto store = [&](V *d, int k, const T (&o)[W]) {
+        vst<T>(d, o);
+        if (xside) {
+            if (mx) vst<T>(d + mx, o);
+            if (mx == 1 || mx == -1) vst<T>(d + 2 * mx, o);
+        }
+        if (yside | zside) {
+            if (my) vst<T>(d + my, o);
+            if (my == row || my == -row) vst<T>(d + 2 * my, o);
+            if (zside) {
+                if (g.bc[4] == DVM_BC_PERIODIC) {
+                    if (k < 2) vst<T>(d + (long)g.nz * sz, o);
+                    else if (k >= g.nz - 2) vst<T>(d - (long)g.nz * sz, o);
+                } else {
+                    if (k == 0 && g.bc[4] == DVM_BC_ZEROGRAD) { vst<T>(d - sz, o); vst<T>(d - 2 * sz, o); }
+                    if (k == g.nz - 1 && g.bc[5] == DVM_BC_ZEROGRAD) { vst<T>(d + sz, o); vst<T>(d + 2 * sz, o); }
+                }
+            }
+        }
     };
 
-    T q[ZC][5];
+    T S0[ZC], S1[ZC], S2[ZC];       // row sums of F, v_x F, v_x^2 F
 #pragma unroll
-    for (int t = 0; t < ZC; ++t)
-#pragma unroll
-        for (int m = 0; m < 5; ++m) q[t][m] = T(0);
-    int fold = 0;
+    for (int t = 0; t < ZC; ++t) S0[t] = S1[t] = S2[t] = T(0);
+    T cg[ZC];                       // FP32: the row's constant of the exponent
+    T kyz[ZC], l5[ZC];              // Shakhov: the row's part of k c.q; 2 log2(A)/log2(e) - 5
+    T Mr[ZC], Rr[ZC], Er[ZC];       // FP64: recurrence, and the row's factor of v_y and v_z
+    VYZ3<T> cyz{};
+    uint32_t keepo = 0, fullo = 0;  // cells to store / without face weights, in upwind order
+    bool pz = true;
+    int yz = g0 / g.nxg, xg = g0 - yz * g.nxg;
+    bool fresh = true;              // a new row (or the split's first group)
     V *const fout = reinterpret_cast<V *>(a.fout);
     for (int gi = 0; gi < ngr; ++gi) {
-        const int grp = g0 + gi;
-        const int yz = grp / g.nxg, xg = grp - yz * g.nxg;
-        const VYZ3<T> cyz = vyztab[yz];
-        T vx[W], nux[W], kx[W];
-        bool xpos = true, xneg = true;
-#pragma unroll
-        for (int e = 0; e < W; ++e) {
-            const VX3<T> cx = vxtab[xg * W + e];
-            vx[e] = cx.vx;
-            nux[e] = cx.nux;
-            kx[e] = T(0.5) * (T(1) - cx.nux);
-            xpos = xpos && cx.vx >= T(0);
-            xneg = xneg && cx.vx <= T(0);
-        }
-        const bool xuni = xpos || xneg;
-        const int ox = xpos ? 1 : -1;
-        const bool py = cyz.vy >= T(0), pz = cyz.vz >= T(0);
-        const int oy = py ? kPlaneX : -kPlaneX;
-        const T ky = T(0.5) * (T(1) - cyz.nuy), kz = T(0.5) * (T(1) - cyz.nuz);
-        const T nzs = pz ? cyz.nuz : -cyz.nuz;
-        const T vyz2 = cyz.vy * cyz.vy + cyz.vz * cyz.vz;
-        V *dst = fout + (long)grp * g.slab;
-        const int base = gi * NP;
-        // rolling window along z: f at z - 1, z, z + 1 and the differences
-        // d(z - 1/2) = f(z) - f(z - 1), d(z + 1/2)
-        T fm1[W], f0[W], fp1[W], dm[W], dp[W], phim[W];
-        {
-            T fm2[W];
-            sld<T>(wait_full(base) + c0, fm2);
-            sld<T>(wait_full(base + 1) + c0, fm1);
-            sld<T>(wait_full(base + 2) + c0, f0);
-            sld<T>(wait_full(base + 3) + c0, fp1);
-            release(base);
-            release(base + 1);
-            // face value at z0 - 1/2
-            const T kw = (masks & 16u) ? kz : T(0);
-#pragma unroll
-            for (int e = 0; e < W; ++e) {
-                dm[e] = f0[e] - fm1[e];
-                dp[e] = fp1[e] - f0[e];
+        if (fresh) {
+            cyz = a.vyz[yz];
+            pz = cyz.vz >= T(0);
+            keepo = (*cellw | *cellw >> 4) & 15u;
+            fullo = fullm;
+            if (!pz) {
+                keepo = __brev(keepo) >> (32 - ZC);
+                fullo = __brev(fullo) >> (32 - ZC);
             }
-            if (!MUSCL) {
 #pragma unroll
-                for (int e = 0; e < W; ++e) phim[e] = pz ? fm1[e] : f0[e];
-            } else if (pz) {
-#pragma unroll
-                for (int e = 0; e < W; ++e) phim[e] = fma(kw, minmod3(dm[e], fm1[e] - fm2[e]), fm1[e]);
-            } else {
-#pragma unroll
-                for (int e = 0; e < W; ++e) phim[e] = fma(-kw, minmod3(dp[e], dm[e]), f0[e]);
-            }
-        }
-#pragma unroll
-        for (int t = 0; t < ZC; ++t) {
-            // the plane of z was waited for as the z + 2 centre two steps ago
-            const V *pl = ring + ((base + t + 2) % kRing3) * PC;
-            T fp2[W];
-            sld<T>(wait_full(base + t + 4) + c0, fp2);
-            const uint32_t mk = (masks >> (8 * t)) & 0x3Fu;
-            // face value at z + 1/2, the z - 1/2 face of the next cell
-            T phip[W], dpp[W];
-#pragma unroll
-            for (int e = 0; e < W; ++e) dpp[e] = fp2[e] - fp1[e];
-            if (!MUSCL) {
-#pragma unroll
-                for (int e = 0; e < W; ++e) phip[e] = pz ? f0[e] : fp1[e];
-            } else {
-                const T kw = (mk & 32u) ? kz : T(0);
-                if (pz) {
-#pragma unroll
-                    for (int e = 0; e < W; ++e) phip[e] = fma(kw, minmod3(dp[e], dm[e]), f0[e]);
+            for (int s = 0; s < ZC; ++s) {
+                const int t = pz ? s : ZC - 1 - s;      // cells in upwind order
+                const T *const cz = cq + t * NCQ * NT + tid;
+                if constexpr (F64) {
+                    const T dy = cyz.vy - cz[kMxUy * NT], dz = cyz.vz - cz[kMxUz * NT];
+                    Er[s] = exp2(-cz[kMxC2 * NT] * (dy * dy + dz * dz));
+                    const int b = xg * W / rec;
+                    Mr[s] = cz[(kMxM + b) * NT] * Er[s];
+                    Rr[s] = cz[(kMxR + b) * NT];
+                    for (int q = b * rec; q < xg * W; ++q) {   // a split that starts inside a row
+                        Mr[s] *= Rr[s];
+                        Rr[s] *= cz[kMxQ * NT];
+                    }
                 } else {
-#pragma unroll
-                    for (int e = 0; e < W; ++e) phip[e] = fma(-kw, minmod3(dpp[e], dp[e]), fp1[e]);
-                }
-            }
-            const bool pl_t = (plainm >> t) & 1u;
-            if (pl_t || ((zerom >> t) & 1u)) {
-                T out[W];
-                if (pl_t) {
-                    const T *cz = coef + t * NCO * NT + tid;
-                    const T c0c = cz[0], c1 = cz[NT], c2 = cz[2 * NT], uy = cz[3 * NT], uz = cz[4 * NT], r = cz[5 * NT];
-                    const T dyv = cyz.vy - uy, dzv = cyz.vz - uz;
-                    const T cg = c0c - c2 * (dyv * dyv + dzv * dzv);
-                    // Shakhov: k c.q = kqx vx + (kqy vy + kqz vz - k u.q)
-                    T kqx = 0, kyz = 0, l5 = 0;
+                    const float4 cv = *reinterpret_cast<const float4 *>(coef + (t * NT + tid) * 4);
+                    const T dy = cyz.vy - cz[0], dz = cyz.vz - cz[NT];
+                    cg[s] = cv.x - cv.z * (dy * dy + dz * dz);
                     if constexpr (SHAK) {
-                        kqx = cz[6 * NT];
-                        kyz = fma(cz[7 * NT], cyz.vy, fma(cz[8 * NT], cyz.vz, cz[9 * NT]));
-                        l5 = cz[10 * NT];
+                        const T ux = cv.y / (T(2) * cv.z);
+                        kyz[s] = fma(cz[3 * NT], dy, fma(cz[4 * NT], dz, -cz[2 * NT] * ux));
+                        l5[s] = T(2.0 / kLog2e) * fma(cv.y * T(0.5), ux, cv.x) - T(5);
                     }
-                    const T omr = T(1) - r;
-                    const T kyo = (mk & (py ? 8u : 4u)) ? ky : T(0), kyi = (mk & (py ? 4u : 8u)) ? ky : T(0);
-                    T yu1[W], yu2[W], yd1[W];
-                    sld<T>(pl + c0 - oy, yu1);
+                }
+            }
+            fresh = false;
+        } else if (F64 && xg * W % rec == 0) {
+#pragma unroll
+            for (int s = 0; s < ZC; ++s) {
+                const T *const cz = cq + (pz ? s : ZC - 1 - s) * NCQ * NT + tid;
+                Mr[s] = cz[(kMxM + xg * W / rec) * NT] * Er[s];
+                Rr[s] = cz[(kMxR + xg * W / rec) * NT];
+            }
+        }
+        // the rows of the x flux are read again for every cell (below)
+        P vx[2], vx2[2];
+        ld_units(vtab + 4 * xg, vx);
+        ld_units(vtab + 4 * xg + 1, vx2);
+        const int sx0 = xsg[2 * xg], sx1 = xsg[2 * xg + 1];
+        const bool mixed = sx0 == 0 || sx1 == 0;
+        const int oy = cyz.vy >= T(0) ? px : -px;
+        const T ky = T(0.5) * (T(1) - cyz.nuy), kz = T(0.5) * (T(1) - cyz.nuz);
+        V *const dst = fout + (long)(g0 + gi) * g.slab;
+        // along z, downwind: centre, difference to the upwind cell, limited
+        // slope of the upwind face
+        P f0[2], dm[2], mi[2];
+        {
+            P um2[2], um1[2], dd[2];
+            wait_full(gi, 0);
+            ld_units(ring + slot_of(gi, 0) * PC + c0, um2);
+            wait_full(gi, 1);
+            ld_units(ring + slot_of(gi, 1) * PC + c0, um1);
+            wait_full(gi, 2);
+            ld_units(ring + slot_of(gi, 2) * PC + c0, f0);
+            release(gi, 0);
+            release(gi, 1);
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                dm[h] = sub2(f0[h], um1[h]);
+                if (MUSCL) {
+                    dd[h] = sub2(um1[h], um2[h]);
+                    mi[h] = minmod2(dm[h], dd[h]);
+                }
+            }
+        }
+#pragma unroll
+        for (int s = 0; s < ZC; ++s) {
+            const V *const pl = ring + slot_of(gi, s + 2) * PC;
+            const int t = pz ? s : ZC - 1 - s;
+            P fd[2], dp[2], mo[2];
+            wait_full(gi, s + 3);
+            if (MUSCL || s + 1 < ZC) {
+                ld_units(ring + slot_of(gi, s + 3) * PC + c0, fd);
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    dp[h] = sub2(fd[h], f0[h]);
+                    if (MUSCL) mo[h] = minmod2(dp[h], dm[h]);
+                }
+            }
+            // the equilibrium, times r in FP64
+            T feq[W], r;
+            P nnux[2], kx[2];
+            ld_units(vtab + 4 * xg + 2, nnux);
+            ld_units(vtab + 4 * xg + 3, kx);
+            if constexpr (F64) {
+                const T *const cz = cq + t * NCQ * NT + tid;
+                const T Q = cz[kMxQ * NT];
+                r = cz[kMxOmr * NT];
+#pragma unroll
+                for (int e = 0; e < W; ++e) {
+                    feq[e] = xg * W + e < g.nvx ? Mr[s] : T(0);
+                    Mr[s] *= Rr[s];
+                    Rr[s] *= Q;
+                }
+            } else {
+                const float4 cv = *reinterpret_cast<const float4 *>(coef + (t * NT + tid) * 4);
+                r = cv.w;
+#pragma unroll
+                for (int e = 0; e < W; ++e) {
+                    const T v = unit_lane(vx[e / LN], e % LN);
+                    const T x = fma(fma(-cv.z, v, cv.y), v, cg[s]);
+                    feq[e] = exp2_state(x);
+                    if constexpr (SHAK) {
+                        // |c|^2/T - 5 = 2 (log2 A - log2 M) / log2 e - 5
+                        const T kc = fma(v, cq[(t * NCQ + 2) * NT + tid], kyz[s]);
+                        feq[e] = fma(feq[e] * kc, fma(T(-2.0 / kLog2e), x, l5[s]), feq[e]);
+                    }
+                }
+            }
+            T out[W];
+            // FULL: no face weights.  Else the weights are 1 where the face's
+            // stencil is all gas and 0 elsewhere, and cells that are not
+            // plain come out 0.
+            const uint32_t mk = *cellw >> (8 + 6 * t);
+            const auto update = [&](auto full_) {
+                constexpr bool FULL = decltype(full_)::value;
+                P yu1[2], yu2[2], yd1[2], xu1[2], xu2[2], xd1[2];
+                ld_units(pl + c0 - oy, yu1);
+                if (MUSCL) {
+                    ld_units(pl + c0 - 2 * oy, yu2);
+                    ld_units(pl + c0 + oy, yd1);
+                }
+                if (sx0 == sx1) {
+                    ld_units(pl + c0 - sx0, xu1);
                     if (MUSCL) {
-                        sld<T>(pl + c0 - 2 * oy, yu2);
-                        sld<T>(pl + c0 + oy, yd1);
+                        ld_units(pl + c0 - 2 * sx0, xu2);
+                        ld_units(pl + c0 + sx0, xd1);
                     }
-                    T dfx[W];
-                    if (xuni) {
-                        const T xo = (mk & (xpos ? 2u : 1u)) ? T(1) : T(0), xi = (mk & (xpos ? 1u : 2u)) ? T(1) : T(0);
-                        T xu1[W], xu2[W], xd1[W];
-                        sld<T>(pl + c0 - ox, xu1);
-                        if (MUSCL) {
-                            sld<T>(pl + c0 - 2 * ox, xu2);
-                            sld<T>(pl + c0 + ox, xd1);
-                        }
-#pragma unroll
-                        for (int e = 0; e < W; ++e)
-                            dfx[e] = dflux<T, MUSCL>(f0[e], xu1[e], MUSCL ? xu2[e] : T(0), MUSCL ? xd1[e] : T(0),
-                                                     xo * kx[e], xi * kx[e]);
-                    } else {
-                        T xm1[W], xp1[W], xm2[W], xp2[W];
-                        sld<T>(pl + c0 - 1, xm1);
-                        sld<T>(pl + c0 + 1, xp1);
-                        if (MUSCL) {
-                            sld<T>(pl + c0 - 2, xm2);
-                            sld<T>(pl + c0 + 2, xp2);
-                        }
-                        const T kxm = (mk & 1u) ? T(1) : T(0), kxp = (mk & 2u) ? T(1) : T(0);
-#pragma unroll
-                        for (int e = 0; e < W; ++e) {
-                            const bool px = vx[e] >= T(0);
-                            dfx[e] = dflux<T, MUSCL>(f0[e], px ? xm1[e] : xp1[e], MUSCL ? (px ? xm2[e] : xp2[e]) : T(0),
-                                                     px ? xp1[e] : xm1[e], kx[e] * (px ? kxp : kxm),
-                                                     kx[e] * (px ? kxm : kxp));
-                        }
-                    }
-                    T s = 0, sx = 0, sxx = 0;
-#pragma unroll
-                    for (int e = 0; e < W; ++e) {
-                        const T dfy = dflux<T, MUSCL>(f0[e], yu1[e], MUSCL ? yu2[e] : T(0), MUSCL ? yd1[e] : T(0), kyo, kyi);
-                        const T xe = fma(fma(-c2, vx[e], c1), vx[e], cg);
-                        T feq = exp2_state(xe);
-                        if constexpr (SHAK) {
-                            // |c|^2/T - 5 = 2 (log2 A - log2 M) / log2 e - 5
-                            const T mk5 = feq * fma(kqx, vx[e], kyz);
-                            feq = fma(mk5, fma(T(-2.0 / kLog2e), xe, l5), feq);
-                        }
-                        T o = fma(r, feq, omr * f0[e]);
-                        o = fma(-nux[e], dfx[e], o);
-                        o = fma(-cyz.nuy, dfy, o);
-                        o = fma(-nzs, phip[e] - phim[e], o);     // nzs carries the sign of v_z
-                        out[e] = o;
-                        s += o;
-                        sx = fma(vx[e], o, sx);
-                        sxx = fma(vx[e] * vx[e], o, sxx);
-                    }
-                    q[t][0] += s;
-                    q[t][1] += sx;
-                    q[t][2] = fma(cyz.vy, s, q[t][2]);
-                    q[t][3] = fma(cyz.vz, s, q[t][3]);
-                    q[t][4] += T(0.5) * fma(vyz2, s, sxx);
                 } else {
 #pragma unroll
-                    for (int e = 0; e < W; ++e) out[e] = T(0);
+                    for (int h = 0; h < 2; ++h) {
+                        const int sx = h ? sx1 : sx0;
+                        xu1[h] = ld_unit(pl + c0 - sx, h);
+                        if (MUSCL) {
+                            xu2[h] = ld_unit(pl + c0 - 2 * sx, h);
+                            xd1[h] = ld_unit(pl + c0 + sx, h);
+                        }
+                    }
                 }
-                const int pc = pc0 + t * sz;
-                vst<T>(dst + pc, out);
-                if ((mirm >> t) & 1u) {
-                    int mir[6];
-                    mirrors3(g, i, j, z0 + t, mir);
 #pragma unroll
-                    for (int u = 0; u < 6; ++u)
-                        if (mir[u] >= 0) vst<T>(dst + mir[u], out);
+                for (int h = 0; h < 2; ++h) {
+                    // the differences on units, the rest lane by lane: the
+                    // limiter has no packed form, and pairs formed from its
+                    // results cost more moves than the packed arithmetic saves
+                    const P ax2 = sub2(f0[h], xu1[h]), ay2 = sub2(f0[h], yu1[h]);
+                    P bx2, by2, cx2, cy2;
+                    if (MUSCL) {
+                        bx2 = sub2(xd1[h], f0[h]); cx2 = sub2(xu1[h], xu2[h]);
+                        by2 = sub2(yd1[h], f0[h]); cy2 = sub2(yu1[h], yu2[h]);
+                    }
+                    const bool xp = (h ? sx1 : sx0) > 0, yp = oy > 0;
+#pragma unroll
+                    for (int l = 0; l < LN; ++l) {
+                        const int e = h * LN + l;
+                        T dx = unit_lane(ax2, l), dy = unit_lane(ay2, l), dz = unit_lane(dm[h], l);
+                        if (MUSCL) {
+                            const T bx = unit_lane(bx2, l), cx = unit_lane(cx2, l), by = unit_lane(by2, l), cy = unit_lane(cy2, l);
+                            const T kxe = unit_lane(kx[h], l);
+                            if constexpr (FULL) {
+                                dx = fma(kxe, minmod_diff(bx, dx, cx), dx);
+                                dy = fma(ky, minmod_diff(by, dy, cy), dy);
+                                dz = fma(kz, unit_lane(mo[h], l) - unit_lane(mi[h], l), dz);
+                            } else {
+                                const auto w = [&](uint32_t bit, T x) { return (mk & bit) ? x : T(0); };
+                                dx = fma(kxe, minmod_diff(bx, dx, cx, w(xp ? 2u : 1u, T(1)), w(xp ? 1u : 2u, T(-1))), dx);
+                                dy = fma(ky, minmod_diff(by, dy, cy, w(yp ? 8u : 4u, T(1)), w(yp ? 4u : 8u, T(-1))), dy);
+                                dz = fma(w(pz ? 32u : 16u, kz), unit_lane(mo[h], l), dz);
+                                dz = fma(w(pz ? 16u : 32u, -kz), unit_lane(mi[h], l), dz);
+                            }
+                        }
+                        const T fc = unit_lane(f0[h], l), q = feq[e];
+                        T o = F64 ? fma(r, fc, q) : fma(r, q - fc, fc);
+                        o = fma(unit_lane(nnux[h], l), dx, o);
+                        o = fma(-cyz.nuy, dy, o);
+                        o = fma(-cyz.nuz, dz, o);
+                        if constexpr (!FULL) o = ((*cellw >> t) & 1u) ? o : T(0);
+                        out[e] = o;
+                    }
+                }
+            };
+            if (F64 || !mixed) {
+                if (fullo & (1u << s)) update(std::true_type{});
+                else update(std::false_type{});
+            } else {
+                // a unit whose lanes have v_x of both signs
+                const bool py = oy > 0;
+                const T yo = (mk & (py ? 8u : 4u)) ? ky : T(0), yi = (mk & (py ? 4u : 8u)) ? ky : T(0);
+                const T zo = (mk & (pz ? 32u : 16u)) ? kz : T(0), zi = (mk & (pz ? 16u : 32u)) ? kz : T(0);
+                const T *const f = reinterpret_cast<const T *>(pl + c0);
+#pragma unroll
+                for (int e = 0; e < W; ++e) {
+                    const int h = e / LN, l = e % LN;
+                    const int sx = unit_lane(vx[h], l) >= T(0) ? W : -W, sy = oy * W;
+                    const T fc = unit_lane(f0[h], l);
+                    T dx = fc - f[e - sx], dy = fc - f[e - sy], dz = unit_lane(dm[h], l);
+                    if (MUSCL) {
+                        const T xo = (mk & (sx > 0 ? 2u : 1u)) ? T(1) : T(0), xi = (mk & (sx > 0 ? 1u : 2u)) ? T(1) : T(0);
+                        const T tx_ = xo * minmod3(f[e + sx] - fc, dx) - xi * minmod3(dx, f[e - sx] - f[e - 2 * sx]);
+                        dx = fma(unit_lane(kx[h], l), tx_, dx);
+                        dy = fma(-yi, minmod3(dy, f[e - sy] - f[e - 2 * sy]), fma(yo, minmod3(f[e + sy] - fc, dy), dy));
+                        dz = fma(-zi, unit_lane(mi[h], l), fma(zo, unit_lane(mo[h], l), dz));
+                    }
+                    const T q = feq[e];
+                    T o = F64 ? fma(r, fc, q) : fma(r, q - fc, fc);
+                    o = fma(unit_lane(nnux[h], l), dx, o);
+                    o = fma(-cyz.nuy, dy, o);
+                    o = fma(-cyz.nuz, dz, o);
+                    out[e] = ((*cellw >> t) & 1u) ? o : T(0);
                 }
             }
+            if (keepo & (1u << s)) store(dst + (pc0 + t * sz), z0 + t, out);
 #pragma unroll
             for (int e = 0; e < W; ++e) {
-                phim[e] = phip[e];
-                dm[e] = dp[e];
-                dp[e] = dpp[e];
-                fm1[e] = f0[e];
-                f0[e] = fp1[e];
-                fp1[e] = fp2[e];
+                S0[s] += out[e];
+                S1[s] = fma(unit_lane(vx[e / LN], e % LN), out[e], S1[s]);
+                S2[s] = fma(unit_lane(vx2[e / LN], e % LN), out[e], S2[s]);
             }
-            release(base + t + 2);
-        }
-        release(base + ZC + 2);
-        release(base + ZC + 3);
-        // fold the plain sums of 8 groups into the compensated sums
-        if (++fold == 8 || gi + 1 == ngr) {
-            fold = 0;
 #pragma unroll
-            for (int t = 0; t < ZC; ++t)
-#pragma unroll
-                for (int m = 0; m < 5; ++m) {
-                    T *ks = ksum + (t * 10 + 2 * m) * NT + tid;
-                    Acc<T> acc;
-                    acc.s = ks[0];
-                    acc.c = ks[NT];
-                    acc.add(q[t][m]);
-                    ks[0] = acc.s;
-                    ks[NT] = acc.c;
-                    q[t][m] = T(0);
+            for (int h = 0; h < 2; ++h) {
+                if (s + 1 < ZC) {
+                    f0[h] = fd[h];
+                    dm[h] = dp[h];
+                    if (MUSCL) mi[h] = mo[h];
                 }
+            }
+            release(gi, s + 2);
+        }
+        release(gi, ZC + 2);
+        // the row's moments into the compensated sums
+        if (++xg == g.nxg || gi + 1 == ngr) {
+            const T vyz2 = cyz.vy * cyz.vy + cyz.vz * cyz.vz;
+#pragma unroll
+            for (int s = 0; s < ZC; ++s) {
+                T *const ks = ksum + (pz ? s : ZC - 1 - s) * NSUM * NT + tid;
+                const T s0 = S0[s], s1 = S1[s], s2 = S2[s];
+                const T m[5] = {s0, s1, cyz.vy * s0, cyz.vz * s0, T(0.5) * fma(vyz2, s0, s2)};
+#pragma unroll
+                for (int q = 0; q < 5; ++q) {
+                    Acc<T> acc;
+                    acc.s = ks[q * NT];
+                    if constexpr (!F64) acc.c = ks[(5 + q) * NT];
+                    acc.add(m[q]);
+                    ks[q * NT] = acc.s;
+                    if constexpr (!F64) ks[(5 + q) * NT] = acc.c;
+                }
+                S0[s] = S1[s] = S2[s] = T(0);
+            }
+            if (xg == g.nxg) {
+                xg = 0;
+                ++yz;
+                fresh = true;
+            }
         }
     }
-#pragma unroll
+    if (bad) atomicExch(&a.err[kErrTimeout], 1);
+#pragma unroll 1
     for (int t = 0; t < ZC; ++t) {
-        if (!(((plainm | zerom) >> t) & 1u)) continue;
+        if (!((*cellw >> t | *cellw >> (4 + t)) & 1u)) continue;
         const long cell = ((long)(z0 + t) * g.ny + j) * g.nx + i;
-#pragma unroll
-        for (int m = 0; m < 5; ++m) {
-            const T *ks = ksum + (t * 10 + 2 * m) * NT + tid;
-            a.pout[((long)split * 5 + m) * nc + cell] = ks[0] - ks[NT];
-        }
+        const T *const ks = ksum + t * NSUM * NT + tid;
+        for (int m = 0; m < 5; ++m)
+            a.pout[((long)split * 5 + m) * nc + cell] = F64 ? ks[m * NT] : ks[m * NT] - ks[(F64 ? 0 : 5 + m) * NT];
     }
 }
 
@@ -1445,8 +1607,9 @@ cudaError_t launch_bulk3(dvm_ctx *c, const Bulk3Args<T> &a)
         if (e != cudaSuccess) return e;
         attr = true;
     }
-    dim3 grid(nb3(c->nx, 32), nb3(c->ny, rows3<T>()), (unsigned)(a.nzc * a.S)), block(32, rows3<T>() + 1);
-    k_bulk3<T, MUSCL, SHAK><<<grid, block, smem, c->stream>>>(a, c->tmap[c->cur]);
+    constexpr int threads = 32 * warps3<T>();
+    const dim3 grid(nb3(c->nx, a.tx), nb3(c->ny, a.ty), (unsigned)(a.nzc * a.S));
+    k_bulk3<T, MUSCL, SHAK><<<grid, threads, smem, c->stream>>>(a, c->tmap[c->cur]);
     return cudaGetLastError();
 }
 
@@ -1603,6 +1766,7 @@ cudaError_t step3d_t(dvm_ctx *c, int phase, double *xbuf)
     }
     Bulk3Args<T> a{};
     a.g = g; a.S = c->S; a.Sin = Sin; a.nzc = (c->nz + kZc3 - 1) / kZc3;
+    tile3d(c, &a.tx, &a.ty);
     a.eqp = cons && !imex ? (const T *)c->eqp : nullptr;
     a.qh = shak ? (const T *)c->qheat : nullptr;
     a.pr1 = T(1.0 - c->Pr);
@@ -1649,6 +1813,41 @@ cudaError_t split_relax3d_t(dvm_ctx *c, const double *xbuf)
 
 }  // namespace
 
+// Tile of the bulk kernel: the cells tx x ty of a plane that a block's threads
+// take, row by row of the tile.  Of all widths, the one whose tiles cover the
+// grid with the least work: a tile takes the time of its warps (in fours,
+// one per SM sub-partition) and of about six more (latencies that few warps do
+// not cover), weighted with a fifth of the halo it re-reads and a little for
+// short rows; what fits a ring
+// slot.  64^2 cells: 32 x 16.  FP32, 45 x 50 cells: 45 x 11, 1.53 ms a launch
+// (37 planes, 14 x 15 x 13 velocities, Shakhov) against 1.82 with 16 x 32 and
+// 2.66 with 5 x 50 (as few lanes outside the grid, but 8 warps an SM).  FP64,
+// 40^2: 40 x 6, 7.7 ms (40 planes, 12^3) against 9.4 with 16 x 16 and 12.1
+// with 32 x 8.
+void tile3d(const dvm_ctx *c, int *tx, int *ty)
+{
+    const int threads = 32 * (c->prec == DVM_FP32 ? warps3<float>() : warps3<double>());
+    const int slot = c->prec == DVM_FP32 ? plane_stride3<float>() : plane_stride3<double>();
+    double least = -1;
+    for (int x = c->nx < 60 ? c->nx : 60; x >= 4; --x) {
+        int y = threads / x;
+        if (y > c->ny) y = c->ny;
+        while (y > 1 && (x + 4) * (y + 4) > slot) --y;
+        if ((x + 4) * (y + 4) > slot || y > 252) continue;
+        const double work = (double)nb3(c->nx, x) * nb3(c->ny, y) * (nb3((long)x * y, 128) * 4 + 6);
+        const double halo = (double)((x + 4) * (y + 4)) / (x * y);
+        const double cost = work * (1.0 + 0.2 * (halo - 1.0) + 0.2 / x);
+        if (least < 0 || cost < least) { least = cost; *tx = x; *ty = y; }
+    }
+}
+
+int bulk3_blocks(const dvm_ctx *c)
+{
+    int tx = 32, ty = 8;
+    tile3d(c, &tx, &ty);
+    return (int)(nb3(c->nx, tx) * nb3(c->ny, ty) * nb3(c->nz, kZc3));
+}
+
 // TMA descriptors of the two state buffers: a 4D view (x: padded cells of a
 // row times the W velocities of a group, y: padded rows, z: padded planes,
 // w: velocity group) with the bulk kernel's plane box (tile plus halo).
@@ -1670,8 +1869,9 @@ int make_tensor_maps3d(dvm_ctx *c)
                                 (cuuint64_t)c->ngrp};
     const cuuint64_t row = (cuuint64_t)(c->nx + 4) * W * c->elem;
     const cuuint64_t strides[3] = {row, row * (c->ny + 4), (cuuint64_t)c->slab * W * c->elem};
-    const cuuint32_t box[4] = {(cuuint32_t)kPlaneX * W,
-                               (cuuint32_t)(c->prec == DVM_FP32 ? rows3<float>() : rows3<double>()) + 4, 1, 1};
+    int tx = 32, ty = 8;
+    tile3d(c, &tx, &ty);
+    const cuuint32_t box[4] = {(cuuint32_t)((tx + 4) * W), (cuuint32_t)(ty + 4), 1, 1};
     const cuuint32_t estr[4] = {1, 1, 1, 1};
     const CUtensorMapDataType dt = c->prec == DVM_FP32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_FLOAT64;
     for (int b = 0; b < 2; ++b) {
