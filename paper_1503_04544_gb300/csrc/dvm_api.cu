@@ -338,13 +338,19 @@ int dvm_create(const dvm_grid *grid, const dvm_vgrid *vg, const dvm_physics *ph,
         // velocity splits: the count that minimises the load of the busiest
         // SM, ceil(blocks / 152) blocks of (groups per split + 5) group
         // times each (5: the per-block prologue and pipeline fill, fitted
-        // to measured bulk times); ties go to the smaller count
+        // to measured bulk times); ties go to the smaller count.  FP64, whose
+        // three resident blocks share the FP64 pipe and whose per-cell values
+        // are formed once for all splits (256^2 x 32^2: S = 3: 5.26 ms, 4:
+        // 5.37, 5: 4.65, 7: 4.58, 9: 4.79): rounds of three blocks, and two
+        // groups of prologue
         const long blocks = (long)((c->nx + 31) / 32) * ((c->ny + kRows - 1) / kRows);
+        const bool f32 = precision == DVM_FP32;
         int S = 1;
         long best = -1;
-        for (int s = 1; s <= 16 && s <= c->ngrp; ++s) {
-            const long per_sm = (blocks * s + 151) / 152;
-            const long cost = per_sm * ((c->ngrp + s - 1) / s + 5);
+        for (int s = 1; s <= (f32 ? 16 : 40) && s <= c->ngrp; ++s) {
+            long per_sm = (blocks * s + 151) / 152;
+            if (!f32 && per_sm > 3) per_sm = (per_sm + 2) / 3 * 3;
+            const long cost = per_sm * ((c->ngrp + s - 1) / s + (f32 ? 5 : 2));
             if (best < 0 || cost < best) { best = cost; S = s; }
         }
         c->S = S;
@@ -420,6 +426,7 @@ int dvm_create(const dvm_grid *grid, const dvm_vgrid *vg, const dvm_physics *ph,
         AL(G.rwz, sizeof(double) * nc); AL(G.vol, sizeof(double) * nc);
         AL(c->flags3, sizeof(uint16_t) * nc);
     }
+    if (c->prec == DVM_FP64) AL(c->cf64, dim == 2 ? cf64_bytes2d(c) : cf64_bytes3d(c));
     AL(c->master, sizeof(int32_t) * nc);
     AL(c->hs, nc);
     AL(c->counts, sizeof(int32_t) * 4);
@@ -476,12 +483,12 @@ void dvm_destroy(dvm_ctx *c)
     cudaFree(c->spec_list); cudaFree(c->wall_list); cudaFree(c->counts);
     cudaFree(c->wphi); cudaFree(c->wcontrib); cudaFree(c->cvinfo);
     cudaFree(c->d_body); cudaFree(c->d_hist); cudaFree(c->d_err);
-    cudaFree(c->d_scratch); cudaFree(c->d_out); cudaFree(c->eqp); cudaFree(c->split_in); cudaFree(c->qheat);
+    cudaFree(c->d_scratch); cudaFree(c->d_out); cudaFree(c->cf64); cudaFree(c->eqp); cudaFree(c->split_in); cudaFree(c->qheat);
     cudaFree(c->hpart[0]); cudaFree(c->hpart[1]);
     cudaFree(c->d_Twseg); cudaFree(c->d_segdir);
     for (int s = 0; s < 6; ++s) cudaFree(c->d_bcstate[s]);
     cudaFree(c->d_prim0);
-    cudaFree(c->snap_f); cudaFree(c->snap_part); cudaFree(c->snap_scratch); cudaFree(c->snap_body);
+    cudaFree(c->snap_f); cudaFree(c->snap_part); cudaFree(c->snap_body);
     free_adjoint2d(c);
     if (c->h_err) cudaFreeHost(c->h_err);
     if (c->gretired) {
@@ -1076,7 +1083,6 @@ static int ensure_snapshot(dvm_ctx *c)
     cudaError_t e = cudaSuccess;
     if (!c->snap_f) e = cudaMalloc(&c->snap_f, c->dev_elems * c->elem);
     if (e == cudaSuccess && !c->snap_part) e = cudaMalloc(&c->snap_part, part_bytes(c));
-    if (e == cudaSuccess && !c->snap_scratch) e = cudaMalloc(&c->snap_scratch, part_bytes(c));
     if (e == cudaSuccess && !c->snap_body) e = cudaMalloc(&c->snap_body, sizeof(dvm::BodyDev));
     if (e != cudaSuccess) {
         cudaGetLastError();
@@ -1114,16 +1120,11 @@ static cudaError_t restore_snapshot(dvm_ctx *c, const StepMark &m)
     return e;
 }
 
-// Moments of the current state into the scratch sums: raises the
-// non-physical flag for a gas cell with rho <= 0 or T <= 0.
-static cudaError_t check_state(dvm_ctx *c)
-{
-    void *keep = c->part[c->cur];
-    c->part[c->cur] = c->snap_scratch;
-    const cudaError_t e = st_partials(c);
-    c->part[c->cur] = keep;
-    return e;
-}
+// Raises the non-physical flag for a gas cell of the current state with rho <=
+// 0 or T <= 0, from the moment sums the step wrote with the state: 4 or 5
+// values per cell and split, where a pass over the state read all of it (FP64
+// 40^3 x 12^3: 2.7 ms a call; FP32 512^2 x 40^2: 0.5 ms).
+static cudaError_t check_state(dvm_ctx *c) { return c->dim == 2 ? check_moments2d(c) : check_moments3d(c); }
 
 // Synchronises and tells whether a flag is raised (without clearing it).
 static cudaError_t flags_raised(dvm_ctx *c, bool *raised)

@@ -496,6 +496,43 @@ __device__ __forceinline__ void mirrors(const Grid2D &g, int i, int j, I (&m)[4]
     }
 }
 
+// ---- per-cell values of the FP64 bulk kernels, formed once a step (k_cell64,
+// k_cell64_3) for all velocity splits: an FP64 operation holds the pipe for 64
+// clocks a warp, and some 400 of them per cell (the sums of the splits, the
+// primitives, the exponentials) in every split's prologue were worth six
+// groups of velocities (31 of a 50 us launch at 32^2 x 16^2).  Eight threads
+// of a warp share a cell: each sums every eighth split, all form the
+// primitives, and the exponentials are dealt out.
+constexpr int kMxBlocks = 4;         // restarts of the Maxwellian's recurrence along a v_x row
+constexpr int kCellThreads = 8;
+
+// Velocities between restarts.
+__device__ __forceinline__ int restart64(int nvx) { return nvx <= 8 * kMxBlocks ? 8 : 16; }
+
+// Sum over the eight threads of a cell (every thread returns it).
+__device__ __forceinline__ double cell_sum(double x)
+{
+#pragma unroll
+    for (int o = kCellThreads / 2; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    return x;
+}
+
+// The recurrence's values of a cell into slots [slot][nc]: Q = 2^(-2 c2 dv^2)
+// in slot q, and for every restart velocity v_b the factor A 2^(-c2 (v_b -
+// ux)^2) in slot m + b and R = 2^(-c2 (2 (v_b - ux) dv + dv^2)) in slot r + b.
+__device__ __forceinline__ void put_recurrence(double *cf, long nc, int k, int nvx, double vmin, double dv, double ux,
+                                               double c2, double A, int q, int m, int r)
+{
+    const int rec = restart64(nvx), nb = (nvx + rec - 1) / rec;
+    for (int v = k; v <= 2 * nb; v += kCellThreads) {
+        const int b = v >> 1;
+        const double dx = vmin + b * rec * dv - ux;
+        const double x = v == 2 * nb ? 2.0 * dv * dv : (v & 1 ? fma(2.0 * dx, dv, dv * dv) : dx * dx);
+        const double e = exp2(-c2 * x);
+        cf[(long)(v == 2 * nb ? q : (v & 1 ? r : m) + b) * nc] = v < 2 * nb && !(v & 1) ? A * e : e;
+    }
+}
+
 // Per-velocity coefficients: vx, vy, nu_x = |vx| dt/dx, nu_y = |vy| dt/dy.
 // Padded velocities carry a huge speed (their Maxwellian is 0) and zero
 // Courant numbers.

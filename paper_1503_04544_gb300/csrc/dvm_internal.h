@@ -198,9 +198,9 @@ struct dvm_ctx {
                                   // about a reference velocity [2][nc] per cell, written by the step that made it
     bool hvalid;                  // hpart[cur] belongs to f[cur] (else the step starts with k_heatflux)
     bool dt_given;                // dt came from dvm_physics, not from the CFL rule
+    double *cf64;                 // FP64: per-cell values of the bulk kernel, [slot][nc] (k_cell64, k_cell64_3)
     void *eqp;                    // [dim + 2][nc] conservative equilibrium parameters (state precision)
     void *snap_f, *snap_part;     // dvm_step: state and moment sums at the last checked step
-    void *snap_scratch;           // dvm_step: moment sums of the state check
     void *snap_body;              // dvm_step: rigid-body record at the last checked step
     bool rollback_off;            // dvm_rollback(ctx, 0): dvm_step without snapshots
     void *gretired;               // std::vector<cudaGraphExec_t> launched, destroyed once the stream is idle
@@ -232,6 +232,7 @@ cudaError_t split_step2d(dvm_ctx *c, int phase, void *xbuf);    // velocity spli
 cudaError_t split_step3d(dvm_ctx *c, int phase, void *xbuf);    // the same in 3D (dvm_step3d.cu)
 cudaError_t fusion2d(dvm_ctx *c, void *f, void *part);          // Eq. FusionDD on a buffer
 cudaError_t mass2d(dvm_ctx *c, double *d_scratch, double *d_out);
+cudaError_t check_moments2d(dvm_ctx *c);           // flags a state whose moment sums are not physical
 cudaError_t moments_out2d(dvm_ctx *c, double *d_out);
 cudaError_t ghost2d(dvm_ctx *c, int side, const double *d_prim, int nside);
 // public and device layout (dvm_layout.cu)
@@ -265,6 +266,7 @@ cudaError_t partials_from_state3d(dvm_ctx *c);
 cudaError_t init_maxwellian3d(dvm_ctx *c, const double *d_prim);
 cudaError_t step3d(dvm_ctx *c);
 cudaError_t mass3d(dvm_ctx *c, double *d_scratch, double *d_out);
+cudaError_t check_moments3d(dvm_ctx *c);
 cudaError_t moments_out3d(dvm_ctx *c, double *d_out);
 cudaError_t ghost3d(dvm_ctx *c, int side, const double *d_prim, int nside);
 cudaError_t zero_solid3d(dvm_ctx *c);
@@ -274,6 +276,8 @@ int make_tensor_maps3d(dvm_ctx *c);                // TMA descriptors of f[0], f
 void tile3d(const dvm_ctx *c, int *tx, int *ty);   // tile of the 3D bulk kernel
 int bulk3_blocks(const dvm_ctx *c);                // its blocks for one velocity split
 size_t cvinfo3_bytes();
+size_t cf64_bytes2d(const dvm_ctx *c);
+size_t cf64_bytes3d(const dvm_ctx *c);
 
 // Limiter-branch words of the 2D MUSCL step (recorded for the adjoint): one
 // uint32 per (velocity group, padded cell) with the row pitch rounded up to

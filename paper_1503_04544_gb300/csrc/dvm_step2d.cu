@@ -48,7 +48,8 @@ template <typename T>
 __device__ __forceinline__ void gather_partials(const T *part, int S, long nc, long cell, T (&s)[4])
 {
     Acc<T> a[4];
-    for (int q = 0; q < S; ++q)
+#pragma unroll 4
+    for (int q = 0; q < S; ++q)       // several splits' loads in flight
 #pragma unroll
         for (int m = 0; m < 4; ++m) a[m].merge(part[((long)q * 4 + m) * nc + cell], T(0));
 #pragma unroll
@@ -69,6 +70,7 @@ template <typename T> struct BulkArgs {
     const ulonglong2 *pt;     // [ngrp][7] packed-pair coefficients (FP32 path)
     const int8_t *gsign;      // [ngrp][2]
     const T *eqp;             // [4][nc] conservative equilibrium parameters, or null (direct moments)
+    const double *cf;         // FP64: per-cell values [C64][nc] (k_cell64)
     const T *qh;              // [2][nc] heat flux of the control volume at t^n (Shakhov model), used when hin is null
     const T *hin;             // Shakhov: raw heat-flux moments of f^n [S][5][nc] and their reference velocity [2][nc]
     T *hout;                  // Shakhov: the same for f^n+1
@@ -398,10 +400,11 @@ template <typename T, bool MUSCL, bool REC, bool SHAK>
 __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<T> a, const __grid_constant__ CUtensorMap tmap)
 {
     constexpr int W = Vec<T>::W;
-    // raw heat-flux moments of the new state (FP32 only: an FP64 step is
-    // bound by the FP64 pipe, where one more read of f^n by k_heatflux costs
-    // less than these sums)
-    constexpr bool HRAW = SHAK && sizeof(T) == 4;
+    // FP32 only (FP64: k_bulk64).  The Shakhov variant leaves raw heat-flux
+    // moments of the new state; an FP64 step is bound by the FP64 pipe, where
+    // one more read of f^n by k_heatflux costs less than these sums.
+    static_assert(sizeof(T) == 4, "the FP32 bulk kernel");
+    constexpr bool HRAW = SHAK;
     using V = typename Vec<T>::type;
     extern __shared__ __align__(128) unsigned char smem[];
     V *ring = reinterpret_cast<V *>(smem);
@@ -500,13 +503,6 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<T> a, const __g
     const bool anymir = __any_sync(0xffffffffu, inside && (mir[0] >= 0 || mir[2] >= 0));
     __syncthreads();
 
-    // FP64: the Maxwellian along a row of the uniform v_x grid by the
-    // recurrence M(v + dv) = M(v) R(v), R(v + dv) = R(v) Qm with
-    // Qm = 2^(-2 c2 dv^2), restarted from a direct evaluation every 8
-    // velocities and at every row start (relative error below 30 ulp)
-    T Mrun = 0, Rrun = 0, Qm = 0;
-    const bool mrec = sizeof(T) == 8 && g.nvx % W == 0;
-    if (sizeof(T) == 8 && plain) Qm = dexp2(T(-2) * c2 * T(g.dvx) * T(g.dvx));
     // the exponent's per-cell terms as pairs (packed path)
     F2 EL0, E1X, E1Y, NC2;
     if constexpr (sizeof(T) == 4 && MUSCL) {
@@ -617,25 +613,10 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<T> a, const __g
                 const VCoef<T> vc = ld_coef(a.vt + q * W + e);
                 vx[e] = vc.vx; vy[e] = vc.vy; nux[e] = vc.nux; nuy[e] = vc.nuy;
             }
-            if (sizeof(T) == 8 && mrec) {
-                const int p0 = q * W;
-                if (it % (8 / W) == 0 || p0 % g.nvx == 0) {
-                    const T dx = vx[0] - ux, dy = vy[0] - uy;
-                    Mrun = A * dexp2(-(dx * dx + dy * dy) * c2);
-                    Rrun = dexp2(-c2 * (T(2) * dx * T(g.dvx) + T(g.dvx) * T(g.dvx)));
-                }
 #pragma unroll
-                for (int e = 0; e < W; ++e) {
-                    feq[e] = Mrun;
-                    Mrun *= Rrun;
-                    Rrun *= Qm;
-                }
-            } else {
-#pragma unroll
-                for (int e = 0; e < W; ++e) {
-                    const T dx = vx[e] - ux, dy = vy[e] - uy;
-                    feq[e] = A * dexp2(-(dx * dx + dy * dy) * c2);
-                }
+            for (int e = 0; e < W; ++e) {
+                const T dx = vx[e] - ux, dy = vy[e] - uy;
+                feq[e] = A * dexp2(-(dx * dx + dy * dy) * c2);
             }
             // Shakhov: the equilibria of f and g (the BGK g equilibrium T/2 M
             // is formed in place after the f update)
@@ -743,6 +724,396 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<T> a, const __g
                 a.hout[((long)a.S * 5 + 1) * nc + cell] = 0;
             }
         }
+    }
+}
+
+// ------------------------------------------------------------ FP64 bulk kernel
+// On this part an FP64 operation holds the pipe of an SM's quarter for 64
+// clocks a warp, so this kernel counts FP64 operations and little else: 33 a
+// velocity pair (f, g) and cell, against 64 of the form it replaced (one cell
+// per thread, every difference from both sides, weights on every face, a
+// limiter whose magnitudes the compiler formed on the FP64 pipe): 7.90 ->
+// 4.31 ms a launch at 256^2 x 32^2, limited fluxes (with k_cell64, 0.14 ms).
+//
+// Block = 32 x 8 cells, four warps of 32 cells in x and two rows.  A thread
+// takes its two cells in upwind order of v_y: they share the face between
+// them, so a pair of cells costs four y differences and three y limiter
+// values instead of six and four.  Warps whose cells all have the limiter on
+// every face use no face weights.  The Maxwellian times dt/tau along a v_x row
+// is the recurrence M(v + dv) = M R, R(v + dv) = R Q, restarted every 8
+// velocities (16 from 33 per axis on) from the cell's v_x factor in shared
+// memory times the row's v_y factor (one exp2 per row and cell); relative
+// error below 30 ulp (130).  A group whose v_y changes sign between its two
+// velocities (odd nvx) takes each velocity's neighbours on its own side.
+constexpr int kRows64 = 4;            // warps of a block
+constexpr int kZ64 = 2;               // rows of a thread
+constexpr int kStages64 = 3;
+static_assert(kRows64 * kZ64 == kRows, "the tile of the state's tensor maps");
+enum C64 { kUy = 0, kC2, kRel, kGf, kQm, kMb, kRb = kMb + kMxBlocks, kC64 = kRb + kMxBlocks,
+           kKqx = kC64, kKqy, kUx, kIT, kC64S };
+
+template <bool SHAK> constexpr size_t bulk64_smem()
+{
+    return (size_t)kStages64 * kStageBytes + (size_t)(SHAK ? kC64S : kC64) * kZ64 * 32 * kRows64 * sizeof(double) +
+           2 * kStages64 * sizeof(uint64_t);
+}
+
+// Branch the limited reconstruction of a face took, as branch_bits, on the
+// bit patterns (b: the second argument of the minmod value m).
+__device__ __forceinline__ uint32_t branch_code(double m, double b)
+{
+    const long long im = __double_as_longlong(m);
+    return (im << 1) == 0 ? 0u : (im == __double_as_longlong(b) ? 2u : 1u);
+}
+
+// The per-cell values of k_bulk64 for the plain cells (dvm_device.cuh): the
+// slots of C64.  Block = 16 cells x kCellThreads.
+template <bool SHAK> __global__ void __launch_bounds__(128) k_cell64(BulkArgs<double> a, double *cf)
+{
+    const Grid2D &g = a.g;
+    const long nc = (long)g.nx * g.ny;
+    const long cell = (long)blockIdx.x * (128 / kCellThreads) + threadIdx.x / kCellThreads;
+    const int k = threadIdx.x % kCellThreads;
+    const bool plain = cell < nc && (a.flags[cell] & kPlain);
+    double s[4] = {0, 0, 0, 0};
+    if (plain)
+#pragma unroll 4
+        for (int q = k; q < a.Sin; q += kCellThreads)
+#pragma unroll
+            for (int m = 0; m < 4; ++m) s[m] += a.pin[((long)q * 4 + m) * nc + cell];
+#pragma unroll
+    for (int m = 0; m < 4; ++m) s[m] = cell_sum(s[m]);
+    if (!plain) return;
+    double rho, ux, uy, tmp;
+    if (!primitives<double>(g.dv, s[0], s[1], s[2], s[3], rho, ux, uy, tmp) && k == 0) atomicExch(&a.err[kErrNonphys], 1);
+    const double r = g.dt_tau0 * rho;
+    if (a.eqp) {
+        // conservative equilibrium (Sec. 3.1): tau from the direct density,
+        // the Maxwellian from the Newton parameters
+        rho = a.eqp[cell]; ux = a.eqp[nc + cell]; uy = a.eqp[2 * nc + cell]; tmp = a.eqp[3 * nc + cell];
+    }
+    const double iT = 1.0 / tmp, c2 = (0.5 * kLog2e) * iT;
+    double *const o = cf + cell;
+    put_recurrence(o, nc, k, g.nvx, g.vxmin, g.dvx, ux, c2, r * rho * (0.5 / kPi) * iT, kQm, kMb, kRb);
+    if (k == kCellThreads - 1) {
+        o[kUy * nc] = uy;
+        o[kC2 * nc] = c2;
+        o[kRel * nc] = r;
+        o[kGf * nc] = 0.5 * tmp;
+        if constexpr (SHAK) {
+            const double kk = a.pr1 / (5.0 * rho * tmp * tmp);
+            o[kKqx * nc] = kk * a.qh[cell];
+            o[kKqy * nc] = kk * a.qh[nc + cell];
+            o[kUx * nc] = ux;
+            o[kIT * nc] = iT;
+        }
+    }
+}
+
+template <bool MUSCL, bool REC, bool SHAK>
+__global__ void __launch_bounds__(32 * kRows64, SHAK ? 2 : 3)
+    k_bulk64(BulkArgs<double> a, const __grid_constant__ CUtensorMap tmap)
+{
+    constexpr int ZC = kZ64, NT = 32 * kRows64, PL = kTileX * kTileY, NST = kStages64;
+    extern __shared__ __align__(128) unsigned char smem[];
+    double2 *const ring = reinterpret_cast<double2 *>(smem);
+    double *const coef = reinterpret_cast<double *>(smem + NST * kStageBytes) + threadIdx.x;   // [C64][ZC][NT]
+    uint64_t *const full = reinterpret_cast<uint64_t *>(smem + NST * kStageBytes) + (SHAK ? kC64S : kC64) * ZC * NT;
+    uint64_t *const empty = full + NST;
+    const Grid2D &g = a.g;
+    const int tid = threadIdx.x, tx = tid & 31, ty = tid >> 5;
+    const int i0 = blockIdx.x * 32, j0 = blockIdx.y * kRows;
+    const int i = i0 + tx, jt = j0 + ty * ZC;
+    const long nc = (long)g.nx * g.ny;
+    const int split = blockIdx.z;
+    const int gps = (g.ngrp + a.S - 1) / a.S;
+    const int g0 = split * gps, g1 = min(g0 + gps, g.ngrp);
+    const int ngr = max(g1 - g0, 0);
+    const int rec = restart64(g.nvx);
+    const auto load_group = [&](int n) {
+        mbar_expect_tx(&full[n % NST], kStageBytes);
+        tma_load_3d(ring + (n % NST) * (kStageBytes / 16), &tmap, &full[n % NST], i0 * 2, j0, (g0 + n) * 2);
+    };
+    if (tid == 0) {
+        for (int st = 0; st < NST; ++st) {
+            mbar_init(&full[st], 1);
+            mbar_init(&empty[st], kRows64);
+        }
+        mbar_fence_init();
+        if (ngr > 0) load_group(0);
+    }
+    uint32_t word = 0, fullm = 0;   // bit t: cell t plain, 4 + t: to be zeroed, 8 + 4 t: its face mask
+#pragma unroll
+    for (int t = 0; t < ZC; ++t) {
+        const int j = jt + t;
+        const bool in = i < g.nx && j < g.ny;
+        const long cell = (long)j * g.nx + i;
+        const uint8_t fl = in ? a.flags[cell] : 0;
+        double *const cz = coef + t * NT;       // slot k of the cell: cz[k * ZC * NT]
+        if (fl & kPlain) {
+            word |= 1u << t;
+#pragma unroll
+            for (int k = 0; k < (SHAK ? kC64S : kC64); ++k) cz[k * ZC * NT] = a.cf[k * nc + cell];
+        }
+        if (fl & kZero) word |= 16u << t;
+        const uint32_t mk = fl >> kMaskShift;
+        word |= mk << (8 + 4 * t);
+        if (__all_sync(0xffffffffu, !in || ((fl & kPlain) && (!MUSCL || mk == 0xF)))) fullm |= 1u << t;
+    }
+    const bool busy = __any_sync(0xffffffffu, (word & 0xFFu) != 0);
+    __syncthreads();
+
+    const int cb = (ty * ZC + 2) * kTileX + tx + 2;
+    const long pc0 = nbr(g, i, jt);
+    const int pitch = g.nx + 4;
+    // padding mirrors along x: offset of the first one (0: none); a second one
+    // twice as far on zero-gradient sides, where the offset is one cell
+    int mx = 0;
+    if (g.bc[0] == DVM_BC_PERIODIC) mx = i < 2 ? g.nx : (i >= g.nx - 2 ? -g.nx : 0);
+    else if (i == 0 && g.bc[0] == DVM_BC_ZEROGRAD) mx = -1;
+    else if (i == g.nx - 1 && g.bc[1] == DVM_BC_ZEROGRAD) mx = 1;
+    const auto store = [&](double2 *d, int j, const double (&o)[2]) {
+        vst<double>(d, o);
+        if (mx) vst<double>(d + mx, o);
+        if (mx == 1 || mx == -1) vst<double>(d + 2 * mx, o);
+        if (g.bc[2] == DVM_BC_PERIODIC) {
+            if (j < 2) vst<double>(d + (long)g.ny * pitch, o);
+            else if (j >= g.ny - 2) vst<double>(d - (long)g.ny * pitch, o);
+        } else {
+            if (j == 0 && g.bc[2] == DVM_BC_ZEROGRAD) { vst<double>(d - pitch, o); vst<double>(d - 2 * pitch, o); }
+            if (j == g.ny - 1 && g.bc[3] == DVM_BC_ZEROGRAD) { vst<double>(d + pitch, o); vst<double>(d + 2 * pitch, o); }
+        }
+    };
+    double q[ZC][4];                        // moment sums of the thread's cells (physical order)
+#pragma unroll
+    for (int t = 0; t < ZC; ++t)
+#pragma unroll
+        for (int m = 0; m < 4; ++m) q[t][m] = 0;
+    double Mr[ZC], Rr[ZC], Er[ZC], kyr[ZC], d4r[ZC];   // recurrence; the row's factor and Shakhov terms
+#pragma unroll
+    for (int t = 0; t < ZC; ++t) Mr[t] = Rr[t] = Er[t] = kyr[t] = d4r[t] = 0;
+    const double2 *const pt = reinterpret_cast<const double2 *>(a.pt);
+    uint32_t bad = 0;
+    int p1 = (g0 * 2) % g.nvx;
+    bool first = true;
+    for (int it = 0; it < ngr; ++it) {
+        if (tid == 0 && it + 1 < ngr) {
+            // the next group into the slot that group it - 2 left
+            if (it + 1 >= NST)
+                mbar_wait_or(smem_u32(&empty[(it + 1) % NST]), (uint32_t)(((it + 1) / NST - 1) & 1), bad);
+            load_group(it + 1);
+        }
+        mbar_wait_or(smem_u32(&full[it % NST]), (uint32_t)((it / NST) & 1), bad);
+        const int grp = g0 + it;
+        if (busy) {
+            const double2 *const tile = ring + (it % NST) * (kStageBytes / 16) + cb;
+            double nnux[2], nnuy[2], kx[2], ky[2], vx[2], vy[2], ke[2];
+            {
+                double *const rows[7] = {nnux, nnuy, kx, ky, vx, vy, ke};
+#pragma unroll
+                for (int k = 0; k < 7; ++k) {
+                    const double2 v = __ldg(pt + (long)grp * 7 + k);
+                    rows[k][0] = v.x;
+                    rows[k][1] = v.y;
+                }
+            }
+            const int sy = a.gsign[2 * grp + 1];
+            // equilibria of f and g (the Maxwellian of f alone under BGK)
+            double fe[ZC][2], ge[ZC][2];
+#pragma unroll
+            for (int e = 0; e < 2; ++e) {
+                const bool pad = grp * 2 + e >= g.nv;
+                if ((p1 % rec == 0 || first) && !pad) {
+                    const int b = p1 / rec;
+#pragma unroll
+                    for (int t = 0; t < ZC; ++t) {
+                        const double *const cz = coef + t * NT;
+                        if (p1 == 0 || first) {
+                            const double dy = vy[e] - cz[kUy * ZC * NT], c2 = cz[kC2 * ZC * NT];
+                            Er[t] = exp2(-c2 * dy * dy);
+                            if constexpr (SHAK) {
+                                // k c.q = kqx dx + kqy dy, |c|^2/T - 4 = dx^2/T + (dy^2/T - 4)
+                                kyr[t] = cz[kKqy * ZC * NT] * dy;
+                                d4r[t] = fma(dy * cz[kIT * ZC * NT], dy, -4.0);
+                            }
+                        }
+                        Mr[t] = cz[(kMb + b) * ZC * NT] * Er[t];
+                        Rr[t] = cz[(kRb + b) * ZC * NT];
+                        for (int k = b * rec; k < p1; ++k) {          // a split that starts inside a row
+                            Mr[t] *= Rr[t];
+                            Rr[t] *= cz[kQm * ZC * NT];
+                        }
+                    }
+                    first = false;
+                }
+#pragma unroll
+                for (int t = 0; t < ZC; ++t) {
+                    const double *const cz = coef + t * NT;
+                    fe[t][e] = pad ? 0.0 : Mr[t];
+                    if constexpr (SHAK) {
+                        const double dx = vx[e] - cz[kUx * ZC * NT];
+                        const double mk = fe[t][e] * fma(cz[kKqx * ZC * NT], dx, kyr[t]);
+                        fe[t][e] = fma(mk, fma(dx * cz[kIT * ZC * NT], dx, d4r[t]), fe[t][e]);
+                        ge[t][e] = fma(2.0, mk, fe[t][e]);
+                    } else {
+                        ge[t][e] = fe[t][e];
+                    }
+                    Mr[t] *= Rr[t];
+                    Rr[t] *= cz[kQm * ZC * NT];
+                }
+                if (++p1 == g.nvx) p1 = 0;
+            }
+            // the row differences beyond the warp's ends, one lane each: the two
+            // of row t, component comp, velocity e in lanes 2 (e + 2 comp + 4 t)
+            // and the next: D(32), and D(-1) (v_x >= 0) or D(33)
+            double xe = 0;
+            {
+                const int e = (tx >> 1) & 1, comp = (tx >> 2) & 1, t = (tx >> 3) & 1;
+                const bool px = (e ? vx[1] : vx[0]) >= 0;
+                const int at = (tx & 1) ? (px ? -1 : 33) : 32;
+                const double2 *const p = tile - tx + comp * PL + t * kTileX + at;
+                xe = ld_unit(p, e) - ld_unit(p - 1, e);
+            }
+            uint32_t bw[ZC] = {0, 0};
+            double2 *const o0 = reinterpret_cast<double2 *>(a.fout) + (long)grp * 2 * g.slab + pc0;
+#pragma unroll
+            for (int comp = 0; comp < 2; ++comp) {
+                const double2 *const pl = tile + comp * PL;
+                // along y: the two rows in physical order and their
+                // neighbours; face s has the rows s and s + 1 on its sides
+                double f[ZC][2], d[ZC + 3][2], m[ZC + 1][2];
+                {
+                    // rows -2 .. ZC + 1 around the cells; the outermost one on
+                    // the downwind side is not read
+                    double r0[2], r1[2], r4[2], r5[2];
+                    ld_units(pl, f[0]);
+                    ld_units(pl + kTileX, f[1]);
+                    ld_units(pl - kTileX, r1);
+                    ld_units(pl + 2 * kTileX, r4);
+                    if (MUSCL) {
+                        if (sy >= 0) ld_units(pl - 2 * kTileX, r0);
+                        if (sy <= 0) ld_units(pl + 3 * kTileX, r5);
+                    }
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        if (MUSCL || sy >= 0) d[1][e] = f[0][e] - r1[e];
+                        d[2][e] = f[1][e] - f[0][e];
+                        if (MUSCL || sy <= 0) d[3][e] = r4[e] - f[1][e];
+                        if (MUSCL) {
+                            if (sy >= 0) d[0][e] = r1[e] - r0[e];
+                            if (sy <= 0) d[4][e] = r5[e] - r4[e];
+                        }
+                        // limiter value of the face below row s: of the
+                        // differences across it and across its upwind
+                        // neighbour; the second argument is the upwind one
+                        if (MUSCL) {
+                            if (sy > 0 || (sy == 0 && vy[e] >= 0)) {
+                                m[0][e] = minmod3(d[1][e], d[0][e]);
+                                m[1][e] = minmod3(d[2][e], d[1][e]);
+                                m[2][e] = minmod3(d[3][e], d[2][e]);
+                            } else {
+                                m[0][e] = minmod3(d[1][e], d[2][e]);
+                                m[1][e] = minmod3(d[2][e], d[3][e]);
+                                m[2][e] = minmod3(d[3][e], d[4][e]);
+                            }
+                        }
+                    }
+                }
+#pragma unroll
+                for (int t = 0; t < ZC; ++t) {
+                    const bool whole = (fullm >> t) & 1u;
+                    const uint32_t mk = word >> (8 + 4 * t);
+                    const double *const cz = coef + t * NT;
+                    const double r = cz[kRel * ZC * NT];
+                    double out[2];
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        const bool px = vx[e] >= 0, py = sy > 0 || (sy == 0 && vy[e] >= 0);
+                        // differences D(i) = f(i) - f(i - 1) along the row: a
+                        // lane forms its own, takes its neighbours' from them,
+                        // and the two beyond the warp's end from xe
+                        const double di = f[t][e] - ld_unit(pl + t * kTileX - 1, e);
+                        double dx = di, dd = 0, du = 0;     // upwind face; next downwind; next upwind
+                        {
+                            const int src = 2 * (e + 2 * comp + 4 * t);
+                            const double e0 = __shfl_sync(0xffffffffu, xe, src), e1 = __shfl_sync(0xffffffffu, xe, src + 1);
+                            double dn = __shfl_down_sync(0xffffffffu, di, 1);
+                            if (tx == 31) dn = e0;                              // D(32)
+                            if (px) {
+                                if (MUSCL) {
+                                    dd = dn;
+                                    du = __shfl_up_sync(0xffffffffu, di, 1);
+                                    if (tx == 0) du = e1;                       // D(-1)
+                                }
+                            } else {
+                                dx = dn;
+                                if (MUSCL) {
+                                    dd = di;
+                                    du = __shfl_down_sync(0xffffffffu, di, 2);
+                                    if (tx == 30) du = e0;
+                                    if (tx == 31) du = e1;                      // D(33)
+                                }
+                            }
+                        }
+                        // the differences across the upwind faces and their
+                        // limited slopes, in +x and +y; nnux and nnuy carry
+                        // the signs of v_x and v_y
+                        double dy = py ? d[t + 1][e] : d[t + 2][e];
+                        if (MUSCL) {
+                            const double mo = minmod3(dd, dx), mi = minmod3(dx, du);
+                            if (REC) {
+                                if (mk & (px ? 2u : 1u)) bw[t] |= branch_code(mo, dx) << ((comp * 4 + e) * 2);
+                                if (mk & (py ? 8u : 4u))
+                                    bw[t] |= (py ? branch_code(m[t + 1][e], d[t + 1][e]) : branch_code(m[t][e], d[t + 2][e]))
+                                             << ((comp * 4 + 2 + e) * 2);
+                            }
+                            // outgoing and incoming face
+                            const double yo = py ? m[t + 1][e] : m[t][e], yi = py ? m[t][e] : m[t + 1][e];
+                            if (whole) {
+                                dx = fma(kx[e], mo - mi, dx);
+                                dy = fma(ky[e], yo - yi, dy);
+                            } else {
+                                const auto w = [&](uint32_t bit, double x) { return (mk & bit) ? x : 0.0; };
+                                dx = fma(w(px ? 2u : 1u, kx[e]), mo, fma(-w(px ? 1u : 2u, kx[e]), mi, dx));
+                                dy = fma(w(py ? 8u : 4u, ky[e]), yo, fma(-w(py ? 4u : 8u, ky[e]), yi, dy));
+                            }
+                        }
+                        // the increment first: r M - r f and the fluxes round
+                        // at their own size, the sum once
+                        double o = fma(-r, f[t][e], comp == 0 ? fe[t][e] : cz[kGf * ZC * NT] * ge[t][e]);
+                        o = fma(nnux[e], dx, o);
+                        o = fma(nnuy[e], dy, o);
+                        o += f[t][e];
+                        if (!whole && !((word >> t) & 1u)) o = 0;
+                        out[e] = o;
+                        if (comp == 0) {
+                            q[t][0] += o;
+                            q[t][1] = fma(vx[e], o, q[t][1]);
+                            q[t][2] = fma(vy[e], o, q[t][2]);
+                            q[t][3] = fma(ke[e], o, q[t][3]);
+                        } else {
+                            q[t][3] += o;
+                        }
+                    }
+                    if (((word >> t) | (word >> (4 + t))) & 1u) store(o0 + comp * g.slab + t * pitch, jt + t, out);
+                }
+            }
+            if (REC)
+#pragma unroll
+                for (int t = 0; t < ZC; ++t)
+                    if ((word >> t) & 1u)
+                        a.bits[(long)grp * a.bslab + (long)(jt + t + 2) * a.bpitch + i + 2] = bw[t];
+        }
+        __syncwarp();
+        mbar_arrive_if(smem_u32(&empty[it % NST]), tx == 0);
+    }
+    if (bad) atomicExch(&a.err[kErrTimeout], 1);
+#pragma unroll
+    for (int t = 0; t < ZC; ++t) {
+        if (!(((word >> t) | (word >> (4 + t))) & 1u)) continue;
+        const long cell = (long)(jt + t) * g.nx + i;
+#pragma unroll
+        for (int m = 0; m < 4; ++m) a.pout[((long)split * 4 + m) * nc + cell] = q[t][m];
     }
 }
 
@@ -1356,6 +1727,18 @@ __global__ void __launch_bounds__(32 * kMomChunks) k_partials(Grid2D g, int S, c
     write_member_partials<T>(part, S, nc, cell, keep, s[0].value(), s[1].value(), s[2].value(), s[3].value());
 }
 
+// Check of a state from the moment sums that the step left with it: raises
+// the non-physical flag for a gas cell with rho <= 0 or T <= 0.
+template <typename T>
+__global__ void k_check(Grid2D g, int S, const T *part, const int8_t *type, int *err)
+{
+    const long nc = (long)g.nx * g.ny, cell = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (cell >= nc || type[cell] == DVM_SOLID) return;
+    T s[4], rho, ux, uy, tmp;
+    gather_partials(part, S, nc, cell, s);
+    if (!primitives<T>(pick<T>(g.dv_f, g.dv), s[0], s[1], s[2], s[3], rho, ux, uy, tmp)) atomicExch(&err[kErrNonphys], 1);
+}
+
 // Moments for output: rho, ux, uy, uz (= 0), T per cell, formed in FP64 from
 // the sums (compensated in the state precision).
 template <typename T>
@@ -1685,20 +2068,55 @@ __global__ void k_tables(Grid2D g, VCoef<T> *vt, int8_t *gsign, float4 *ptab)
         }
         if (W == 4)
             for (int r = 0; r < 7; ++r) ptab[p * 7 + r] = make_float4(row[r][0], row[r][1], row[r][2], row[r][3]);
+        if (W == 2) {
+            // FP64: seven double2 rows -nu_x and -nu_y with the velocity's
+            // sign, (1 - nu_x)/2, (1 - nu_y)/2, vx, vy, |v|^2/2
+            double2 *const d = reinterpret_cast<double2 *>(ptab) + p * 7;
+            for (int e = 0; e < 2; ++e) {
+                const int q = p * 2 + e;
+                double vx = 0, vy = 0, nux = 0, nuy = 0;
+                if (q < g.nv) {
+                    vx = g.vxmin + (q % g.nvx) * g.dvx;
+                    vy = g.vymin + (q / g.nvx) * g.dvy;
+                    nux = fabs(vx) * (g.dt / g.dx);
+                    nuy = fabs(vy) * (g.dt / g.dy);
+                }
+                const double r[7] = {vx < 0 ? nux : -nux, vy < 0 ? nuy : -nuy, 0.5 * (1.0 - nux), 0.5 * (1.0 - nuy), vx, vy,
+                                     0.5 * (vx * vx + vy * vy)};
+                for (int k = 0; k < 7; ++k) (e ? d[k].y : d[k].x) = r[k];
+            }
+        }
     }
 }
 
 inline int nblk(long n, int b) { return (int)((n + b - 1) / b); }
 
+// The bulk kernel of a precision, its threads and shared memory.
+template <bool MUSCL, bool REC, bool SHAK> struct BulkKernel {
+    static constexpr auto kernel32 = k_bulk<float, MUSCL, REC, SHAK>;
+    static constexpr auto kernel64 = k_bulk64<MUSCL, REC, SHAK>;
+    static constexpr size_t smem32 = (size_t)kStages * kStageBytes + 2 * kStages * sizeof(uint64_t) +
+                                     (SHAK ? kSaccBytes : 0);
+    static constexpr size_t smem64 = bulk64_smem<SHAK>();
+};
+
 template <typename T, bool MUSCL, bool REC, bool SHAK>
 cudaError_t launch_bulk(dvm_ctx *c, const BulkArgs<T> &a)
 {
-    const size_t smem = (size_t)kStages * kStageBytes + 2 * kStages * sizeof(uint64_t) +
-                        (SHAK && sizeof(T) == 4 ? kSaccBytes : 0);
+    using K = BulkKernel<MUSCL, REC, SHAK>;
+    constexpr size_t smem = sizeof(T) == 4 ? K::smem32 : K::smem64;
+    if constexpr (sizeof(T) == 8) {
+        constexpr int cells = 128 / kCellThreads;
+        k_cell64<SHAK><<<(unsigned)((c->nc + cells - 1) / cells), 128, 0, c->stream>>>(a, c->cf64);
+        c->launches += 1;
+    }
+    const auto kernel = [] {
+        if constexpr (sizeof(T) == 4) return K::kernel32;
+        else return K::kernel64;
+    }();
     static bool attr = false;
     if (!attr) {
-        cudaError_t e = cudaFuncSetAttribute(k_bulk<T, MUSCL, REC, SHAK>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                             (int)smem);
+        cudaError_t e = cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
         attr = true;
     }
@@ -1715,7 +2133,7 @@ cudaError_t launch_bulk(dvm_ctx *c, const BulkArgs<T> &a)
     }();
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(nblk(c->nx, 32), nblk(c->ny, kRows), c->S);
-    cfg.blockDim = dim3(32, kRows);
+    cfg.blockDim = sizeof(T) == 4 ? dim3(32, kRows) : dim3(32 * kRows64);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = c->stream;
     cudaLaunchAttribute at[1];
@@ -1723,7 +2141,7 @@ cudaError_t launch_bulk(dvm_ctx *c, const BulkArgs<T> &a)
     at[0].val.priority = prio;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_bulk<T, MUSCL, REC, SHAK>, a, c->tmap[c->cur]);
+    return cudaLaunchKernelEx(&cfg, kernel, a, c->tmap[c->cur]);
 }
 
 // Moment sums of each cell over this context's velocities, folded over the
@@ -1901,6 +2319,7 @@ cudaError_t step2d_t(dvm_ctx *c, int phase, double *xbuf)
     a.g = g; a.S = c->S; a.Sin = Sin; a.fin = fin; a.fout = fout; a.pin = pin; a.pout = pout;
     a.flags = c->flags; a.vt = (const VCoef<T> *)c->vtab; a.gsign = c->gsign; a.err = c->d_err;
     a.pt = (const ulonglong2 *)c->ptab;
+    a.cf = c->cf64;
     a.eqp = cons && !imex ? (const T *)c->eqp : nullptr;
     a.qh = shak && !hraw ? (const T *)c->qheat : nullptr;
     a.hin = hraw ? (const T *)c->hpart[c->cur] : nullptr;
@@ -2008,6 +2427,8 @@ size_t vcoef_bytes(int prec) { return prec == DVM_FP32 ? sizeof(VCoef<float>) : 
 
 size_t cvinfo_bytes() { return sizeof(CvInfo); }
 
+size_t cf64_bytes2d(const dvm_ctx *c) { return sizeof(double) * kC64S * (size_t)c->nc; }
+
 cudaError_t members2d(dvm_ctx *c, bool moving)
 {
     CvArgs cv{};
@@ -2081,6 +2502,17 @@ cudaError_t partials_from_state2d(dvm_ctx *c)
         k_partials<double><<<grid, block, 0, c->stream>>>(g, c->S, (const double *)c->f[c->cur],
                                                           (const VCoef<double> *)c->vtab, (double *)c->part[c->cur],
                                                           c->geo[c->gcur].type, c->d_err);
+    return cudaGetLastError();
+}
+
+cudaError_t check_moments2d(dvm_ctx *c)
+{
+    const Grid2D g = grid2d(c);
+    const int8_t *type = c->geo[c->gcur].type;
+    if (c->prec == DVM_FP32)
+        k_check<float><<<nblk(c->nc, 128), 128, 0, c->stream>>>(g, c->S, (const float *)c->part[c->cur], type, c->d_err);
+    else
+        k_check<double><<<nblk(c->nc, 128), 128, 0, c->stream>>>(g, c->S, (const double *)c->part[c->cur], type, c->d_err);
     return cudaGetLastError();
 }
 

@@ -113,7 +113,8 @@ template <typename T>
 __device__ __forceinline__ void gather_partials3(const T *part, int S, long nc, long cell, T (&s)[5])
 {
     Acc<T> a[5];
-    for (int q = 0; q < S; ++q)
+#pragma unroll 4
+    for (int q = 0; q < S; ++q)       // several splits' loads in flight
 #pragma unroll
         for (int m = 0; m < 5; ++m) a[m].merge(part[((long)q * 5 + m) * nc + cell], T(0));
 #pragma unroll
@@ -142,6 +143,7 @@ template <typename T> struct Bulk3Args {
     const VX3<T> *vxt;        // [nvxp]
     const VYZ3<T> *vyz;       // [nvy * nvz]
     const T *eqp;             // [5][nc] conservative equilibrium parameters, or null (direct moments)
+    const double *cf;         // FP64: per-cell values [kMxCount][nc] (k_cell64_3)
     const T *qh;              // [3][nc] heat flux of the control volume at t^n (Shakhov model)
     T pr1;                    // 1 - Pr (Shakhov model)
     int *err;
@@ -166,8 +168,7 @@ template <bool SHAK> __host__ __device__ constexpr int ring3() { return SHAK?5:k
 // Per-cell values of the bulk kernel in shared memory.  FP32: c0, c1, c2, r
 // (one vector), uy, uz, and the Shakhov model's k q.  FP64: the values of
 // MxSlot for the Maxwellian's recurrence along v_x.
-constexpr int kMxBlocks = 4;         // restarts of the recurrence along a v_x row
-enum MxSlot { kMxUy = 0, kMxUz, kMxC2, kMxOmr, kMxQ, kMxM, kMxR = kMxM + kMxBlocks, kMxCount = kMxR + kMxBlocks };
+enum MxSlot { kMxUy = 0, kMxUz, kMxC2, kMxRel, kMxQ, kMxM, kMxR = kMxM + kMxBlocks, kMxCount = kMxR + kMxBlocks };
 template <typename T, bool SHAK> __host__ __device__ constexpr int ncoef3()
 {
     return sizeof(T) == 8 ? kMxCount : (SHAK ? 9 : 6);
@@ -200,6 +201,44 @@ __device__ __forceinline__ double exp2_state(double x) { return exp2(x); }
 // Lane l of a unit.
 __device__ __forceinline__ float unit_lane(F2 x, int l) { float a, b; f2_get(x, a, b); return l ? b : a; }
 __device__ __forceinline__ double unit_lane(double x, int) { return x; }
+
+// The per-cell values of the FP64 bulk kernel for the plain cells
+// (dvm_device.cuh): the slots of MxSlot.  Block = 16 cells x kCellThreads.
+__global__ void __launch_bounds__(128) k_cell64_3(Bulk3Args<double> a, double *cf)
+{
+    const Grid3D &g = a.g;
+    const long nc = (long)g.nx * g.ny * g.nz;
+    const long cell = (long)blockIdx.x * (128 / kCellThreads) + threadIdx.x / kCellThreads;
+    const int k = threadIdx.x % kCellThreads;
+    const bool plain = cell < nc && (a.flags[cell] & kPlain);
+    double s[5] = {0, 0, 0, 0, 0};
+    if (plain)
+#pragma unroll 4
+        for (int q = k; q < a.Sin; q += kCellThreads)
+#pragma unroll
+            for (int m = 0; m < 5; ++m) s[m] += a.pin[((long)q * 5 + m) * nc + cell];
+#pragma unroll
+    for (int m = 0; m < 5; ++m) s[m] = cell_sum(s[m]);
+    if (!plain) return;
+    double rho, ux, uy, uz, tmp;
+    if (!primitives3<double>(g.dv, s, rho, ux, uy, uz, tmp) && k == 0) atomicExch(&a.err[kErrNonphys], 1);
+    const double r = g.dt_tau0 * rho;
+    if (a.eqp) {
+        // conservative equilibrium (Sec. 3.1): tau from the direct density,
+        // the Maxwellian from the Newton parameters
+        rho = a.eqp[cell]; ux = a.eqp[nc + cell]; uy = a.eqp[2 * nc + cell];
+        uz = a.eqp[3 * nc + cell]; tmp = a.eqp[4 * nc + cell];
+    }
+    const double c2 = (0.5 * kLog2e) / tmp;
+    double *const o = cf + cell;
+    put_recurrence(o, nc, k, g.nvx, g.vxmin, g.dvx, ux, c2, r * rho * norm3(tmp), kMxQ, kMxM, kMxR);
+    if (k == kCellThreads - 1) {
+        o[kMxUy * nc] = uy;
+        o[kMxUz * nc] = uz;
+        o[kMxC2 * nc] = c2;
+        o[kMxRel * nc] = r;
+    }
+}
 
 // Bulk update of every gas cell that is a control volume on its own.
 //
@@ -292,7 +331,7 @@ __global__ void __launch_bounds__(32 * warps3<T>(), 1)
         tma_load_4d(ring + slot * PC, &tmap, &full[slot], i0 * W, j0, grp >= gpos ? z0 + o : z0 + ZC + 3 - o, grp);
     };
     // velocities between restarts of the FP64 recurrence
-    const int rec = g.nvx <= 8 * kMxBlocks ? 8 : 16;
+    const int rec = restart64(g.nvx);
 
     if (tid == 0) {
         for (int st = 0; st < RING; ++st) {
@@ -340,31 +379,22 @@ __global__ void __launch_bounds__(32 * warps3<T>(), 1)
         T *const cz = cq + t * NCQ * NT + tid;
         if (fl & kPlain) {
             word |= 1u << t;
-            T s[5];
-            gather_partials3(a.pin, a.Sin, nc, cell, s);
-            T rho, ux, uy, uz, tmp;
-            if (!primitives3<T>(pick<T>(g.dv_f, g.dv), s, rho, ux, uy, uz, tmp)) atomicExch(&a.err[kErrNonphys], 1);
-            const T r = pick<T>(g.dt_tau0_f, g.dt_tau0) * rho;
-            if (a.eqp) {
-                // conservative equilibrium (Sec. 3.1): tau from the direct
-                // density, the Maxwellian from the Newton parameters
-                rho = a.eqp[cell]; ux = a.eqp[nc + cell]; uy = a.eqp[2 * nc + cell];
-                uz = a.eqp[3 * nc + cell]; tmp = a.eqp[4 * nc + cell];
-            }
-            const T c2 = T(kLog2e) / (T(2) * tmp);
             if constexpr (F64) {
-                const T dv = T(g.dvx), A = r * rho * norm3(tmp);
-                cz[kMxUy * NT] = uy;
-                cz[kMxUz * NT] = uz;
-                cz[kMxC2 * NT] = c2;
-                cz[kMxOmr * NT] = T(1) - r;
-                cz[kMxQ * NT] = exp2(T(-2) * c2 * dv * dv);
-                for (int b = 0; b * rec < g.nvxp; ++b) {
-                    const T dx = T(g.vxmin) + T(b * rec) * dv - ux;
-                    cz[(kMxM + b) * NT] = A * exp2(-c2 * dx * dx);
-                    cz[(kMxR + b) * NT] = exp2(-c2 * (T(2) * dx * dv + dv * dv));
-                }
+#pragma unroll
+                for (int k = 0; k < NCO; ++k) cz[k * NT] = a.cf[k * nc + cell];
             } else {
+                T s[5];
+                gather_partials3(a.pin, a.Sin, nc, cell, s);
+                T rho, ux, uy, uz, tmp;
+                if (!primitives3<T>(g.dv_f, s, rho, ux, uy, uz, tmp)) atomicExch(&a.err[kErrNonphys], 1);
+                const T r = g.dt_tau0_f * rho;
+                if (a.eqp) {
+                    // conservative equilibrium (Sec. 3.1): tau from the direct
+                    // density, the Maxwellian from the Newton parameters
+                    rho = a.eqp[cell]; ux = a.eqp[nc + cell]; uy = a.eqp[2 * nc + cell];
+                    uz = a.eqp[3 * nc + cell]; tmp = a.eqp[4 * nc + cell];
+                }
+                const T c2 = T(kLog2e) / (T(2) * tmp);
                 T *const cv = coef + (t * NT + tid) * 4;
                 cv[0] = log2(rho * norm3(tmp)) - c2 * ux * ux;
                 cv[1] = T(2) * c2 * ux;
@@ -564,7 +594,7 @@ __global__ void __launch_bounds__(32 * warps3<T>(), 1)
             if constexpr (F64) {
                 const T *const cz = cq + t * NCQ * NT + tid;
                 const T Q = cz[kMxQ * NT];
-                r = cz[kMxOmr * NT];
+                r = cz[kMxRel * NT];
 #pragma unroll
                 for (int e = 0; e < W; ++e) {
                     feq[e] = xg * W + e < g.nvx ? Mr[s] : T(0);
@@ -648,10 +678,13 @@ __global__ void __launch_bounds__(32 * warps3<T>(), 1)
                             }
                         }
                         const T fc = unit_lane(f0[h], l), q = feq[e];
-                        T o = F64 ? fma(r, fc, q) : fma(r, q - fc, fc);
+                        // FP64 (q is r M): the increment first, so that it
+                        // rounds at its own size and the sum once
+                        T o = F64 ? fma(-r, fc, q) : fma(r, q - fc, fc);
                         o = fma(unit_lane(nnux[h], l), dx, o);
                         o = fma(-cyz.nuy, dy, o);
                         o = fma(-cyz.nuz, dz, o);
+                        if (F64) o += fc;
                         if constexpr (!FULL) o = ((*cellw >> t) & 1u) ? o : T(0);
                         out[e] = o;
                     }
@@ -680,10 +713,11 @@ __global__ void __launch_bounds__(32 * warps3<T>(), 1)
                         dz = fma(-zi, unit_lane(mi[h], l), fma(zo, unit_lane(mo[h], l), dz));
                     }
                     const T q = feq[e];
-                    T o = F64 ? fma(r, fc, q) : fma(r, q - fc, fc);
+                    T o = F64 ? fma(-r, fc, q) : fma(r, q - fc, fc);
                     o = fma(unit_lane(nnux[h], l), dx, o);
                     o = fma(-cyz.nuy, dy, o);
                     o = fma(-cyz.nuz, dz, o);
+                    if (F64) o += fc;
                     out[e] = ((*cellw >> t) & 1u) ? o : T(0);
                 }
             }
@@ -1271,6 +1305,17 @@ __global__ void __launch_bounds__(32 * kMomChunks) k_partials3(Grid3D g, int S, 
         for (int m = 0; m < 5; ++m) part[((long)q * 5 + m) * nc + cell] = q == 0 ? v[m] : T(0);
 }
 
+// Check of a state from the moment sums that the step left with it, as in 2D.
+template <typename T>
+__global__ void k_check3(Grid3D g, int S, const T *part, const int8_t *type, int *err)
+{
+    const long nc = (long)g.nx * g.ny * g.nz, cell = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (cell >= nc || type[cell] == DVM_SOLID) return;
+    T s[5], rho, ux, uy, uz, tmp;
+    gather_partials3(part, S, nc, cell, s);
+    if (!primitives3<T>(pick<T>(g.dv_f, g.dv), s, rho, ux, uy, uz, tmp)) atomicExch(&err[kErrNonphys], 1);
+}
+
 // Moments for output: rho, ux, uy, uz, T per cell, formed in FP64 from the
 // sums (compensated in the state precision).
 template <typename T>
@@ -1607,6 +1652,11 @@ cudaError_t launch_bulk3(dvm_ctx *c, const Bulk3Args<T> &a)
         if (e != cudaSuccess) return e;
         attr = true;
     }
+    if constexpr (sizeof(T) == 8) {
+        constexpr int cells = 128 / kCellThreads;
+        k_cell64_3<<<(unsigned)((c->nc + cells - 1) / cells), 128, 0, c->stream>>>(a, c->cf64);
+        c->launches += 1;
+    }
     constexpr int threads = 32 * warps3<T>();
     const dim3 grid(nb3(c->nx, a.tx), nb3(c->ny, a.ty), (unsigned)(a.nzc * a.S));
     k_bulk3<T, MUSCL, SHAK><<<grid, threads, smem, c->stream>>>(a, c->tmap[c->cur]);
@@ -1771,6 +1821,7 @@ cudaError_t step3d_t(dvm_ctx *c, int phase, double *xbuf)
     a.qh = shak ? (const T *)c->qheat : nullptr;
     a.pr1 = T(1.0 - c->Pr);
     a.fin = fin; a.fout = fout; a.pin = pin; a.pout = pout;
+    a.cf = c->cf64;
     a.flags = c->flags3; a.vxt = vx_table<T>(c); a.vyz = vyz_table<T>(c); a.err = c->d_err;
     if ((e = timing_mark(c, 0)) != cudaSuccess) return e;
     e = launch_bulk3_any<T>(c, a, shak);
@@ -1890,6 +1941,8 @@ size_t vtab3_bytes(const dvm_ctx *c) { return (size_t)c->nvxp * 2 * c->elem + (s
 
 size_t cvinfo3_bytes() { return sizeof(CvInfo3); }
 
+size_t cf64_bytes3d(const dvm_ctx *c) { return sizeof(double) * kMxCount * (size_t)c->nc; }
+
 cudaError_t members3d(dvm_ctx *c)
 {
     k_members3<<<4 * 152, 256, 0, c->stream>>>(cv3_args(c), (CvInfo3 *)c->cvinfo);
@@ -1934,6 +1987,18 @@ cudaError_t partials_from_state3d(dvm_ctx *c)
         k_partials3<double><<<grid, block, 0, c->stream>>>(g, c->S, (const double *)c->f[c->cur],
                                                            vx_table<double>(c), vyz_table<double>(c),
                                                            (double *)c->part[c->cur], c->geo3.type, c->d_err);
+    return cudaGetLastError();
+}
+
+cudaError_t check_moments3d(dvm_ctx *c)
+{
+    const Grid3D g = grid3d(c);
+    if (c->prec == DVM_FP32)
+        k_check3<float><<<nb3(c->nc, 128), 128, 0, c->stream>>>(g, c->S, (const float *)c->part[c->cur], c->geo3.type,
+                                                                c->d_err);
+    else
+        k_check3<double><<<nb3(c->nc, 128), 128, 0, c->stream>>>(g, c->S, (const double *)c->part[c->cur], c->geo3.type,
+                                                                 c->d_err);
     return cudaGetLastError();
 }
 
