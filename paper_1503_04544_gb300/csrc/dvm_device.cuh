@@ -419,6 +419,37 @@ __device__ __forceinline__ T block_acc(Acc<T> a, T *red)
     return t.value();
 }
 
+// N compensated sums at once over each group of kw consecutive warps of the
+// block, in three barriers: out[m] on every thread of the group, formed as
+// block_acc forms it (a warp tree, then the warps in order).  red: 2 N values
+// per warp and N per warp after them.  Every thread of the block calls it.
+template <int N, typename T>
+__device__ __forceinline__ void group_acc(Acc<T> (&a)[N], T (&out)[N], T *red, int kw)
+{
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, w0 = warp / kw * kw;
+    const int w1 = min(w0 + kw, (int)(blockDim.x >> 5));
+#pragma unroll
+    for (int m = 0; m < N; ++m) a[m].warp_reduce();
+    __syncthreads();                  // the last use of red is over
+    if (lane == 0)
+#pragma unroll
+        for (int m = 0; m < N; ++m) {
+            red[2 * (warp * N + m)] = a[m].s;
+            red[2 * (warp * N + m) + 1] = a[m].c;
+        }
+    __syncthreads();
+    T *const res = red + 2 * N * (blockDim.x >> 5);
+    const int m = threadIdx.x - 32 * w0;
+    if (m < N) {
+        Acc<T> t;
+        for (int w = w0; w < w1; ++w) t.merge(red[2 * (w * N + m)], red[2 * (w * N + m) + 1]);
+        res[w0 * N + m] = t.value();
+    }
+    __syncthreads();
+#pragma unroll
+    for (int q = 0; q < N; ++q) out[q] = res[w0 * N + q];
+}
+
 template <typename T>
 __device__ __forceinline__ T block_sum(T v, T *red)
 {

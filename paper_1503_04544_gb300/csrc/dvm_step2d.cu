@@ -265,6 +265,32 @@ __device__ __forceinline__ void bulk_tile_x2(const float4 *t, int c0, int ux1, i
     }
 }
 
+// The first-order form: no limited terms, two neighbours a cell.
+template <int COMP>
+__device__ __forceinline__ void bulk_tile_up_x2(const float4 *t, int c0, int ux1, int uy1, const PairCoef &P,
+                                                const F2 (&feq)[2], F2 r, float (&out)[4], F2 (&Q)[4])
+{
+    F2 f[2], u1[2], w1[2];
+    ld_units(t + c0, f);
+    ld_units(t + c0 - ux1, u1);
+    ld_units(t + c0 - uy1, w1);
+#pragma unroll
+    for (int h = 0; h < 2; ++h) {
+        F2 O = fma2(P.nnx[h], sub2(f[h], u1[h]), f[h]);
+        O = fma2(P.nny[h], sub2(f[h], w1[h]), O);
+        O = fma2(r, sub2(feq[h], f[h]), O);
+        f2_get(O, out[2 * h], out[2 * h + 1]);
+        if (COMP == 0) {
+            Q[0] = add2(Q[0], O);
+            Q[1] = fma2(P.vx[h], O, Q[1]);
+            Q[2] = fma2(P.vy[h], O, Q[2]);
+            Q[3] = fma2(P.ke[h], O, Q[3]);
+        } else {
+            Q[3] = add2(Q[3], O);
+        }
+    }
+}
+
 // Adds the two lanes of each packed moment sum to q0..q3 and clears them.
 template <typename T>
 __device__ __forceinline__ void fold_pairs(F2 (&Q)[4], T &q0, T &q1, T &q2, T &q3)
@@ -505,7 +531,7 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<T> a, const __g
 
     // the exponent's per-cell terms as pairs (packed path)
     F2 EL0, E1X, E1Y, NC2;
-    if constexpr (sizeof(T) == 4 && MUSCL) {
+    {
         EL0 = f2(el0); E1X = f2(e1x); E1Y = f2(e1y); NC2 = f2(-2.f * c2);
     }
     Acc<T> m0, m1, m2, m3;
@@ -545,7 +571,7 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<T> a, const __g
             // pairs: the scalar path's sums of this group go there at its end
             T t0 = 0, t1 = 0, t2 = 0, t3 = 0;
             T &p0 = sel<HRAW>(t0, q0), &p1 = sel<HRAW>(t1, q1), &p2 = sel<HRAW>(t2, q2), &p3 = sel<HRAW>(t3, q3);
-            if constexpr (sizeof(T) == 4 && MUSCL) {
+            {
                 if (sx != 0 && sy != 0) {
                     // packed FP32 path of the sign-uniform groups, coefficients
                     // from the group's rows of the packed table
@@ -565,13 +591,23 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<T> a, const __g
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
                         {
-                            // log2 M = el0 - 2 c2 |v|^2/2 + e1x vx + e1y vy
-                            F2 X = fma2(NC2, P.ke[h], EL0);
-                            X = fma2(E1X, P.vx[h], X);
-                            X = fma2(E1Y, P.vy[h], X);
+                            F2 X;
                             float x0, x1;
-                            f2_get(X, x0, x1);
-                            fq[h] = f2(ex2_fast(x0), ex2_fast(x1));
+                            if constexpr (MUSCL || SHAK) {
+                                // log2 M = el0 - 2 c2 |v|^2/2 + e1x vx + e1y vy
+                                X = fma2(NC2, P.ke[h], EL0);
+                                X = fma2(E1X, P.vx[h], X);
+                                X = fma2(E1Y, P.vy[h], X);
+                                f2_get(X, x0, x1);
+                                fq[h] = f2(ex2_fast(x0), ex2_fast(x1));
+                            } else {
+                                // M = A 2^(-c2 |v - u|^2): the first-order form
+                                // is bound by memory and has room for it
+                                const F2 DX = sub2(P.vx[h], f2(ux)), DY = sub2(P.vy[h], f2(uy));
+                                X = mul2(fma2(DY, DY, mul2(DX, DX)), f2(-c2));
+                                f2_get(X, x0, x1);
+                                fq[h] = mul2(f2(A), f2(ex2_fast(x0), ex2_fast(x1)));
+                            }
                             if constexpr (SHAK) {
                                 // |c|^2/T - 4 = 2 (log2 A - log2 M) / log2 e - 4,
                                 // k c.q = kqx vx + kqy vy - (kqx ux + kqy uy);
@@ -586,7 +622,10 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<T> a, const __g
                         }
                     }
                     const F2 r2 = f2(r);
-                    bulk_tile_x2<0, REC>(tile, c0, ux1, uy1, P, fq, wxm, wxp, wym, wyp, r2, out, Qp, bw);
+                    if constexpr (MUSCL)
+                        bulk_tile_x2<0, REC>(tile, c0, ux1, uy1, P, fq, wxm, wxp, wym, wyp, r2, out, Qp, bw);
+                    else
+                        bulk_tile_up_x2<0>(tile, c0, ux1, uy1, P, fq, r2, out, Qp);
                     store_cell<T>(o0, pc, mir, anymir, out);
                     if constexpr (SHAK) {
                         hmom_x2<0>(f2(out[0], out[1]), P.vx[0], P.vy[0], P.ke[0], Hp);
@@ -598,8 +637,11 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<T> a, const __g
                         const F2 gf = f2(gfac);
                         fq[0] = mul2(fq[0], gf); fq[1] = mul2(fq[1], gf);
                     }
-                    bulk_tile_x2<1, REC>(tile + kTileY * kTileX, c0, ux1, uy1, P, fq, wxm, wxp, wym, wyp, r2, out,
-                                         Qp, bw);
+                    if constexpr (MUSCL)
+                        bulk_tile_x2<1, REC>(tile + kTileY * kTileX, c0, ux1, uy1, P, fq, wxm, wxp, wym, wyp, r2, out,
+                                             Qp, bw);
+                    else
+                        bulk_tile_up_x2<1>(tile + kTileY * kTileX, c0, ux1, uy1, P, fq, r2, out, Qp);
                     store_cell<T>(o0 + g.slab, pc, mir, anymir, out);
                     if constexpr (SHAK) {
                         hmom_x2<1>(f2(out[0], out[1]), P.vx[0], P.vy[0], P.ke[0], Hp);
@@ -671,7 +713,7 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<T> a, const __g
                     fold_lanes<4>(Qp, 0, sacc, tid);
                     fold_lanes<5>(Hp, 4, sacc, tid);
                 } else {
-                    if constexpr (sizeof(T) == 4 && MUSCL) fold_pairs(Qp, q0, q1, q2, q3);
+                    fold_pairs(Qp, q0, q1, q2, q3);
                     m0.add(q0); m1.add(q1); m2.add(q2); m3.add(q3);
                     q0 = q1 = q2 = q3 = 0;
                 }
@@ -706,7 +748,7 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<T> a, const __g
                 a.hout[((long)a.S * 5 + 1) * nc + cell] = 0;
             }
         } else {
-            if constexpr (sizeof(T) == 4 && MUSCL) fold_pairs(Qp, q0, q1, q2, q3);
+            fold_pairs(Qp, q0, q1, q2, q3);
             m0.add(q0); m1.add(q1); m2.add(q2); m3.add(q3);
             a.pout[((long)split * 4 + 0) * nc + cell] = m0.value();
             a.pout[((long)split * 4 + 1) * nc + cell] = m1.value();
@@ -1277,33 +1319,44 @@ __device__ __forceinline__ void write_split_partials(T *part, int s, long nc, lo
     part[((long)s * 4 + 3) * nc + k] = keep ? s3 : T(0);
 }
 
+// Copy of one control-volume record into shared memory (16-byte words).
+__device__ __forceinline__ void load_info(const CvInfo *src, CvInfo *dst)
+{
+    static_assert(sizeof(CvInfo) % 16 == 0, "CvInfo is copied in 16-byte words");
+    const int4 *s4 = reinterpret_cast<const int4 *>(src);
+    int4 *d4 = reinterpret_cast<int4 *>(dst);
+    for (int q = threadIdx.x; q < (int)(sizeof(CvInfo) / 16); q += blockDim.x) d4[q] = __ldg(s4 + q);
+    __syncthreads();
+}
+
 // Fusion (Eq. FusionDD): f_CV = sum sbar f / S over a merged control volume,
 // written back to every member, with the moment sums of the result.  One
 // work item is one control volume and one velocity split.
 template <typename T>
 __global__ void __launch_bounds__(256) k_fusion(CvArgs c, T *f, T *part)
 {
-    __shared__ T red[8 * 2];
+    __shared__ T red[8 * 3 * 4];
+    __shared__ __align__(16) CvInfo I;
     const Grid2D &g = c.g;
     const CvInfo *info = reinterpret_cast<const CvInfo *>(c.cvinfo);
     const VCoef<T> *vt = reinterpret_cast<const VCoef<T> *>(c.vt);
     const long nc = (long)g.nx * g.ny;
     const int n = min(c.counts[0], c.cap) * c.S;
     for (int item = blockIdx.x; item < n; item += gridDim.x) {
-        const CvInfo &I = info[item / c.S];
         const int sp = item % c.S;
-        const int nm = I.nm;
+        const int nm = info[item / c.S].nm;
         if (nm <= 1) continue;
+        load_info(info + item / c.S, &I);
         int v0, v1;
         split_range(c, sp, Vec<T>::W, v0, v1);
-        const double S = I.Sn;
-        Acc<T> a0, a1, a2, a3;
+        const double rS = 1.0 / I.Sn;    // a division per value was most of the FP64 work
+        Acc<T> a[4];
         for (int comp = 0; comp < 2; ++comp)
             for (int p = v0 + threadIdx.x; p < v1; p += blockDim.x) {
                 const long base = ebase<T>(g, comp, p);
                 double acc = 0;
                 for (int q = 0; q < nm; ++q) acc += I.mem[q].sb * (double)f[base + I.mem[q].pc * Vec<T>::W];
-                const T fcv = (T)(acc / S);
+                const T fcv = (T)(acc * rS);
                 for (int q = 0; q < nm; ++q) {
                     f[base + I.mem[q].pc * Vec<T>::W] = fcv;
                     for (int t = 0; t < 4; ++t)
@@ -1311,17 +1364,18 @@ __global__ void __launch_bounds__(256) k_fusion(CvArgs c, T *f, T *part)
                 }
                 const VCoef<T> vc = ld_coef(vt + p);
                 if (comp == 0) {
-                    a0.add(fcv); a1.add(vc.vx * fcv); a2.add(vc.vy * fcv);
-                    a3.add(T(0.5) * (vc.vx * vc.vx + vc.vy * vc.vy) * fcv);
+                    a[0].add(fcv); a[1].add(vc.vx * fcv); a[2].add(vc.vy * fcv);
+                    a[3].add(T(0.5) * (vc.vx * vc.vx + vc.vy * vc.vy) * fcv);
                 } else {
-                    a3.add(fcv);
+                    a[3].add(fcv);
                 }
             }
-        const T t0 = block_acc(a0, red), t1 = block_acc(a1, red), t2 = block_acc(a2, red), t3 = block_acc(a3, red);
+        T t[4];
+        group_acc(a, t, red, 8);
         if (threadIdx.x < nm) {
             const CvMember &M = I.mem[threadIdx.x];
             const long k = (long)M.j * g.nx + M.i;
-            write_split_partials<T>(part, sp, nc, k, M.live != 0, t0, t1, t2, t3);
+            write_split_partials<T>(part, sp, nc, k, M.live != 0, t[0], t[1], t[2], t[3]);
         }
         __syncthreads();
     }
@@ -1341,6 +1395,9 @@ struct WallGeom {
     double rx, ry, uwx, uwy, Tw, nwx, nwy, lw;
 };
 
+// Called by a whole warp: the sectors of a piecewise wall temperature are
+// tested 32 at a time (64 of them one after the other, twice a wall cell, took
+// 35 of the 59 us of the wall kernel).
 __device__ __forceinline__ WallGeom wall_geom(const CvArgs &c, const BodyParams &b, long k, double omega)
 {
     WallGeom w;
@@ -1348,7 +1405,21 @@ __device__ __forceinline__ WallGeom wall_geom(const CvArgs &c, const BodyParams 
     w.ry = c.Gn.rwy[k] - b.cy;
     w.uwx = b.vbx - w.ry * omega;
     w.uwy = b.vby + w.rx * omega;
-    w.Tw = wall_temperature(b, w.rx, w.ry);
+    w.Tw = b.Tw;
+    if (b.nseg > 0) {
+        // the first sector that holds the point, as wall_temperature
+        int s = 0;
+        for (int s0 = 0; s0 < b.nseg; s0 += 32) {
+            const int q = s0 + (threadIdx.x & 31), t = (q + 1) % b.nseg;
+            bool in = false;
+            if (q < b.nseg)
+                in = b.seg_dir[2 * q] * w.ry - b.seg_dir[2 * q + 1] * w.rx >= 0 &&
+                     b.seg_dir[2 * t] * w.ry - b.seg_dir[2 * t + 1] * w.rx < 0;
+            const unsigned hit = __ballot_sync(0xffffffffu, in);
+            if (hit) { s = s0 + __ffs(hit) - 1; break; }
+        }
+        w.Tw = b.Tw_seg[s];
+    }
     w.nwx = c.Gn.nwx[k];
     w.nwy = c.Gn.nwy[k];
     w.lw = c.Gn.lw[k];
@@ -1373,8 +1444,9 @@ __global__ void __launch_bounds__(256) k_wall(CvArgs c, BodyParams b, BodyDev *b
     __shared__ double red[8 * 8];
     __shared__ double ex[kMaxAxisNv], ey[kMaxAxisNv];
     __shared__ double wsc[6];   // uwx, uwy, nwx, nwy, 1/(2 pi Tw), 2 Tw
+    __shared__ WallGeom wg;
     using WA = typename std::conditional<sizeof(T) == 4, float, double>::type;   // wall-sum type
-    __shared__ WA wred[8 * 2];
+    __shared__ WA wred[8 * 3 * 8];
     __shared__ bool last;
     const Grid2D &g = c.g;
     const int nw = min(c.counts[1], c.cap);
@@ -1383,15 +1455,18 @@ __global__ void __launch_bounds__(256) k_wall(CvArgs c, BodyParams b, BodyDev *b
     for (int idx = blockIdx.x; idx < nw; idx += gridDim.x) {
         const long k = c.wall_list[idx];
         double r0, r1, r2, r3, r4, r5, r6, r7;
+        if (tid < 32) {
+            const WallGeom w = wall_geom(c, b, k, omega);
+            if (tid == 0) {
+                wg = w;
+                wsc[0] = w.uwx; wsc[1] = w.uwy; wsc[2] = w.nwx; wsc[3] = w.nwy;
+                wsc[4] = 1.0 / (2.0 * kPi * w.Tw); wsc[5] = 2.0 * w.Tw;
+            }
+        }
         if (mode == 2) {
             const double *x = xw + 8L * idx;
             r0 = x[0]; r1 = x[1]; r2 = x[2]; r3 = x[3]; r4 = x[4]; r5 = x[5]; r6 = x[6]; r7 = x[7];
         } else {
-        if (tid == 0) {
-            const WallGeom w = wall_geom(c, b, k, omega);
-            wsc[0] = w.uwx; wsc[1] = w.uwy; wsc[2] = w.nwx; wsc[3] = w.nwy;
-            wsc[4] = 1.0 / (2.0 * kPi * w.Tw); wsc[5] = 2.0 * w.Tw;
-        }
         __syncthreads();
         const double uwx = wsc[0], uwy = wsc[1], nwx = wsc[2], nwy = wsc[3], cm = wsc[4], twoTw = wsc[5];
         // separable Maxwellian M[1, u_w, T_w] = ex[p1] ey[p2] / (2 pi T_w)
@@ -1401,7 +1476,7 @@ __global__ void __launch_bounds__(256) k_wall(CvArgs c, BodyParams b, BodyDev *b
         }
         __syncthreads();
         const long pck = pcell(g, k) * Vec<T>::W;
-        Acc<WA> a0, a1, a2, a3, a4, a5, a6, a7;
+        Acc<WA> w8[8];
         int p1 = tid % g.nvx, p2 = tid / g.nvx;
         const int dp1 = blockDim.x % g.nvx, dp2 = blockDim.x / g.nvx;
         for (int p = tid; p < g.nv; p += blockDim.x) {
@@ -1410,19 +1485,19 @@ __global__ void __launch_bounds__(256) k_wall(CvArgs c, BodyParams b, BodyDev *b
             const WA cw = (WA)cp, axw = (WA)ax, ayw = (WA)ay;
             if (cp > 0.0) {
                 const WA fv = (WA)f[ebase<T>(g, 0, p) + pck];
-                a0.add(cw * fv);
-                a5.add(axw * axw * fv); a6.add(axw * ayw * fv); a7.add(ayw * ayw * fv);
+                w8[0].add(cw * fv);
+                w8[5].add(axw * axw * fv); w8[6].add(axw * ayw * fv); w8[7].add(ayw * ayw * fv);
             } else if (cp < 0.0) {
                 const WA m1 = (WA)(cm * ex[p1] * ey[p2]);
-                a1.add(cw * m1);
-                a2.add(axw * axw * m1); a3.add(axw * ayw * m1); a4.add(ayw * ayw * m1);
+                w8[1].add(cw * m1);
+                w8[2].add(axw * axw * m1); w8[3].add(axw * ayw * m1); w8[4].add(ayw * ayw * m1);
             }
             p1 += dp1; p2 += dp2;
             if (p1 >= g.nvx) { p1 -= g.nvx; p2 += 1; }
         }
-        r0 = block_acc(a0, wred); r1 = block_acc(a1, wred); r2 = block_acc(a2, wred);
-        r3 = block_acc(a3, wred); r4 = block_acc(a4, wred); r5 = block_acc(a5, wred);
-        r6 = block_acc(a6, wred); r7 = block_acc(a7, wred);
+        WA rv[8];
+        group_acc(w8, rv, wred, 8);
+        r0 = rv[0]; r1 = rv[1]; r2 = rv[2]; r3 = rv[3]; r4 = rv[4]; r5 = rv[5]; r6 = rv[6]; r7 = rv[7];
         if (mode == 1) {
             if (tid == 0) {
                 double *x = xw + 8L * idx;
@@ -1433,7 +1508,7 @@ __global__ void __launch_bounds__(256) k_wall(CvArgs c, BodyParams b, BodyDev *b
         }
         }
         if (tid == 0) {
-            const WallGeom w = wall_geom(c, b, k, omega);
+            const WallGeom w = wg;
             const double phi = -(r0 * g.dv) / (r1 * g.dv);
             const double sxx = (phi * r2 + r5) * g.dv, sxy = (phi * r3 + r6) * g.dv;
             const double syy = (phi * r4 + r7) * g.dv;
@@ -1488,36 +1563,36 @@ __device__ __forceinline__ T fval(const Grid2D &g, const T *f, int i, int j, int
 // incoming velocities (Eq. BoundaryDDv; phi from the FP64 wall kernel), area
 // ratio S^n / S^{n+1,*}, relaxation, then distribution to the members (Eq.
 // UpdateDD; members solid at t^{n+1} hold 0) and the moment sums of the
-// velocity split.  One work item is one control volume and one split.
-// Copy of one control-volume record into shared memory (16-byte words).
-__device__ __forceinline__ void load_info(const CvInfo *src, CvInfo *dst)
-{
-    static_assert(sizeof(CvInfo) % 16 == 0, "CvInfo is copied in 16-byte words");
-    const int4 *s4 = reinterpret_cast<const int4 *>(src);
-    int4 *d4 = reinterpret_cast<int4 *>(dst);
-    for (int q = threadIdx.x; q < (int)(sizeof(CvInfo) / 16); q += blockDim.x) d4[q] = __ldg(s4 + q);
-    __syncthreads();
-}
-
+// velocity split.  One work item is one control volume and as many splits as
+// the block's warps hold: a split of up to 32 kw velocities takes kw warps, so
+// that the short splits of a small velocity grid share a block (64^2 x 20^2
+// cells, 16 splits of 28 velocities: 48 us a launch with a block for each,
+// @SP@ us with eight a block) and their sums are formed as by a block of their
+// own.
 template <typename T>
 __global__ void __launch_bounds__(256) k_special(CvArgs c, const T *fin, T *fout, const T *pin,
                                                  T *pout, const double *wdat)
 {
-    __shared__ T red[8 * 2];
+    __shared__ T red[8 * 3 * 5];
     __shared__ __align__(16) CvInfo I;
     const Grid2D &g = c.g;
     const CvInfo *info = reinterpret_cast<const CvInfo *>(c.cvinfo);
     const VCoef<T> *vt = reinterpret_cast<const VCoef<T> *>(c.vt);
     const long nc = (long)g.nx * g.ny;
-    const int n = min(c.counts[0], c.cap) * c.S;
     constexpr int W = Vec<T>::W;
+    // warps of a split (1, 2, 4 or 8), splits of a block
+    const int range = c.gps * W, kw = range <= 32 ? 1 : range <= 64 ? 2 : range <= 128 ? 4 : 8, nsb = 8 / kw;
+    const int items = (c.S + nsb - 1) / nsb;
+    const int n = min(c.counts[0], c.cap) * items;
+    const int gt = threadIdx.x % (32 * kw);          // thread of the split's warps
     for (int item = blockIdx.x; item < n; item += gridDim.x) {
-        const int idx = item / c.S, sp = item % c.S;
+        const int idx = item / items, sp = item % items * nsb + (threadIdx.x >> 5) / kw;
         load_info(info + idx, &I);
         if (!I.ok) { __syncthreads(); continue; }
         const int nm = I.nm;
         int v0, v1;
         split_range(c, sp, W, v0, v1);
+        const bool on = sp < c.S;
         const long m = c.spec_list[idx];
         T s[4];
         gather_partials(pin, c.Sin, nc, m, s);
@@ -1535,24 +1610,26 @@ __global__ void __launch_bounds__(256) k_special(CvArgs c, const T *fin, T *fout
         // volume at t^n, summed here over every velocity of its (fused) state
         T kqx = 0, kqy = 0;
         if (c.shak) {
-            Acc<T> h0, h1;
+            Acc<T> h[2];
             for (int p = threadIdx.x; p < g.nv; p += blockDim.x) {
                 const VCoef<T> vc = ld_coef(vt + p);
                 const T dx = vc.vx - ux, dy = vc.vy - uy;
                 const T fa = fin[ebase<T>(g, 0, p) + I.pcm * W], fb = fin[ebase<T>(g, 1, p) + I.pcm * W];
                 const T w = T(0.5) * (dx * dx + dy * dy) * fa + fb;
-                h0.add(dx * w);
-                h1.add(dy * w);
+                h[0].add(dx * w);
+                h[1].add(dy * w);
             }
             const T dv = pick<T>(g.dv_f, g.dv);
-            const T qx = block_acc(h0, red) * dv, qy = block_acc(h1, red) * dv;
+            T hv[2];
+            group_acc(h, hv, red, 8);
+            const T qx = hv[0] * dv, qy = hv[1] * dv;
             const T k = T(c.pr1) / (T(5) * rho * tmp * tmp);
             kqx = k * qx;
             kqy = k * qy;
         }
-        Acc<T> s0, s1, s2, s3;
+        Acc<T> sum[4];
         Acc<T> hs[5];     // Shakhov: raw heat-flux moments of the new state about (ux, uy)
-        for (int p = v0 + threadIdx.x; p < v1; p += blockDim.x) {
+        for (int p = v0 + gt; p < v1; p += 32 * kw) {
             const VCoef<T> vc = ld_coef(vt + p);
             const T vx = vc.vx, vy = vc.vy, nux = vc.nux, nuy = vc.nuy;
             const T dxu = vx - ux, dyu = vy - uy;
@@ -1617,10 +1694,10 @@ __global__ void __launch_bounds__(256) k_special(CvArgs c, const T *fin, T *fout
                         if (M.mir[t] >= 0) fout[base + M.mir[t] * W] = v;
                 }
                 if (comp == 0) {
-                    s0.add(fn); s1.add(vx * fn); s2.add(vy * fn);
-                    s3.add(T(0.5) * (vx * vx + vy * vy) * fn);
+                    sum[0].add(fn); sum[1].add(vx * fn); sum[2].add(vy * fn);
+                    sum[3].add(T(0.5) * (vx * vx + vy * vy) * fn);
                 } else {
-                    s3.add(fn);
+                    sum[3].add(fn);
                 }
                 if (c.hout) {
                     if (comp == 0) {
@@ -1633,18 +1710,17 @@ __global__ void __launch_bounds__(256) k_special(CvArgs c, const T *fin, T *fout
                 }
             }
         }
-        const T t0 = block_acc(s0, red), t1 = block_acc(s1, red);
-        const T t2 = block_acc(s2, red), t3 = block_acc(s3, red);
-        if (threadIdx.x < nm) {
-            const CvMember &M = I.mem[threadIdx.x];
-            write_split_partials<T>(pout, sp, nc, (long)M.j * g.nx + M.i, M.keep != 0, t0, t1, t2, t3);
+        T tv[4];
+        group_acc(sum, tv, red, kw);
+        if (on && gt < nm) {
+            const CvMember &M = I.mem[gt];
+            write_split_partials<T>(pout, sp, nc, (long)M.j * g.nx + M.i, M.keep != 0, tv[0], tv[1], tv[2], tv[3]);
         }
         if (c.hout) {
             T hv[5];
-#pragma unroll
-            for (int q = 0; q < 5; ++q) hv[q] = block_acc(hs[q], red);
-            if (threadIdx.x < nm) {
-                const CvMember &M = I.mem[threadIdx.x];
+            group_acc(hs, hv, red, kw);
+            if (on && gt < nm) {
+                const CvMember &M = I.mem[gt];
                 const long k = (long)M.j * g.nx + M.i;
                 const bool keep = M.keep != 0;
                 T *ho = static_cast<T *>(c.hout);
