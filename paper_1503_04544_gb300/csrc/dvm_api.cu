@@ -350,6 +350,9 @@ int dvm_create(const dvm_grid *grid, const dvm_vgrid *vg, const dvm_physics *ph,
         for (int s = 1; s <= (f32 ? 16 : 40) && s <= c->ngrp; ++s) {
             long per_sm = (blocks * s + 151) / 152;
             if (!f32 && per_sm > 3) per_sm = (per_sm + 2) / 3 * 3;
+            // first order in FP32, bound by memory: rounds of the two resident
+            // blocks (512^2 x 40^2: S = 1: 1.42 ms, 2: 1.31, 3: 1.38, 4: 1.32)
+            if (f32 && scheme == DVM_UPWIND) per_sm = (blocks * s + 303) / 304;
             const long cost = per_sm * ((c->ngrp + s - 1) / s + (f32 ? 5 : 2));
             if (best < 0 || cost < best) { best = cost; S = s; }
         }
@@ -402,7 +405,7 @@ int dvm_create(const dvm_grid *grid, const dvm_vgrid *vg, const dvm_physics *ph,
     if (dim == 2) {
         AL(c->vtab, (size_t)c->nvp * vcoef_bytes(c->prec));
         AL(c->gsign, (size_t)2 * c->ngrp);
-        AL(c->ptab, (size_t)c->ngrp * 7 * 16);
+        AL(c->ptab, (size_t)c->ngrp * 8 * 16);
         for (int l = 0; l < 2; ++l) {
             dvm::Geo2D &G = c->geo[l];
             AL(G.phi, sizeof(double) * (c->nx + 1) * (c->ny + 1));

@@ -67,8 +67,7 @@ template <typename T> struct BulkArgs {
     T *pout;                  // partial moments of f^n+1 [S][4][nc]
     const uint8_t *flags;
     const VCoef<T> *vt;       // [nvp]
-    const ulonglong2 *pt;     // [ngrp][7] packed-pair coefficients (FP32 path)
-    const int8_t *gsign;      // [ngrp][2]
+    const float4 *pt;         // [ngrp][kTabRows] coefficients of a group (k_tables)
     const T *eqp;             // [4][nc] conservative equilibrium parameters, or null (direct moments)
     const double *cf;         // FP64: per-cell values [C64][nc] (k_cell64)
     const T *qh;              // [2][nc] heat flux of the control volume at t^n (Shakhov model), used when hin is null
@@ -83,6 +82,13 @@ template <typename T> struct BulkArgs {
 
 // ------------------------------------------------------------ bulk kernel
 constexpr int kStageBytes = 2 * kTileY * kTileX * 16;     // both components of one group
+
+// Rows of a group in the coefficient table: seven rows of coefficients and one
+// with the signs of v_x and v_y in the group (0: mixed).  The FP32 bulk kernel
+// copies a group's rows into its ring stage together with the tile: read
+// through L1 at the start of every group they cost its warps an L2 latency.
+constexpr int kTabRows = 8;
+constexpr int kTabBytes = kTabRows * 16;
 
 
 // Branch the limited reconstruction of a downwind face took (recorded for the
@@ -434,7 +440,8 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<T> a, const __g
     using V = typename Vec<T>::type;
     extern __shared__ __align__(128) unsigned char smem[];
     V *ring = reinterpret_cast<V *>(smem);
-    uint64_t *full = reinterpret_cast<uint64_t *>(smem + kStages * kStageBytes);
+    const float4 *const tab = reinterpret_cast<const float4 *>(smem + kStages * kStageBytes);   // [kStages][kTabRows]
+    uint64_t *full = reinterpret_cast<uint64_t *>(smem + kStages * (kStageBytes + kTabBytes));
     uint64_t *empty = full + kStages;
     const Grid2D &g = a.g;
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * 32 + tx;
@@ -452,16 +459,20 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<T> a, const __g
     const bool plain = (fl & kPlain) != 0, zero = (fl & kZero) != 0;
     V *fout = reinterpret_cast<V *>(a.fout);
 
+    // tile and coefficients of group n of the split into its stage
+    const auto load_group = [&](int n) {
+        const int st = n % kStages;
+        mbar_expect_tx(&full[st], kStageBytes + kTabBytes);
+        tma_load_3d(ring + (long)st * (kStageBytes / 16), &tmap, &full[st], i0 * W, j0, (g0 + n) * 2);
+        bulk_load(smem + kStages * kStageBytes + st * kTabBytes, a.pt + (long)(g0 + n) * kTabRows, kTabBytes, &full[st]);
+    };
     if (tid == 0) {
         for (int st = 0; st < kStages; ++st) {
             mbar_init(&full[st], 1);
             mbar_init(&empty[st], kRows);
         }
         mbar_fence_init();
-        for (int st = 0; st < kStages - 1 && st < ngr; ++st) {
-            mbar_expect_tx(&full[st], kStageBytes);
-            tma_load_3d(ring + (long)st * (kStageBytes / 16), &tmap, &full[st], i0 * W, j0, (g0 + st) * 2);
-        }
+        for (int st = 0; st < kStages - 1 && st < ngr; ++st) load_group(st);
     }
 
     // equilibrium of the cell at t^n
@@ -545,7 +556,7 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<T> a, const __g
     F2 Hp[5];
 #pragma unroll
     for (int m = 0; m < 5; ++m) Hp[m] = f2(0.f);
-    float *sacc = reinterpret_cast<float *>(smem + kStages * kStageBytes + 2 * kStages * sizeof(uint64_t));
+    float *sacc = reinterpret_cast<float *>(smem + kStages * (kStageBytes + kTabBytes) + 2 * kStages * sizeof(uint64_t));
     if constexpr (HRAW) {
 #pragma unroll
         for (int m = 0; m < 2 * kSaccRows; ++m) sacc[m * 32 * kRows + tid] = 0;
@@ -557,14 +568,15 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<T> a, const __g
             const int k = it + kStages - 1, s2 = k % kStages;
             if (k >= kStages && !mbar_wait(&empty[s2], (uint32_t)((k / kStages - 1) & 1)))
                 atomicExch(&a.err[kErrTimeout], 1);
-            mbar_expect_tx(&full[s2], kStageBytes);
-            tma_load_3d(ring + (long)s2 * (kStageBytes / 16), &tmap, &full[s2], i0 * W, j0, (g0 + k) * 2);
+            load_group(k);
         }
         if (!mbar_wait(&full[st], (uint32_t)((it / kStages) & 1))) atomicExch(&a.err[kErrTimeout], 1);
         const V *tile = ring + (long)st * (kStageBytes / 16);
         V *o0 = fout + (long)q * 2 * g.slab;
         if (plain) {
-            const int sx = a.gsign[2 * q], sy = a.gsign[2 * q + 1];
+            const ulonglong2 *const pt = reinterpret_cast<const ulonglong2 *>(tab + st * kTabRows);
+            const int2 sg = *reinterpret_cast<const int2 *>(pt + 7);
+            const int sx = sg.x, sy = sg.y;
             T vx[W], vy[W], nux[W], nuy[W], feq[W], out[W];
             uint32_t bw = 0;
             // the FP32 Shakhov variant keeps every moment sum in the per-lane
@@ -578,11 +590,10 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<T> a, const __g
                     const int ux1 = sx > 0 ? 1 : -1, uy1 = sy > 0 ? kTileX : -kTileX;
                     PairCoef P;
                     {
-                        const ulonglong2 *pt = a.pt + (long)q * 7;
                         F2 *rows[7] = {P.nnx, P.nny, P.onx, P.ony, P.vx, P.vy, P.ke};
 #pragma unroll
                         for (int k = 0; k < 7; ++k) {
-                            const ulonglong2 v = __ldg(pt + k);
+                            const ulonglong2 v = pt[k];
                             rows[k][0].v = v.x;
                             rows[k][1].v = v.y;
                         }
@@ -954,12 +965,12 @@ __global__ void __launch_bounds__(32 * kRows64, SHAK ? 2 : 3)
                 double *const rows[7] = {nnux, nnuy, kx, ky, vx, vy, ke};
 #pragma unroll
                 for (int k = 0; k < 7; ++k) {
-                    const double2 v = __ldg(pt + (long)grp * 7 + k);
+                    const double2 v = __ldg(pt + (long)grp * kTabRows + k);
                     rows[k][0] = v.x;
                     rows[k][1] = v.y;
                 }
             }
-            const int sy = a.gsign[2 * grp + 1];
+            const int sy = __ldg(reinterpret_cast<const int2 *>(pt + (long)grp * kTabRows + 7)).y;
             // equilibria of f and g (the Maxwellian of f alone under BGK)
             double fe[ZC][2], ge[ZC][2];
 #pragma unroll
@@ -2096,9 +2107,10 @@ __global__ void __launch_bounds__(1024) k_sum(const double *x, long n, double *o
 }
 
 // Per-velocity coefficients, per-group sign of the velocity components and
-// the FP32 coefficients of each group in the order of the packed path: seven
-// float4 rows -nux, -nuy, 1 - nux, 1 - nuy, vx, vy, |v|^2/2 over the group's
-// four lanes (lanes 0, 1 and 2, 3 form the two pairs).
+// the coefficients of each group, kTabRows rows: FP32 seven float4 rows -nux,
+// -nuy, 1 - nux, 1 - nuy, vx, vy, |v|^2/2 over the group's four lanes (lanes 0,
+// 1 and 2, 3 form the two pairs), FP64 seven double2 rows, and in both the
+// signs as two integers.
 template <typename T>
 __global__ void k_tables(Grid2D g, VCoef<T> *vt, int8_t *gsign, float4 *ptab)
 {
@@ -2127,6 +2139,8 @@ __global__ void k_tables(Grid2D g, VCoef<T> *vt, int8_t *gsign, float4 *ptab)
         }
         gsign[2 * p] = xp ? 1 : (xn ? -1 : 0);
         gsign[2 * p + 1] = yp ? 1 : (yn ? -1 : 0);
+        ptab[p * kTabRows + 7] = make_float4(__int_as_float(xp ? 1 : (xn ? -1 : 0)), __int_as_float(yp ? 1 : (yn ? -1 : 0)),
+                                             0.f, 0.f);
         float row[7][4];
         for (int e = 0; e < 4; ++e) {
             const int q = p * 4 + e;
@@ -2143,11 +2157,11 @@ __global__ void k_tables(Grid2D g, VCoef<T> *vt, int8_t *gsign, float4 *ptab)
             row[6][e] = 0.5f * (vx * vx + vy * vy);
         }
         if (W == 4)
-            for (int r = 0; r < 7; ++r) ptab[p * 7 + r] = make_float4(row[r][0], row[r][1], row[r][2], row[r][3]);
+            for (int r = 0; r < 7; ++r) ptab[p * kTabRows + r] = make_float4(row[r][0], row[r][1], row[r][2], row[r][3]);
         if (W == 2) {
             // FP64: seven double2 rows -nu_x and -nu_y with the velocity's
             // sign, (1 - nu_x)/2, (1 - nu_y)/2, vx, vy, |v|^2/2
-            double2 *const d = reinterpret_cast<double2 *>(ptab) + p * 7;
+            double2 *const d = reinterpret_cast<double2 *>(ptab) + p * kTabRows;
             for (int e = 0; e < 2; ++e) {
                 const int q = p * 2 + e;
                 double vx = 0, vy = 0, nux = 0, nuy = 0;
@@ -2171,7 +2185,7 @@ inline int nblk(long n, int b) { return (int)((n + b - 1) / b); }
 template <bool MUSCL, bool REC, bool SHAK> struct BulkKernel {
     static constexpr auto kernel32 = k_bulk<float, MUSCL, REC, SHAK>;
     static constexpr auto kernel64 = k_bulk64<MUSCL, REC, SHAK>;
-    static constexpr size_t smem32 = (size_t)kStages * kStageBytes + 2 * kStages * sizeof(uint64_t) +
+    static constexpr size_t smem32 = (size_t)kStages * (kStageBytes + kTabBytes) + 2 * kStages * sizeof(uint64_t) +
                                      (SHAK ? kSaccBytes : 0);
     static constexpr size_t smem64 = bulk64_smem<SHAK>();
 };
@@ -2393,8 +2407,8 @@ cudaError_t step2d_t(dvm_ctx *c, int phase, double *xbuf)
     }
     BulkArgs<T> a{};
     a.g = g; a.S = c->S; a.Sin = Sin; a.fin = fin; a.fout = fout; a.pin = pin; a.pout = pout;
-    a.flags = c->flags; a.vt = (const VCoef<T> *)c->vtab; a.gsign = c->gsign; a.err = c->d_err;
-    a.pt = (const ulonglong2 *)c->ptab;
+    a.flags = c->flags; a.vt = (const VCoef<T> *)c->vtab; a.err = c->d_err;
+    a.pt = (const float4 *)c->ptab;
     a.cf = c->cf64;
     a.eqp = cons && !imex ? (const T *)c->eqp : nullptr;
     a.qh = shak && !hraw ? (const T *)c->qheat : nullptr;
