@@ -573,6 +573,13 @@ __device__ __forceinline__ void put_recurrence(double *cf, long nc, int k, int n
     }
 }
 
+// Rows of a group in the coefficient table: seven rows of coefficients and one
+// with the signs of v_x and v_y in the group (0: mixed).  The FP32 bulk kernel
+// copies a group's rows into its ring stage together with the tile: read
+// through L1 at the start of every group they cost its warps an L2 latency.
+constexpr int kTabRows = 8;
+constexpr int kTabBytes = kTabRows * 16;
+
 // Per-velocity coefficients: vx, vy, nu_x = |vx| dt/dx, nu_y = |vy| dt/dy.
 // Padded velocities carry a huge speed (their Maxwellian is 0) and zero
 // Courant numbers.

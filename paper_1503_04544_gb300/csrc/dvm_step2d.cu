@@ -5,10 +5,10 @@
 // reduced pair (f, g) (Eqs. FluxDD, ExSchemeDD, BGKDD) and distribution
 // (Eq. UpdateDD).  Device layout: see dvm_internal.h.
 //
-// Kernels of one step (fixed obstacle): k_wall (FP64 wall density, wall
-// fluxes, force/torque, rigid-body update in its last block), k_bulk (every
-// gas cell that is a control volume on its own), k_special (cut and merged
-// control volumes).  A moving obstacle adds the geometry of t^{n+1}, the
+// Kernels of one step (fixed obstacle): k_wall (FP64 wall density and wall
+// fluxes), k_bulk (every gas cell that is a control volume on its own),
+// k_special (cut and merged control volumes; force/torque and rigid-body update
+// in its last block).  A moving obstacle adds the geometry of t^{n+1}, the
 // control volumes of t^n and k_fusion before them.
 //
 // k_bulk: one thread per cell, 32 consecutive cells in x per warp and kRows
@@ -82,13 +82,6 @@ template <typename T> struct BulkArgs {
 
 // ------------------------------------------------------------ bulk kernel
 constexpr int kStageBytes = 2 * kTileY * kTileX * 16;     // both components of one group
-
-// Rows of a group in the coefficient table: seven rows of coefficients and one
-// with the signs of v_x and v_y in the group (0: mixed).  The FP32 bulk kernel
-// copies a group's rows into its ring stage together with the tile: read
-// through L1 at the start of every group they cost its warps an L2 latency.
-constexpr int kTabRows = 8;
-constexpr int kTabBytes = kTabRows * 16;
 
 
 // Branch the limited reconstruction of a downwind face took (recorded for the
@@ -1187,7 +1180,6 @@ struct CvArgs {
     const void *cvinfo;       // control-volume records
     const void *vt;           // per-velocity coefficients (state precision)
     const void *eqp;          // [4][nc] conservative equilibrium parameters, or null
-    int shak;                 // the Shakhov model under the explicit scheme
     void *hout;               // Shakhov: raw heat-flux moments of f^n+1 [S][5][nc] and reference velocity [2][nc]
     double pr1;               // 1 - Pr (Shakhov model)
     int *err;
@@ -1397,11 +1389,9 @@ __global__ void __launch_bounds__(256) k_fusion(CvArgs c, T *f, T *part)
 // torque (Eqs. eq-force, eq-torque), in FP64.  The wall velocity is
 // u_w = u_c + (r - c)^perp omega (Eq. uwDD) at t^n.  A work item is one wall
 // cell and one velocity split: it writes the split's sums over outgoing
-// velocities (of f) and incoming ones (of M[1, u_w, T_w]).  The last block to
-// finish combines the splits of every wall cell in list order: wall density
-// phi, stress, force and torque, their sum over the body, the angular
-// velocity at t^{n+1} (Eq. motionDD_vit) and the history record.  It leaves
-// (phi, u_w, T_w) of each wall cell for the control-volume kernel.
+// velocities (of f) and incoming ones (of M[1, u_w, T_w]), then wall density
+// phi, stress, force and torque.  It leaves (phi, u_w, T_w) of each wall cell
+// and its force and torque for the control-volume kernel.
 struct WallGeom {
     double rx, ry, uwx, uwy, Tw, nwx, nwy, lw;
 };
@@ -1448,17 +1438,14 @@ __device__ __forceinline__ WallGeom wall_geom(const CvArgs &c, const BodyParams 
 // about 1e-7 relative); the wall density, the stress, the force, the torque
 // and the rotation are FP64.
 template <typename T>
-__global__ void __launch_bounds__(256) k_wall(CvArgs c, BodyParams b, BodyDev *body, const T *f,
-                                              double *wdat, double *wcontrib, int *ticket,
-                                              double *hist, int moving, int mode, double *xw)
+__global__ void __launch_bounds__(256) k_wall(CvArgs c, BodyParams b, const BodyDev *body, const T *f,
+                                              double *wdat, double *wcontrib, int mode, double *xw)
 {
-    __shared__ double red[8 * 8];
     __shared__ double ex[kMaxAxisNv], ey[kMaxAxisNv];
     __shared__ double wsc[6];   // uwx, uwy, nwx, nwy, 1/(2 pi Tw), 2 Tw
     __shared__ WallGeom wg;
     using WA = typename std::conditional<sizeof(T) == 4, float, double>::type;   // wall-sum type
     __shared__ WA wred[8 * 3 * 8];
-    __shared__ bool last;
     const Grid2D &g = c.g;
     const int nw = min(c.counts[1], c.cap);
     const double omega = body->omega;
@@ -1532,14 +1519,18 @@ __global__ void __launch_bounds__(256) k_wall(CvArgs c, BodyParams b, BodyDev *b
         }
         __syncthreads();
     }
-    if (mode == 1) return;
-    // the last block sums the contributions in list order
-    __threadfence();
-    __syncthreads();
-    if (tid == 0) last = atomicAdd(ticket, 1) == (int)gridDim.x - 1;
-    __syncthreads();
-    if (!last) return;
-    __threadfence();
+}
+
+// Force and torque over the body, the sum of the wall cells' contributions in
+// a fixed order, then the rotation (Eqs. motionDD_posit, motionDD_vit) and the
+// history record: the work of one block of the control-volume kernel, beside
+// the others (a last block of the wall kernel had the control volumes wait
+// for it, 4 us a step).
+__device__ __forceinline__ void body_update(const CvArgs &c, const BodyParams &b, BodyDev *body, const double *wcontrib,
+                                            double *hist, int moving, double *red)
+{
+    const Grid2D &g = c.g;
+    const int nw = min(c.counts[1], c.cap), tid = threadIdx.x;
     double fx = 0, fy = 0, tq = 0;
     for (int t = tid; t < nw; t += blockDim.x) {
         fx += wcontrib[3 * t]; fy += wcontrib[3 * t + 1]; tq += wcontrib[3 * t + 2];
@@ -1555,7 +1546,6 @@ __global__ void __launch_bounds__(256) k_wall(CvArgs c, BodyParams b, BodyDev *b
         double *h = hist + 6 * (body->step % kHistCap);
         h[0] = fx; h[1] = fy; h[2] = 0; h[3] = tq; h[4] = body->theta; h[5] = om1;
         body->step += 1;
-        *ticket = 0;
     }
 }
 
@@ -1578,13 +1568,23 @@ __device__ __forceinline__ T fval(const Grid2D &g, const T *f, int i, int j, int
 // the block's warps hold: a split of up to 32 kw velocities takes kw warps, so
 // that the short splits of a small velocity grid share a block (64^2 x 20^2
 // cells, 16 splits of 28 velocities: 48 us a launch with a block for each,
-// @SP@ us with eight a block) and their sums are formed as by a block of their
+// 20 us with eight a block) and their sums are formed as by a block of their
 // own.
-template <typename T>
-__global__ void __launch_bounds__(256) k_special(CvArgs c, const T *fin, T *fout, const T *pin,
-                                                 T *pout, const double *wdat)
+// SHAK: the Shakhov model under the explicit scheme.  The last block of the
+// grid updates the body instead (body_update).  One and a half rounds of work
+// items are usual (64^2 x 20^2: 320 on 304 block slots), so the registers are
+// bounded for three blocks per SM (FP32 BGK), which is one round.
+template <typename T, bool SHAK>
+__global__ void __launch_bounds__(256, (sizeof(T) == 4) + !SHAK + 1)
+    k_special(CvArgs c, BodyParams bp, BodyDev *body, const T *fin, T *fout, const T *pin, T *pout, const double *wdat,
+              const double *wcontrib, double *hist, int moving)
 {
     __shared__ T red[8 * 3 * 5];
+    if (blockIdx.x == gridDim.x - 1) {
+        __shared__ double bred[8 * 3];
+        body_update(c, bp, body, wcontrib, hist, moving, bred);
+        return;
+    }
     __shared__ __align__(16) CvInfo I;
     const Grid2D &g = c.g;
     const CvInfo *info = reinterpret_cast<const CvInfo *>(c.cvinfo);
@@ -1596,7 +1596,7 @@ __global__ void __launch_bounds__(256) k_special(CvArgs c, const T *fin, T *fout
     const int items = (c.S + nsb - 1) / nsb;
     const int n = min(c.counts[0], c.cap) * items;
     const int gt = threadIdx.x % (32 * kw);          // thread of the split's warps
-    for (int item = blockIdx.x; item < n; item += gridDim.x) {
+    for (int item = blockIdx.x; item < n; item += gridDim.x - 1) {
         const int idx = item / items, sp = item % items * nsb + (threadIdx.x >> 5) / kw;
         load_info(info + idx, &I);
         if (!I.ok) { __syncthreads(); continue; }
@@ -1620,7 +1620,7 @@ __global__ void __launch_bounds__(256) k_special(CvArgs c, const T *fin, T *fout
         // Shakhov (Eq. ShakhovDD): k q with the heat flux of the control
         // volume at t^n, summed here over every velocity of its (fused) state
         T kqx = 0, kqy = 0;
-        if (c.shak) {
+        if constexpr (SHAK) {
             Acc<T> h[2];
             for (int p = threadIdx.x; p < g.nv; p += blockDim.x) {
                 const VCoef<T> vc = ld_coef(vt + p);
@@ -1646,7 +1646,7 @@ __global__ void __launch_bounds__(256) k_special(CvArgs c, const T *fin, T *fout
             const T dxu = vx - ux, dyu = vy - uy;
             const T feq0 = A * dexp(-(dxu * dxu + dyu * dyu) * i2T);
             T sf = T(1), sg = T(1);
-            if (c.shak) {
+            if constexpr (SHAK) {
                 const T kcq = kqx * dxu + kqy * dyu, d2 = (dxu * dxu + dyu * dyu) * T(2) * i2T;
                 sf = fma(kcq, d2 - T(4), T(1));
                 sg = fma(kcq, d2 - T(2), T(1));
@@ -1710,7 +1710,7 @@ __global__ void __launch_bounds__(256) k_special(CvArgs c, const T *fin, T *fout
                 } else {
                     sum[3].add(fn);
                 }
-                if (c.hout) {
+                if (SHAK && c.hout) {
                     if (comp == 0) {
                         const T tx = dxu * fn, ty = dyu * fn, k2 = T(0.5) * (dxu * dxu + dyu * dyu);
                         hs[0].add(k2 * tx); hs[1].add(k2 * ty);
@@ -1727,7 +1727,7 @@ __global__ void __launch_bounds__(256) k_special(CvArgs c, const T *fin, T *fout
             const CvMember &M = I.mem[gt];
             write_split_partials<T>(pout, sp, nc, (long)M.j * g.nx + M.i, M.keep != 0, tv[0], tv[1], tv[2], tv[3]);
         }
-        if (c.hout) {
+        if (SHAK && c.hout) {
             T hv[5];
             group_acc(hs, hv, red, kw);
             if (on && gt < nm) {
@@ -2359,7 +2359,6 @@ cudaError_t step2d_t(dvm_ctx *c, int phase, double *xbuf)
     const bool shak = c->model == DVM_SHAKHOV && !imex;
     const bool hkeep = shak && c->prec == DVM_FP32;      // raw heat-flux moments kept (FP32)
     const bool hraw = hkeep && c->hvalid;
-    cv.shak = shak ? 1 : 0;
     cv.hout = hkeep ? c->hpart[1 - c->cur] : nullptr;
     cv.pr1 = 1.0 - c->Pr;
     cv.err = c->d_err;
@@ -2376,8 +2375,7 @@ cudaError_t step2d_t(dvm_ctx *c, int phase, double *xbuf)
             k_fold_partials<T><<<nblk(nc, 256), 256, 0, c->stream>>>(pin, c->S, nc, xbuf);
             c->launches += 1;
             if (body) {
-                k_wall<T><<<cvgrid, 256, 0, c->stream>>>(cv, bp, c->d_body, fin, c->wphi, c->wcontrib, c->ticket,
-                                                          c->d_hist, moving ? 1 : 0, 1, xw);
+                k_wall<T><<<cvgrid, 256, 0, c->stream>>>(cv, bp, c->d_body, fin, c->wphi, c->wcontrib, 1, xw);
                 c->launches += 1;
             }
             return cudaGetLastError();
@@ -2401,8 +2399,8 @@ cudaError_t step2d_t(dvm_ctx *c, int phase, double *xbuf)
         // the bulk kernel only the plain cells
         if ((e = cudaEventRecord(c->ev_wfork, c->stream)) != cudaSuccess) return e;
         if ((e = cudaStreamWaitEvent(c->wstream, c->ev_wfork, 0)) != cudaSuccess) return e;
-        k_wall<T><<<cvgrid, 256, 0, c->wstream>>>(cv, bp, c->d_body, fin, c->wphi, c->wcontrib, c->ticket,
-                                                   c->d_hist, moving ? 1 : 0, phase == 2 ? 2 : 0, xw);
+        k_wall<T><<<cvgrid, 256, 0, c->wstream>>>(cv, bp, c->d_body, fin, c->wphi, c->wcontrib,
+                                                   phase == 2 ? 2 : 0, xw);
         c->launches += 1;
     }
     BulkArgs<T> a{};
@@ -2426,7 +2424,9 @@ cudaError_t step2d_t(dvm_ctx *c, int phase, double *xbuf)
     if ((e = timing_mark(c, 1)) != cudaSuccess) return e;
     c->launches += 1;
     if (body) {
-        k_special<T><<<cvgrid, 256, 0, c->wstream>>>(cv, fin, fout, pin, pout, c->wphi);
+        const auto special = shak ? k_special<T, true> : k_special<T, false>;
+        special<<<cvgrid + 1, 256, 0, c->wstream>>>(cv, bp, c->d_body, fin, fout, pin, pout, c->wphi, c->wcontrib,
+                                                    c->d_hist, moving ? 1 : 0);
         if ((e = cudaEventRecord(c->ev_wjoin, c->wstream)) != cudaSuccess) return e;
         // the step ends when both streams are done
         if ((e = cudaStreamWaitEvent(c->stream, c->ev_wjoin, 0)) != cudaSuccess) return e;
