@@ -540,14 +540,21 @@ static_assert(kAdjLamBytes % 128 == 0 && kAdjStageBytes % 128 == 0,
 template <typename T, bool MUSCL>
 __global__ void __launch_bounds__(32 * kRows, 2) k_adj_gather_fast(AdjArgs a, const __grid_constant__ CUtensorMap lmap,
                                                                    const __grid_constant__ CUtensorMap bmap,
-                                                                   const int8_t *gsign, const T *aux,
+                                                                   const float4 *ptab, const T *aux,
                                                                    const uint8_t *fast, T *lam_out)
 {
     using V = typename Vec<T>::type;
     constexpr int W = Vec<T>::W;
-    constexpr uint32_t kBytes = MUSCL ? kAdjLamBytes + kTileY * kTileX * 4 : kAdjLamBytes;
+    // a group's W coefficients (64 bytes in both precisions) and its signs
+    // arrive with its tile: read through L1 they cost an L2 latency a group
+    // (261 -> 248 us a launch at 256^2 x 32^2)
+    constexpr uint32_t kCoef = W * sizeof(VCoef<T>);
+    constexpr uint32_t kBytes = (MUSCL ? kAdjLamBytes + kTileY * kTileX * 4 : kAdjLamBytes) + kCoef + 16;
+    static_assert(kCoef + 16 <= kTabBytes, "a stage's table slot");
     extern __shared__ __align__(128) unsigned char smem[];
-    uint64_t *full = reinterpret_cast<uint64_t *>(smem + kAdjStages * kAdjStageBytes);
+    // the group's velocity coefficients and signs, [kAdjStages][kTabBytes]
+    unsigned char *const tab = smem + kAdjStages * kAdjStageBytes;
+    uint64_t *full = reinterpret_cast<uint64_t *>(tab + kAdjStages * kTabBytes);
     uint64_t *empty = full + kAdjStages;
     const Grid2D &g = a.g;
     const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * 32 + tx;
@@ -559,11 +566,14 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_adj_gather_fast(AdjArgs a, co
     const int gps = (g.ngrp + gridDim.z - 1) / gridDim.z;
     const int g0 = blockIdx.z * gps, g1 = min(g0 + gps, g.ngrp);
     const int ngr = max(g1 - g0, 0);
+    const VCoef<T> *vt = reinterpret_cast<const VCoef<T> *>(a.vt);
     const auto issue = [&](int st, int q) {
         unsigned char *dst = smem + (long)st * kAdjStageBytes;
         mbar_expect_tx(&full[st], kBytes);
         tma_load_3d(dst, &lmap, &full[st], i0 * W, j0, q * 2);
         if (MUSCL) tma_load_3d(dst + kAdjLamBytes, &bmap, &full[st], i0, j0, q);
+        bulk_load(tab + st * kTabBytes, vt + (long)q * W, kCoef, &full[st]);
+        bulk_load(tab + st * kTabBytes + kCoef, ptab + (long)q * kTabRows + 7, 16, &full[st]);
     };
     if (tid == 0) {
         for (int st = 0; st < kAdjStages; ++st) {
@@ -573,7 +583,6 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_adj_gather_fast(AdjArgs a, co
         mbar_fence_init();
         for (int st = 0; st < kAdjStages - 1 && st < ngr; ++st) issue(st, g0 + st);
     }
-    const VCoef<T> *vt = reinterpret_cast<const VCoef<T> *>(a.vt);
     T omr = 0, S0 = 0, S1 = 0, S2 = 0, S3 = 0;
     if (isfast) {
         const T *o = aux + 5 * k;
@@ -600,11 +609,12 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_adj_gather_fast(AdjArgs a, co
             T vx[W], vy[W], nux[W], nuy[W], rel0[W];
 #pragma unroll
             for (int e = 0; e < W; ++e) {
-                const VCoef<T> vc = ld_coef(vt + p + e);
+                const VCoef<T> vc = reinterpret_cast<const VCoef<T> *>(tab + st * kTabBytes)[e];
                 vx[e] = vc.vx; vy[e] = vc.vy; nux[e] = vc.nux; nuy[e] = vc.nuy;
                 rel0[e] = dv * (S0 + S1 * vx[e] + S2 * vy[e] + S3 * T(0.5) * (vx[e] * vx[e] + vy[e] * vy[e]));
             }
-            const int sgx = gsign[2 * q], sgy = gsign[2 * q + 1];
+            const int2 sg = *reinterpret_cast<const int2 *>(tab + st * kTabBytes + kCoef);
+            const int sgx = sg.x, sgy = sg.y;
             uint32_t bo = 0, bxm = 0, bxp = 0, bym = 0, byp = 0;
             if (MUSCL) {
                 bo = bt[c0]; bxm = bt[c0 - 1]; bxp = bt[c0 + 1]; bym = bt[c0 - kTileX]; byp = bt[c0 + kTileX];
@@ -1442,7 +1452,7 @@ template <typename T, bool MUSCL>
 cudaError_t launch_gather_fast(dvm_ctx *c, const AdjArgs &a, const AdjWork &w, const CUtensorMap &lmap,
                                const CUtensorMap *bmap, T *lam_out)
 {
-    const size_t smem = (size_t)kAdjStages * kAdjStageBytes + 2 * kAdjStages * sizeof(uint64_t);
+    const size_t smem = (size_t)kAdjStages * (kAdjStageBytes + kTabBytes) + 2 * kAdjStages * sizeof(uint64_t);
     static bool attr = false;
     if (!attr) {
         cudaError_t e = cudaFuncSetAttribute(k_adj_gather_fast<T, MUSCL>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1451,7 +1461,7 @@ cudaError_t launch_gather_fast(dvm_ctx *c, const AdjArgs &a, const AdjWork &w, c
         attr = true;
     }
     const dim3 grid(nba(c->nx, 32), nba(c->ny, kRows), w.Zf), block(32, kRows);
-    k_adj_gather_fast<T, MUSCL><<<grid, block, smem, c->stream>>>(a, lmap, bmap ? *bmap : lmap, c->gsign,
+    k_adj_gather_fast<T, MUSCL><<<grid, block, smem, c->stream>>>(a, lmap, bmap ? *bmap : lmap, (const float4 *)c->ptab,
                                                                    (const T *)w.aux, w.fast, lam_out);
     return cudaGetLastError();
 }
