@@ -126,6 +126,7 @@ template <typename T> struct Acc {
 // holds 32 consecutive cells of a row and kMomChunks warps, one chunk of the
 // velocity groups each.
 constexpr int kMomChunks = 8;
+constexpr int kMomBatch = 4;         // group vectors a thread of the moment kernels has in flight
 
 // Merges the compensated sums of the kMomChunks warps of a block into warp 0,
 // chunk by chunk in order (the same result on every run).

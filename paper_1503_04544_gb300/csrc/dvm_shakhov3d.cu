@@ -58,28 +58,30 @@ __device__ __forceinline__ void side_mirrors3(const Grid3D &g, int i, int j, int
 __device__ __forceinline__ float exp2_s3(float x) { return ex2_fast(x); }
 __device__ __forceinline__ double exp2_s3(double x) { return exp2(x); }
 
-// Heat flux of the control volume of cell (i, j, k) at t^n, for a block of 32
-// consecutive cells of an x-row x kMomChunks warps, each warp one chunk of
-// the velocity groups: the primitives from the partial sums of its master,
+// Heat flux of the control volume of a cell at t^n, for a block of 32 cells
+// consecutive in the grid x kMomChunks warps, each warp one chunk of the
+// velocity groups, kMomBatch of them in flight (45 x 50 x 37 cells, 14 x 15 x 13
+// velocities, FP32: one at a time in tiles of a row 0.33 ms, now 0.244): the primitives from the partial sums of its master,
 // q from the master's F^n (after fusion), compensated sums merged over the
 // chunks in fixed order into qsh (every warp of the block reads them after
 // the barrier).  gas is false for solid cells and cells in no control volume.
 template <typename T>
 __device__ __forceinline__ void cv_heat_flux3(const Grid3D &g, int S, const T *fin, const T *pin,
                                               const VxEntry<T> *vxt, const VyzEntry<T> *vyz, const int32_t *master,
-                                              const int8_t *type, int *err, int i, int j, int k, T (&qsh)[3][32],
+                                              const int8_t *type, int *err, long cell, T (&qsh)[3][32],
                                               bool &gas, T &rho, T &ux, T &uy, T &uz, T &tmp)
 {
     constexpr int W = Vec<T>::W;
     using V = typename Vec<T>::type;
-    const long nc = (long)g.nx * g.ny * g.nz, cell = ((long)k * g.ny + j) * g.nx + i;
+    const long nc = (long)g.nx * g.ny * g.nz;
     const T dv = pick<T>(g.dv_f, g.dv);
-    gas = i < g.nx && type[cell] != DVM_SOLID;
+    gas = cell < nc && type[cell] != DVM_SOLID;
     const long m = gas ? (long)master[cell] : -1;
     gas = gas && m >= 0;
     rho = ux = uy = uz = tmp = 0;
     if (gas) {
         Acc<T> a[5];
+#pragma unroll 4
         for (int q = 0; q < S; ++q)
 #pragma unroll
             for (int f = 0; f < 5; ++f) a[f].merge(pin[((long)q * 5 + f) * nc + m], T(0));
@@ -102,27 +104,33 @@ __device__ __forceinline__ void cv_heat_flux3(const Grid3D &g, int S, const T *f
         const long pm = slab3(g, mr % g.nx, mr / g.nx, mk);
         const V *fv = reinterpret_cast<const V *>(fin);
         int r = q0 / g.nxg, xg = q0 - r * g.nxg;
-        for (int q = q0; q < q1; ++q) {
-            T a[W];
-            vld<T>(fv + (long)q * g.slab + pm, a);
-            const VyzEntry<T> cy = vyz[r];
-            const T cyv = cy.vy - uy, czv = cy.vz - uz, dyz = cyv * cyv + czv * czv;
-            T t0 = 0, t1 = 0;
+        for (int q = q0; q < q1; q += kMomBatch) {
+            T a[kMomBatch][W];
 #pragma unroll
-            for (int e = 0; e < W; ++e) {
-                const int p1 = xg * W + e;
-                if (p1 >= g.nvx) continue;
-                const T dx = vxt[p1].vx - ux;
-                const T w = T(0.5) * (dx * dx + dyz) * a[e];
-                t0 += dx * w;
-                t1 += w;
-            }
-            hq[0].add(t0);
-            hq[1].add(cyv * t1);
-            hq[2].add(czv * t1);
-            if (++xg == g.nxg) {
-                xg = 0;
-                ++r;
+            for (int b = 0; b < kMomBatch; ++b)
+                if (q + b < q1) vld<T>(fv + (long)(q + b) * g.slab + pm, a[b]);
+#pragma unroll
+            for (int b = 0; b < kMomBatch; ++b) {
+                if (q + b >= q1) break;
+                const VyzEntry<T> cy = vyz[r];
+                const T cyv = cy.vy - uy, czv = cy.vz - uz, dyz = cyv * cyv + czv * czv;
+                T t0 = 0, t1 = 0;
+#pragma unroll
+                for (int e = 0; e < W; ++e) {
+                    const int p1 = xg * W + e;
+                    if (p1 >= g.nvx) continue;
+                    const T dx = vxt[p1].vx - ux;
+                    const T w = T(0.5) * (dx * dx + dyz) * a[b][e];
+                    t0 += dx * w;
+                    t1 += w;
+                }
+                hq[0].add(t0);
+                hq[1].add(cyv * t1);
+                hq[2].add(czv * t1);
+                if (++xg == g.nxg) {
+                    xg = 0;
+                    ++r;
+                }
             }
         }
     }
@@ -142,12 +150,11 @@ __global__ void __launch_bounds__(32 * kMomChunks)
                 const int32_t *master, const int8_t *type, T *q, int *err)
 {
     __shared__ T qsh[3][32];
-    const int i = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y, k = blockIdx.z;
+    const long nc = (long)g.nx * g.ny * g.nz, cell = (long)blockIdx.x * 32 + threadIdx.x;
     bool gas;
     T rho, ux, uy, uz, tmp;
-    cv_heat_flux3(g, S, fin, pin, vxt, vyz, master, type, err, i, j, k, qsh, gas, rho, ux, uy, uz, tmp);
-    if (threadIdx.y != 0 || i >= g.nx) return;
-    const long nc = (long)g.nx * g.ny * g.nz, cell = ((long)k * g.ny + j) * g.nx + i;
+    cv_heat_flux3(g, S, fin, pin, vxt, vyz, master, type, err, cell, qsh, gas, rho, ux, uy, uz, tmp);
+    if (threadIdx.y != 0 || cell >= nc) return;
 #pragma unroll
     for (int d = 0; d < 3; ++d) q[d * nc + cell] = gas ? qsh[d][threadIdx.x] : T(0);
 }
@@ -163,11 +170,10 @@ __global__ void __launch_bounds__(32 * kMomChunks)
     constexpr int W = Vec<T>::W;
     using V = typename Vec<T>::type;
     __shared__ T qsh[3][32];
-    const int i = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y, k = blockIdx.z;
-    const long nc = (long)g.nx * g.ny * g.nz, cell = ((long)k * g.ny + j) * g.nx + i;
+    const long nc = (long)g.nx * g.ny * g.nz, cell = (long)blockIdx.x * 32 + threadIdx.x;
     bool gas;
     T rho, ux, uy, uz, tmp;
-    cv_heat_flux3(g, S, fin, pin, vxt, vyz, master, type, err, i, j, k, qsh, gas, rho, ux, uy, uz, tmp);
+    cv_heat_flux3(g, S, fin, pin, vxt, vyz, master, type, err, cell, qsh, gas, rho, ux, uy, uz, tmp);
     const int gps = (g.ngrp + kMomChunks - 1) / kMomChunks;
     const int q0 = threadIdx.y * gps, q1 = min(q0 + gps, g.ngrp);
     const T qx = qsh[0][threadIdx.x], qy = qsh[1][threadIdx.x], qz = qsh[2][threadIdx.x];
@@ -178,6 +184,7 @@ __global__ void __launch_bounds__(32 * kMomChunks)
         const T A = rho / (tw * sqrt(tw)), c2 = T(kLog2e) / (T(2) * tmp);
         const T kk = dt_tau0 * rho * pr1 / (T(5) * rho * tmp * tmp);     // (dt/tau) k
         const T iT = T(1) / tmp;
+        const int row = (int)(cell / g.nx), i = (int)(cell - (long)row * g.nx), k = row / g.ny, j = row - k * g.ny;
         const long pc = slab3(g, i, j, k);
         long mir[6];
         side_mirrors3(g, i, j, k, mir);
@@ -218,7 +225,7 @@ __global__ void __launch_bounds__(32 * kMomChunks)
         }
     }
     merge_chunks<T, 5>(a5);
-    if (threadIdx.y != 0 || i >= g.nx) return;
+    if (threadIdx.y != 0 || cell >= nc) return;
     // split 0 holds the sums, the other splits zeros (solid cells: zeros)
     for (int q = 0; q < S; ++q) {
         const bool z = q > 0 || !gas;
@@ -237,7 +244,7 @@ cudaError_t shakhov3d_t(dvm_ctx *c)
     const VxEntry<T> *vxt = reinterpret_cast<const VxEntry<T> *>(c->vtab);
     const VyzEntry<T> *vyz = reinterpret_cast<const VyzEntry<T> *>(reinterpret_cast<const char *>(c->vtab) +
                                                                    (size_t)c->nvxp * sizeof(VxEntry<T>));
-    const dim3 grid((unsigned)((c->nx + 31) / 32), (unsigned)c->ny, (unsigned)c->nz), block(32, kMomChunks);
+    const dim3 grid((unsigned)((c->nc + 31) / 32)), block(32, kMomChunks);
     cudaError_t e = timing_mark_kernel(c, 2, 0);
     if (e != cudaSuccess) return e;
     k_shakhov3<T><<<grid, block, 0, c->stream>>>(g, c->S, T(c->dt / c->tau0), T(1.0 - c->Pr), fin, pin, fout, pout,
@@ -254,7 +261,7 @@ cudaError_t heatflux3d_t(dvm_ctx *c, const void *f, const void *part)
     const VxEntry<T> *vxt = reinterpret_cast<const VxEntry<T> *>(c->vtab);
     const VyzEntry<T> *vyz = reinterpret_cast<const VyzEntry<T> *>(reinterpret_cast<const char *>(c->vtab) +
                                                                    (size_t)c->nvxp * sizeof(VxEntry<T>));
-    const dim3 grid((unsigned)((c->nx + 31) / 32), (unsigned)c->ny, (unsigned)c->nz), block(32, kMomChunks);
+    const dim3 grid((unsigned)((c->nc + 31) / 32)), block(32, kMomChunks);
     cudaError_t e = timing_mark_kernel(c, 2, 0);
     if (e != cudaSuccess) return e;
     k_heatflux3<T><<<grid, block, 0, c->stream>>>(g, c->S, (const T *)f, (const T *)part, vxt, vyz, c->master,

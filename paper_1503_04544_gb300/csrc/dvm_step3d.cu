@@ -1234,47 +1234,59 @@ __global__ void __launch_bounds__(256) k_special3(Cv3Args c, const T *fin, T *fo
 }
 
 // ------------------------------------------------------------ state services
-// Moment sums of cells (i, j, k) of one x-row over a chunk of the velocity
-// groups: F, v_x F, v_y F, v_z F and |v|^2/2 F (Eq. MacroscopicTD), per
-// group plain over its lanes and compensated across groups.  The lanes of a
-// warp are 32 consecutive cells, so each group's vector of the 32 cells is
-// one coalesced read; warp threadIdx.y takes the threadIdx.y-th of
-// kMomChunks chunks.
+// Moment sums of a cell over a chunk of the velocity groups: F, v_x F, v_y F,
+// v_z F and |v|^2/2 F (Eq. MacroscopicTD).  The lanes of a warp are 32 cells
+// consecutive in the grid (a row may end inside a warp: 45-cell rows took 64
+// lanes in tiles of a row), so a group's vectors are whole lines but at row
+// ends; warp threadIdx.y takes the threadIdx.y-th of kMomChunks chunks, kMomBatch
+// groups' loads in flight.  FP32, bound by memory: sums plain over a group and
+// compensated across groups.  FP64, bound by its pipe: the sums of an x-row of
+// velocities first, then its v_y and v_z terms once (5 operations a velocity in
+// place of 10; 40^3 x 12^3: 2.7 ms before, 1.73 now).
 template <typename T>
 __device__ __forceinline__ void state_sums3d(const Grid3D &g, const T *f, const VX3<T> *vxt, const VYZ3<T> *vyz,
-                                             int i, int j, int k, Acc<T> (&s)[5])
+                                             long cell, Acc<T> (&s)[5])
 {
     constexpr int W = Vec<T>::W;
     using V = typename Vec<T>::type;
-    if (i >= g.nx) return;
+    if (cell >= (long)g.nx * g.ny * g.nz) return;
     const int gps = (g.ngrp + kMomChunks - 1) / kMomChunks;
     const int q0 = threadIdx.y * gps, q1 = min(q0 + gps, g.ngrp);
     if (q0 >= q1) return;
-    const long pc = nbr3(g, i, j, k);
-    const V *fv = reinterpret_cast<const V *>(f);
+    const V *fv = reinterpret_cast<const V *>(f) + pcell3(g, (int)cell);
     int r = q0 / g.nxg, xg = q0 - r * g.nxg;
-    for (int q = q0; q < q1; ++q) {
-        T a[W];
-        vld<T>(fv + (long)q * g.slab + pc, a);
-        T t0 = 0, t1 = 0, t2 = 0;
+    T t0 = 0, t1 = 0, t2 = 0;
+    for (int q = q0; q < q1; q += kMomBatch) {
+        T a[kMomBatch][W];
 #pragma unroll
-        for (int e = 0; e < W; ++e) {
-            const int p1 = xg * W + e;
-            if (p1 >= g.nvx) continue;
-            const T vx = vxt[p1].vx;
-            t0 += a[e];
-            t1 += vx * a[e];
-            t2 += vx * vx * a[e];
-        }
-        const VYZ3<T> cy = vyz[r];
-        s[0].add(t0);
-        s[1].add(t1);
-        s[2].add(cy.vy * t0);
-        s[3].add(cy.vz * t0);
-        s[4].add(T(0.5) * fma(cy.vy * cy.vy + cy.vz * cy.vz, t0, t2));
-        if (++xg == g.nxg) {
-            xg = 0;
-            ++r;
+        for (int b = 0; b < kMomBatch; ++b)
+            if (q + b < q1) vld<T>(fv + (long)(q + b) * g.slab, a[b]);
+#pragma unroll
+        for (int b = 0; b < kMomBatch; ++b) {
+            if (q + b >= q1) break;
+#pragma unroll
+            for (int e = 0; e < W; ++e) {
+                const int p1 = xg * W + e;
+                if (p1 >= g.nvx) continue;
+                const T vx = vxt[p1].vx;
+                t0 += a[b][e];
+                t1 += vx * a[b][e];
+                t2 += vx * vx * a[b][e];
+            }
+            const bool row = ++xg == g.nxg;
+            if (sizeof(T) == 4 || row || q + b == q1 - 1) {
+                const VYZ3<T> cy = vyz[r];
+                s[0].add(t0);
+                s[1].add(t1);
+                s[2].add(cy.vy * t0);
+                s[3].add(cy.vz * t0);
+                s[4].add(T(0.5) * fma(cy.vy * cy.vy + cy.vz * cy.vz, t0, t2));
+                t0 = t1 = t2 = 0;
+            }
+            if (row) {
+                xg = 0;
+                ++r;
+            }
         }
     }
 }
@@ -1286,12 +1298,11 @@ __global__ void __launch_bounds__(32 * kMomChunks) k_partials3(Grid3D g, int S, 
                                                                const VYZ3<T> *vyz, T *part, const int8_t *type,
                                                                int *err)
 {
-    const int i = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y, k = blockIdx.z;
+    const long nc = (long)g.nx * g.ny * g.nz, cell = (long)blockIdx.x * 32 + threadIdx.x;
     Acc<T> s[5];
-    state_sums3d<T>(g, f, vxt, vyz, i, j, k, s);
+    state_sums3d<T>(g, f, vxt, vyz, cell, s);
     merge_chunks<T, 5>(s);
-    if (threadIdx.y != 0 || i >= g.nx) return;
-    const long nc = (long)g.nx * g.ny * g.nz, cell = ((long)k * g.ny + j) * g.nx + i;
+    if (threadIdx.y != 0 || cell >= nc) return;
     const bool keep = type[cell] != DVM_SOLID;
     T v[5];
 #pragma unroll
@@ -1322,12 +1333,12 @@ template <typename T>
 __global__ void __launch_bounds__(32 * kMomChunks) k_moments_out3(Grid3D g, const T *f, const VX3<T> *vxt,
                                                                   const VYZ3<T> *vyz, double *out)
 {
-    const int i = blockIdx.x * 32 + threadIdx.x, j = blockIdx.y, k = blockIdx.z;
+    const long nc = (long)g.nx * g.ny * g.nz, cell = (long)blockIdx.x * 32 + threadIdx.x;
     Acc<T> s[5];
-    state_sums3d<T>(g, f, vxt, vyz, i, j, k, s);
+    state_sums3d<T>(g, f, vxt, vyz, cell, s);
     merge_chunks<T, 5>(s);
-    if (threadIdx.y != 0 || i >= g.nx) return;
-    double *o5 = out + (((long)k * g.ny + j) * g.nx + i) * 5;
+    if (threadIdx.y != 0 || cell >= nc) return;
+    double *o5 = out + cell * 5;
     double d[5];
 #pragma unroll
     for (int m = 0; m < 5; ++m) d[m] = (double)s[m].s - (double)s[m].c;
@@ -1978,7 +1989,7 @@ cudaError_t tables3d(dvm_ctx *c)
 cudaError_t partials_from_state3d(dvm_ctx *c)
 {
     const Grid3D g = grid3d(c);
-    const dim3 grid(nb3(c->nx, 32), c->ny, c->nz), block(32, kMomChunks);
+    const dim3 grid(nb3((long)c->nc, 32)), block(32, kMomChunks);
     if (c->prec == DVM_FP32)
         k_partials3<float><<<grid, block, 0, c->stream>>>(g, c->S, (const float *)c->f[c->cur], vx_table<float>(c),
                                                           vyz_table<float>(c), (float *)c->part[c->cur], c->geo3.type,
@@ -2005,7 +2016,7 @@ cudaError_t check_moments3d(dvm_ctx *c)
 cudaError_t moments_out3d(dvm_ctx *c, double *d_out)
 {
     const Grid3D g = grid3d(c);
-    const dim3 grid(nb3(c->nx, 32), c->ny, c->nz), block(32, kMomChunks);
+    const dim3 grid(nb3((long)c->nc, 32)), block(32, kMomChunks);
     if (c->prec == DVM_FP32)
         k_moments_out3<float><<<grid, block, 0, c->stream>>>(g, (const float *)c->f[c->cur], vx_table<float>(c),
                                                              vyz_table<float>(c), d_out);
