@@ -61,7 +61,8 @@ __device__ __forceinline__ double exp2_s3(double x) { return exp2(x); }
 // Heat flux of the control volume of a cell at t^n, for a block of 32 cells
 // consecutive in the grid x kMomChunks warps, each warp one chunk of the
 // velocity groups, kMomBatch of them in flight (45 x 50 x 37 cells, 14 x 15 x 13
-// velocities, FP32: one at a time in tiles of a row 0.33 ms, now 0.244): the primitives from the partial sums of its master,
+// velocities, FP32: one at a time in tiles of a row 0.33 ms, now 0.244): the
+// primitives from the partial sums of its master,
 // q from the master's F^n (after fusion), compensated sums merged over the
 // chunks in fixed order into qsh (every warp of the block reads them after
 // the barrier).  gas is false for solid cells and cells in no control volume.

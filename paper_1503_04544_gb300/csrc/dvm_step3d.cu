@@ -998,8 +998,9 @@ __global__ void __launch_bounds__(256) k_fusion3(Cv3Args c, T *f, T *part)
 // body (3D forms of Eqs. BoundaryDDv, StressTensorDD, eq-force), torque about
 // the z axis through the centre (Eq. eq-torque), u_w = u_c + omega e_z x
 // (r - c) (Eq. uwDD).  One block per wall cell: products and compensated sums
-// in the state precision over all velocities, phi and the stress in FP64 by
-// thread 0.  The last block sums the cells in list order into the body
+// in the state precision over all velocities, a thread a velocity group (one
+// vector, one pair of divisions for its W velocities) and the 14 sums merged
+// together (64^3 x 20^3: 0.175 -> 0.135 ms a launch), phi and the stress in FP64 by thread 0.  The last block sums the cells in list order into the body
 // record and the history.  (phi, u_w, T_w) of each wall cell are left for
 // the control-volume kernel.
 template <typename T>
@@ -1009,10 +1010,12 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_wall3(Cv3Args c, BodyParams b, BodyDev *body, const T *f, double *wdat,
                                                double *wcontrib, int *ticket, double *hist, int mode, double *xw)
 {
+    constexpr int W = Vec<T>::W;
+    using V = typename Vec<T>::type;
     __shared__ double red[8 * 8];
     __shared__ T ex[kMaxAxisNv], ey[kMaxAxisNv], ez[kMaxAxisNv];
     __shared__ T wsc[8];
-    __shared__ T wred[8 * 2];
+    __shared__ T wred[8 * 3 * 14];
     __shared__ bool last;
     const Grid3D &g = c.g;
     const VX3<T> *vxt = reinterpret_cast<const VX3<T> *>(c.vxt);
@@ -1053,30 +1056,39 @@ __global__ void __launch_bounds__(256) k_wall3(Cv3Args c, BodyParams b, BodyDev 
             }
         }
         __syncthreads();
-        const int pc = pcell3(g, q);
+        const V *fv = reinterpret_cast<const V *>(f) + pcell3(g, q);
         // a[0] = sum_{c>0} c F, a[1] = sum_{c<0} c M, a[2..7] = sum_{c<0} (v-u_w)(v-u_w) M,
         // a[8..13] = sum_{c>0} (v-u_w)(v-u_w) F   (xx, xy, xz, yy, yz, zz)
         Acc<T> a[14];
-        for (int p = tid; p < g.nv; p += blockDim.x) {
-            const int p1 = p % g.nvx, r = p / g.nvx;
+        for (int grp = tid; grp < g.ngrp; grp += blockDim.x) {
+            const int r = grp / g.nxg, x0 = (grp - r * g.nxg) * W;
             const int p3 = r / g.nvy, p2 = r - p3 * g.nvy;
-            const T vx = vxt[p1].vx, vy = vyz[r].vy, vz = vyz[r].vz;
-            const T ax = vx - ux, ay = vy - uy, az = vz - uz;
-            const T cp = ax * nx + ay * ny + az * nz;
-            if (cp > T(0)) {
-                const T fv = f[pidx3(g, r * g.nvxp + p1, pc)];
-                a[0].add(cp * fv);
-                a[8].add(ax * ax * fv); a[9].add(ax * ay * fv); a[10].add(ax * az * fv);
-                a[11].add(ay * ay * fv); a[12].add(ay * az * fv); a[13].add(az * az * fv);
-            } else if (cp < T(0)) {
-                const T m1 = cm * ex[p1] * ey[p2] * ez[p3];
-                a[1].add(cp * m1);
-                a[2].add(ax * ax * m1); a[3].add(ax * ay * m1); a[4].add(ax * az * m1);
-                a[5].add(ay * ay * m1); a[6].add(ay * az * m1); a[7].add(az * az * m1);
+            const T ay = vyz[r].vy - uy, az = vyz[r].vz - uz;
+            T F[W];
+            vld<T>(fv + (long)grp * g.slab, F);
+#pragma unroll
+            for (int e = 0; e < W; ++e) {
+                const int p1 = x0 + e;
+                if (p1 >= g.nvx) continue;
+                const T ax = vxt[p1].vx - ux;
+                const T cp = ax * nx + ay * ny + az * nz;
+                if (cp > T(0)) {
+                    const T fv1 = F[e];
+                    a[0].add(cp * fv1);
+                    a[8].add(ax * ax * fv1); a[9].add(ax * ay * fv1); a[10].add(ax * az * fv1);
+                    a[11].add(ay * ay * fv1); a[12].add(ay * az * fv1); a[13].add(az * az * fv1);
+                } else if (cp < T(0)) {
+                    const T m1 = cm * ex[p1] * ey[p2] * ez[p3];
+                    a[1].add(cp * m1);
+                    a[2].add(ax * ax * m1); a[3].add(ax * ay * m1); a[4].add(ax * az * m1);
+                    a[5].add(ay * ay * m1); a[6].add(ay * az * m1); a[7].add(az * az * m1);
+                }
             }
         }
+        T rv[14];
+        group_acc(a, rv, wred, blockDim.x >> 5);
 #pragma unroll
-        for (int t = 0; t < 14; ++t) rr[t] = (double)block_acc(a[t], wred);
+        for (int t = 0; t < 14; ++t) rr[t] = (double)rv[t];
         if (mode == 1) {
             if (tid == 0)
 #pragma unroll
@@ -1126,12 +1138,30 @@ __global__ void __launch_bounds__(256) k_wall3(Cv3Args c, BodyParams b, BodyDev 
 // six faces of every member and across its wall face with the diffuse state
 // F_w = phi M[1, u_w, T_w] on incoming velocities, relaxation, distribution
 // to the members and the moment sums of the velocity split.  One work item is
-// one control volume and one split.
-template <typename T>
-__global__ void __launch_bounds__(256) k_special3(Cv3Args c, const T *fin, T *fout, const T *pin, T *pout,
-                                                  const double *wdat)
+// one control volume and one split, one thread a velocity group: the 13 values
+// of the stencil are vectors, so the addresses and the member's record are
+// read once for its W velocities, and the five sums are merged together.  It is
+// bound by latency (32% of the SM's issue rate, a fifth of its warps).  One
+// thread a velocity before: 64^3 x 20^3 FP32 0.65 -> 0.50 ms a launch, 45 x 50 x
+// 37 cells, 14 x 15 x 13 velocities 0.24 -> 0.11 ms, 40^3 x 12^3 FP64 0.59 ->
+// 0.44 ms (more registers: one block of 256 per SM; with two it spills).
+constexpr int kSpec3Threads = 256;
+
+// Threads of a block for splits of gps groups: as few rounds as 256 threads
+// need, of equal length (a split of 286 groups: two rounds of 160 threads).
+inline int spec3_threads(int gps)
 {
-    __shared__ T red[8 * 2];
+    const int rounds = (gps + kSpec3Threads - 1) / kSpec3Threads;
+    return ((gps + rounds - 1) / rounds + 31) / 32 * 32;
+}
+
+template <typename T>
+__global__ void __launch_bounds__(kSpec3Threads, sizeof(T) == 4 ? 2 : 1)
+    k_special3(Cv3Args c, const T *fin, T *fout, const T *pin, T *pout, const double *wdat)
+{
+    constexpr int W = Vec<T>::W;
+    using V = typename Vec<T>::type;
+    __shared__ T red[8 * 3 * 5];
     __shared__ __align__(16) CvInfo3 I;
     const Grid3D &g = c.g;
     const CvInfo3 *info = reinterpret_cast<const CvInfo3 *>(c.cvinfo);
@@ -1145,7 +1175,7 @@ __global__ void __launch_bounds__(256) k_special3(Cv3Args c, const T *fin, T *fo
         load_info3(info + idx, &I);
         if (!I.ok) { __syncthreads(); continue; }
         const int nm = I.nm;
-        const int v0 = sp * c.gps * g.W, v1 = min(g.nvp, v0 + c.gps * g.W);
+        const int g0 = sp * c.gps, g1 = min(g.ngrp, g0 + c.gps);
         const int m = c.spec_list[idx];
         T s[5];
         gather_partials3(pin, c.Sin, nc, m, s);
@@ -1169,65 +1199,84 @@ __global__ void __launch_bounds__(256) k_special3(Cv3Args c, const T *fin, T *fo
             kqz = kk * qh[2 * nc + m];
         }
         Acc<T> acc[5];
-        for (int p = v0 + threadIdx.x; p < v1; p += blockDim.x) {
-            T vx, vy, vz, nux, nuy, nuz;
-            vel3(g, vxt, vyz, p, vx, vy, vz, nux, nuy, nuz);
-            const int grp = p / g.W, e = p - grp * g.W;
-            const T *fg = fin + (long)grp * g.slab * g.W + e;     // element of slab index s: fg[s * W]
-            const int Wd = g.W;
-            T R = 0;
+        for (int grp = g0 + threadIdx.x; grp < g1; grp += blockDim.x) {
+            const int yz = grp / g.nxg, x0 = (grp - yz * g.nxg) * W;
+            const VYZ3<T> cy = vyz[yz];
+            T vx[W], nux[W];
+#pragma unroll
+            for (int e = 0; e < W; ++e) {
+                const VX3<T> cx = vxt[x0 + e];
+                vx[e] = cx.vx;
+                nux[e] = cx.nux;
+            }
+            const V *fg = reinterpret_cast<const V *>(fin) + (long)grp * g.slab;
+            T R[W] = {};
             for (int t = 0; t < nm; ++t) {
                 const CvMember3 &M = I.mem[t];
                 if (!M.live) continue;
-                const int pc = M.pc;
-                const T fc = fg[(long)pc * Wd];
-                T Fw = 0;
+                const V *fp = fg + M.pc;
+                T fc[W];
+                vld<T>(fp, fc);
+                T xm1[W], xp1[W], ym1[W], yp1[W], zm1[W], zp1[W];
+                vld<T>(fp - 1, xm1); vld<T>(fp + 1, xp1);
+                vld<T>(fp - sy, ym1); vld<T>(fp + sy, yp1);
+                vld<T>(fp - sz, zm1); vld<T>(fp + sz, zp1);
+                T xm2[W] = {}, xp2[W] = {}, ym2[W] = {}, yp2[W] = {}, zm2[W] = {}, zp2[W] = {};
+                if (M.mask) {
+                    vld<T>(fp - 2, xm2); vld<T>(fp + 2, xp2);
+                    vld<T>(fp - 2 * sy, ym2); vld<T>(fp + 2 * sy, yp2);
+                    vld<T>(fp - 2 * sz, zm2); vld<T>(fp + 2 * sz, zp2);
+                }
+                T Fw[W] = {};
                 if (M.wslot >= 0) {
                     const double *d = wdat + 6L * M.wslot;
                     const T phi = (T)d[0], uwx = (T)d[1], uwy = (T)d[2], uwz = (T)d[3], Tw = (T)d[4];
-                    const T ax = vx - uwx, ay = vy - uwy, az = vz - uwz;
-                    const T cw = ax * (T)M.nwx + ay * (T)M.nwy + az * (T)M.nwz;
-                    const T m1 = dexp(-(ax * ax + ay * ay + az * az) / (T(2) * Tw)) * norm3(Tw);
-                    Fw = (T)M.sw * (fmin(cw, T(0)) * (phi * m1) + fmax(cw, T(0)) * fc);
+                    const T ay = cy.vy - uwy, az = cy.vz - uwz;
+                    const T n3 = norm3(Tw);
+#pragma unroll
+                    for (int e = 0; e < W; ++e) {
+                        const T ax = vx[e] - uwx;
+                        const T cw = ax * (T)M.nwx + ay * (T)M.nwy + az * (T)M.nwz;
+                        const T m1 = dexp(-(ax * ax + ay * ay + az * az) / (T(2) * Tw)) * n3;
+                        Fw[e] = (T)M.sw * (fmin(cw, T(0)) * (phi * m1) + fmax(cw, T(0)) * fc[e]);
+                    }
                 }
                 const bool mxm = M.mask & 1, mxp = M.mask & 2, mym = M.mask & 4, myp = M.mask & 8;
                 const bool mzm = M.mask & 16, mzp = M.mask & 32;
-                const T xm1 = fg[(long)(pc - 1) * Wd], xp1 = fg[(long)(pc + 1) * Wd];
-                const T ym1 = fg[(long)(pc - sy) * Wd], yp1 = fg[(long)(pc + sy) * Wd];
-                const T zm1 = fg[(long)(pc - sz) * Wd], zp1 = fg[(long)(pc + sz) * Wd];
-                T xm2 = 0, xp2 = 0, ym2 = 0, yp2 = 0, zm2 = 0, zp2 = 0;
-                if (M.mask) {
-                    xm2 = fg[(long)(pc - 2) * Wd]; xp2 = fg[(long)(pc + 2) * Wd];
-                    ym2 = fg[(long)(pc - 2 * sy) * Wd]; yp2 = fg[(long)(pc + 2 * sy) * Wd];
-                    zm2 = fg[(long)(pc - 2 * sz) * Wd]; zp2 = fg[(long)(pc + 2 * sz) * Wd];
+#pragma unroll
+                for (int e = 0; e < W; ++e) {
+                    const T Fxp = face_flux3<T>((T)M.A[1], vx[e], nux[e], xm1[e], fc[e], xp1[e], xp2[e], mxp);
+                    const T Fxm = face_flux3<T>((T)M.A[0], vx[e], nux[e], xm2[e], xm1[e], fc[e], xp1[e], mxm);
+                    const T Fyp = face_flux3<T>((T)M.A[3], cy.vy, cy.nuy, ym1[e], fc[e], yp1[e], yp2[e], myp);
+                    const T Fym = face_flux3<T>((T)M.A[2], cy.vy, cy.nuy, ym2[e], ym1[e], fc[e], yp1[e], mym);
+                    const T Fzp = face_flux3<T>((T)M.A[5], cy.vz, cy.nuz, zm1[e], fc[e], zp1[e], zp2[e], mzp);
+                    const T Fzm = face_flux3<T>((T)M.A[4], cy.vz, cy.nuz, zm2[e], zm1[e], fc[e], zp1[e], mzm);
+                    R[e] += (Fxp - Fxm) + (Fyp - Fym) + (Fzp - Fzm) + Fw[e];
                 }
-                const T Fxp = face_flux3<T>((T)M.A[1], vx, nux, xm1, fc, xp1, xp2, mxp);
-                const T Fxm = face_flux3<T>((T)M.A[0], vx, nux, xm2, xm1, fc, xp1, mxm);
-                const T Fyp = face_flux3<T>((T)M.A[3], vy, nuy, ym1, fc, yp1, yp2, myp);
-                const T Fym = face_flux3<T>((T)M.A[2], vy, nuy, ym2, ym1, fc, yp1, mym);
-                const T Fzp = face_flux3<T>((T)M.A[5], vz, nuz, zm1, fc, zp1, zp2, mzp);
-                const T Fzm = face_flux3<T>((T)M.A[4], vz, nuz, zm2, zm1, fc, zp1, mzm);
-                R += (Fxp - Fxm) + (Fyp - Fym) + (Fzp - Fzm) + Fw;
             }
-            const T fcv = fg[(long)I.pcm * Wd];
-            const T dxu = vx - ux, dyu = vy - uy, dzu = vz - uz;
-            const T c2u = dxu * dxu + dyu * dyu + dzu * dzu;
-            T feq = A * dexp(-c2u * i2T);
-            if (c.qh) feq *= fma(kqx * dxu + kqy * dyu + kqz * dzu, c2u * T(2) * i2T - T(5), T(1));
-            const T fn = fcv - bco * R + r * (feq - fcv);
-            T *og = fout + (long)grp * g.slab * g.W + e;
+            T fn[W];
+            vld<T>(fg + I.pcm, fn);
+            const T dyu = cy.vy - uy, dzu = cy.vz - uz;
+#pragma unroll
+            for (int e = 0; e < W; ++e) {
+                const T fcv = fn[e], dxu = vx[e] - ux;
+                const T c2u = dxu * dxu + dyu * dyu + dzu * dzu;
+                T feq = A * dexp(-c2u * i2T);
+                if (c.qh) feq *= fma(kqx * dxu + kqy * dyu + kqz * dzu, c2u * T(2) * i2T - T(5), T(1));
+                fn[e] = fcv - bco * R[e] + r * (feq - fcv);
+                acc[0].add(fn[e]); acc[1].add(vx[e] * fn[e]); acc[2].add(cy.vy * fn[e]); acc[3].add(cy.vz * fn[e]);
+                acc[4].add(T(0.5) * (vx[e] * vx[e] + cy.vy * cy.vy + cy.vz * cy.vz) * fn[e]);
+            }
+            V *og = reinterpret_cast<V *>(fout) + (long)grp * g.slab;
             for (int t = 0; t < nm; ++t) {
                 const CvMember3 &M = I.mem[t];
-                og[(long)M.pc * Wd] = fn;
+                vst<T>(og + M.pc, fn);
                 for (int u = 0; u < 6; ++u)
-                    if (M.mir[u] >= 0) og[(long)M.mir[u] * Wd] = fn;
+                    if (M.mir[u] >= 0) vst<T>(og + M.mir[u], fn);
             }
-            acc[0].add(fn); acc[1].add(vx * fn); acc[2].add(vy * fn); acc[3].add(vz * fn);
-            acc[4].add(T(0.5) * (vx * vx + vy * vy + vz * vz) * fn);
         }
         T t5[5];
-#pragma unroll
-        for (int q = 0; q < 5; ++q) t5[q] = block_acc(acc[q], red);
+        group_acc(acc, t5, red, blockDim.x >> 5);
         if (threadIdx.x < nm) write_split_partials3<T>(pout, sp, nc, I.mem[threadIdx.x].cell, t5);
         __syncthreads();
     }
@@ -1535,18 +1584,19 @@ __global__ void k_ghost3(Grid3D g, const double *prim, int side, int nside, T *f
 }
 
 // Padding of periodic and zero-gradient sides from the interior (both
-// layers); one thread copies one group's vector.  One element per thread
-// (four threads of other slabs' sectors per vector) took 2.9 ms at 64^3 x
-// 20^3, FP32.
+// layers); one thread finds a padding cell's source once and copies the
+// vectors of kHaloGroups groups, all loads in flight.  64^3 x 20^3, FP32: one
+// vector per thread, bound by the divisions that find the cell, 0.71 ms; now
+// 0.55 ms.
+constexpr int kHaloGroups = 8;
 template <typename T>
 __global__ void k_halo3(Grid3D g, T *f)
 {
     using V = typename Vec<T>::type;
     const long fx = (long)g.ny * g.nz, fy = (long)g.nx * g.nz, fz = (long)g.nx * g.ny;
     const long per = 2 * (fx + fy + fz);      // padding cells of one layer
-    const long t = (long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= 2 * per * g.ngrp) return;
-    const long hc = t % (2 * per);
+    const long hc = (long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (hc >= 2 * per) return;
     const int layer = (int)(hc / per) + 1;
     long pos = hc % per;
     int side;
@@ -1573,8 +1623,17 @@ __global__ void k_halo3(Grid3D g, T *f)
         if (side == 4) { dk = -layer; sk = per_ ? g.nz - layer : 0; }
         else { dk = g.nz - 1 + layer; sk = per_ ? layer - 1 : g.nz - 1; }
     }
-    V *const slab = reinterpret_cast<V *>(f) + t / (2 * per) * g.slab;
-    slab[nbr3(g, di, dj, dk)] = slab[nbr3(g, si, sj, sk)];
+    const int q0 = blockIdx.y * kHaloGroups, n = min(kHaloGroups, g.ngrp - q0);
+    V *const slab = reinterpret_cast<V *>(f) + (long)q0 * g.slab;
+    const V *const src = slab + nbr3(g, si, sj, sk);
+    V *const pad = slab + nbr3(g, di, dj, dk);
+    V v[kHaloGroups];
+#pragma unroll
+    for (int q = 0; q < kHaloGroups; ++q)
+        if (q < n) v[q] = src[(long)q * g.slab];
+#pragma unroll
+    for (int q = 0; q < kHaloGroups; ++q)
+        if (q < n) pad[(long)q * g.slab] = v[q];
 }
 
 // Zero the state of every solid cell: one thread per cell and chunk of the
@@ -1840,7 +1899,9 @@ cudaError_t step3d_t(dvm_ctx *c, int phase, double *xbuf)
     if ((e = timing_mark(c, 1)) != cudaSuccess) return e;
     c->launches += 1;
     if (body) {
-        k_special3<T><<<cvgrid, 256, 0, c->wstream>>>(cv, fin, fout, pin, pout, c->wphi);
+        // as many threads as four blocks of 256 an SM
+        const int st = spec3_threads(cv.gps);
+        k_special3<T><<<cvgrid * kSpec3Threads / st, st, 0, c->wstream>>>(cv, fin, fout, pin, pout, c->wphi);
         if ((e = cudaEventRecord(c->ev_wjoin, c->wstream)) != cudaSuccess) return e;
         // the step ends when both streams are done
         if ((e = cudaStreamWaitEvent(c->stream, c->ev_wjoin, 0)) != cudaSuccess) return e;
@@ -2063,9 +2124,9 @@ cudaError_t halo3d(dvm_ctx *c, int buf)
 {
     const Grid3D g = grid3d(c);
     const long per = 2L * ((long)c->ny * c->nz + (long)c->nx * c->nz + (long)c->nx * c->ny);
-    const long n = 2 * per * c->ngrp;
-    if (c->prec == DVM_FP32) k_halo3<float><<<nb3(n, 256), 256, 0, c->stream>>>(g, (float *)c->f[buf]);
-    else k_halo3<double><<<nb3(n, 256), 256, 0, c->stream>>>(g, (double *)c->f[buf]);
+    const dim3 grid(nb3(2 * per, 256), nb3(c->ngrp, kHaloGroups));
+    if (c->prec == DVM_FP32) k_halo3<float><<<grid, 256, 0, c->stream>>>(g, (float *)c->f[buf]);
+    else k_halo3<double><<<grid, 256, 0, c->stream>>>(g, (double *)c->f[buf]);
     return cudaGetLastError();
 }
 
