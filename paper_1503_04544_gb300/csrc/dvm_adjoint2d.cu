@@ -545,10 +545,11 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_adj_gather_fast(AdjArgs a, co
 {
     using V = typename Vec<T>::type;
     constexpr int W = Vec<T>::W;
-    // a group's W coefficients (64 bytes in both precisions) and its signs
-    // arrive with its tile: read through L1 they cost an L2 latency a group
-    // (261 -> 248 us a launch at 256^2 x 32^2)
-    constexpr uint32_t kCoef = W * sizeof(VCoef<T>);
+    // a group's coefficients and its signs (FP32: its rows of k_tables, FP64:
+    // its W VCoef and the row of signs) arrive with its tile: read through L1
+    // they cost an L2 latency a group (261 -> 248 us a launch at 256^2 x 32^2)
+    constexpr bool PK = sizeof(T) == 4;
+    constexpr uint32_t kCoef = PK ? kTabBytes - 16 : W * sizeof(VCoef<T>);
     constexpr uint32_t kBytes = (MUSCL ? kAdjLamBytes + kTileY * kTileX * 4 : kAdjLamBytes) + kCoef + 16;
     static_assert(kCoef + 16 <= kTabBytes, "a stage's table slot");
     extern __shared__ __align__(128) unsigned char smem[];
@@ -572,8 +573,12 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_adj_gather_fast(AdjArgs a, co
         mbar_expect_tx(&full[st], kBytes);
         tma_load_3d(dst, &lmap, &full[st], i0 * W, j0, q * 2);
         if (MUSCL) tma_load_3d(dst + kAdjLamBytes, &bmap, &full[st], i0, j0, q);
-        bulk_load(tab + st * kTabBytes, vt + (long)q * W, kCoef, &full[st]);
-        bulk_load(tab + st * kTabBytes + kCoef, ptab + (long)q * kTabRows + 7, 16, &full[st]);
+        if (PK) {
+            bulk_load(tab + st * kTabBytes, ptab + (long)q * kTabRows, kTabBytes, &full[st]);
+        } else {
+            bulk_load(tab + st * kTabBytes, vt + (long)q * W, kCoef, &full[st]);
+            bulk_load(tab + st * kTabBytes + kCoef, ptab + (long)q * kTabRows + 7, 16, &full[st]);
+        }
     };
     if (tid == 0) {
         for (int st = 0; st < kAdjStages; ++st) {
@@ -606,25 +611,102 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_adj_gather_fast(AdjArgs a, co
             const unsigned char *base = smem + (long)st * kAdjStageBytes;
             const uint32_t *bt = reinterpret_cast<const uint32_t *>(base + kAdjLamBytes);
             const int p = q * W;
-            T vx[W], vy[W], nux[W], nuy[W], rel0[W];
-#pragma unroll
-            for (int e = 0; e < W; ++e) {
-                const VCoef<T> vc = reinterpret_cast<const VCoef<T> *>(tab + st * kTabBytes)[e];
-                vx[e] = vc.vx; vy[e] = vc.vy; nux[e] = vc.nux; nuy[e] = vc.nuy;
-                rel0[e] = dv * (S0 + S1 * vx[e] + S2 * vy[e] + S3 * T(0.5) * (vx[e] * vx[e] + vy[e] * vy[e]));
-            }
             const int2 sg = *reinterpret_cast<const int2 *>(tab + st * kTabBytes + kCoef);
             const int sgx = sg.x, sgy = sg.y;
             uint32_t bo = 0, bxm = 0, bxp = 0, bym = 0, byp = 0;
             if (MUSCL) {
                 bo = bt[c0]; bxm = bt[c0 - 1]; bxp = bt[c0 + 1]; bym = bt[c0 - kTileX]; byp = bt[c0 + kTileX];
             }
+            if constexpr (PK) {
+                if (sgx != 0 && sgy != 0) {
+                    // upwind direction uniform over the group: pairs of
+                    // velocities, the differences and sums packed (one
+                    // velocity at a time: 248 us a launch at 256^2 x 32^2,
+                    // now 207)
+                    const float4 *const row = reinterpret_cast<const float4 *>(tab + st * kTabBytes);
+                    F2 nn[2][2], kap[2][2], rel[2], w[2];      // [axis][pair]: -nu, (1 - nu)/2
+                    ld_units(row, nn[0]); ld_units(row + 1, nn[1]);
+                    ld_units(row + 2, kap[0]); ld_units(row + 3, kap[1]);
+#pragma unroll
+                    for (int h = 0; h < 4; ++h) kap[h >> 1][h & 1] = mul2(f2(0.5f), kap[h >> 1][h & 1]);
+                    rel[0] = rel[1] = f2(S0);
+                    const T sm[3] = {S1, S2, S3};
+#pragma unroll
+                    for (int m = 0; m < 3; ++m) {
+                        ld_units(row + 4 + m, w);
+                        rel[0] = fma2(f2(sm[m]), w[0], rel[0]);
+                        rel[1] = fma2(f2(sm[m]), w[1], rel[1]);
+                    }
+                    const int up[2] = {sgx > 0 ? 1 : -1, sgy > 0 ? kTileX : -kTileX};
+                    const uint32_t bm[2] = {sgx > 0 ? bxm : bxp, sgy > 0 ? bym : byp};
+                    const uint32_t bp[2] = {sgx > 0 ? bxp : bxm, sgy > 0 ? byp : bym};
+#pragma unroll
+                    for (int comp = 0; comp < 2; ++comp) {
+                        const float4 *t = reinterpret_cast<const float4 *>(base) + comp * kTileY * kTileX + c0;
+                        F2 l0[2], o[2];
+                        ld_units(t, l0);
+#pragma unroll
+                        for (int h = 0; h < 2; ++h)
+                            o[h] = fma2(l0[h], f2(omr), comp == 0 ? mul2(f2(dv), rel[h]) : f2(dv * S3));
+#pragma unroll
+                        for (int ax = 0; ax < 2; ++ax) {
+                            // adj_axis with every sign turned, for -nu
+                            F2 lm[2], lp[2], lq[2];
+                            ld_units(t + up[ax], lp);
+                            if (MUSCL) {
+                                ld_units(t - up[ax], lm);
+                                ld_units(t + 2 * up[ax], lq);
+                            }
+#pragma unroll
+                            for (int h = 0; h < 2; ++h) {
+                                const F2 wk = sub2(l0[h], lp[h]);
+                                F2 d = wk;
+                                if (MUSCL) {
+                                    float k[2], m[2], n[2], cr[2];
+                                    f2_get(wk, k[0], k[1]);
+                                    f2_get(sub2(lm[h], l0[h]), m[0], m[1]);
+                                    f2_get(sub2(lq[h], lp[h]), n[0], n[1]);
+#pragma unroll
+                                    for (int l = 0; l < 2; ++l) {
+                                        const uint32_t b1 = 1u << (((comp * 2 + ax) * 4 + 2 * h + l) * 2), b2 = 2 * b1;
+                                        cr[l] = (bo & b1) ? -k[l] : ((bo & b2) ? k[l] : 0.f);
+                                        if (bm[ax] & b1) cr[l] += m[l];
+                                        if (bp[ax] & b2) cr[l] += n[l];
+                                    }
+                                    d = fma2(kap[ax][h], f2(cr[0], cr[1]), wk);
+                                }
+                                o[h] = fma2(nn[ax][h], d, o[h]);
+                            }
+                        }
+                        T out[W];
+                        f2_get(o[0], out[0], out[1]);
+                        f2_get(o[1], out[2], out[3]);
+                        if (p + W > g.nv)
+#pragma unroll
+                            for (int e = 0; e < W; ++e) out[e] = p + e < g.nv ? out[e] : T(0);
+                        vst<T>(reinterpret_cast<V *>(lam_out + ebase<T>(g, comp, p)) + pc, out);
+                    }
+                    goto released;
+                }
+            }
+            T vx[W], vy[W], nux[W], nuy[W], rel0[W];
+#pragma unroll
+            for (int e = 0; e < W; ++e) {
+                if constexpr (PK) {
+                    const float *row = reinterpret_cast<const float *>(tab + st * kTabBytes) + e;
+                    nux[e] = -row[0]; nuy[e] = -row[4]; vx[e] = row[16]; vy[e] = row[20];
+                } else {
+                    const VCoef<T> vc = reinterpret_cast<const VCoef<T> *>(tab + st * kTabBytes)[e];
+                    vx[e] = vc.vx; vy[e] = vc.vy; nux[e] = vc.nux; nuy[e] = vc.nuy;
+                }
+                rel0[e] = dv * (S0 + S1 * vx[e] + S2 * vy[e] + S3 * T(0.5) * (vx[e] * vx[e] + vy[e] * vy[e]));
+            }
 #pragma unroll
             for (int comp = 0; comp < 2; ++comp) {
                 const V *t = reinterpret_cast<const V *>(base) + comp * kTileY * kTileX;
                 T l0[W], out[W];
                 sld<T>(t + c0, l0);
-                if (sgx != 0 && sgy != 0) {
+                if (!PK && sgx != 0 && sgy != 0) {
                     // upwind direction uniform over the group
                     const int ux = sgx > 0 ? 1 : -1, uy = sgy > 0 ? kTileX : -kTileX;
                     T xm[W], xp[W], xq[W], ym[W], yp[W], yq[W];
@@ -670,6 +752,7 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_adj_gather_fast(AdjArgs a, co
                 }
                 vst<T>(reinterpret_cast<V *>(lam_out + ebase<T>(g, comp, p)) + pc, out);
             }
+        [[maybe_unused]] released:;
         }
         __syncwarp();
         if (tx == 0) mbar_arrive(&empty[st]);
