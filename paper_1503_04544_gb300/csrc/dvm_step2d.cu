@@ -1441,10 +1441,15 @@ template <typename T>
 __global__ void __launch_bounds__(256) k_wall(CvArgs c, BodyParams b, const BodyDev *body, const T *f,
                                               double *wdat, double *wcontrib, int mode, double *xw)
 {
-    __shared__ double ex[kMaxAxisNv], ey[kMaxAxisNv];
+    // per axis: the Maxwellian's factors and the velocities about the wall's,
+    // in FP64 and in the type of the sums.  Formed for every velocity instead
+    // (15 FP64 operations and conversions, now 5) they bounded the kernel:
+    // 14.2 -> 12.5 us a launch at 64^2 x 20^2, 18.8 -> 14.7 us at 256^2 x 32^2.
+    using WA = typename std::conditional<sizeof(T) == 4, float, double>::type;   // wall-sum type
+    __shared__ double ex[kMaxAxisNv], ey[kMaxAxisNv], axd[kMaxAxisNv], ayd[kMaxAxisNv];
+    __shared__ WA axs[kMaxAxisNv], ays[kMaxAxisNv];
     __shared__ double wsc[6];   // uwx, uwy, nwx, nwy, 1/(2 pi Tw), 2 Tw
     __shared__ WallGeom wg;
-    using WA = typename std::conditional<sizeof(T) == 4, float, double>::type;   // wall-sum type
     __shared__ WA wred[8 * 3 * 8];
     const Grid2D &g = c.g;
     const int nw = min(c.counts[1], c.cap);
@@ -1467,10 +1472,20 @@ __global__ void __launch_bounds__(256) k_wall(CvArgs c, BodyParams b, const Body
         } else {
         __syncthreads();
         const double uwx = wsc[0], uwy = wsc[1], nwx = wsc[2], nwy = wsc[3], cm = wsc[4], twoTw = wsc[5];
-        // separable Maxwellian M[1, u_w, T_w] = ex[p1] ey[p2] / (2 pi T_w)
+        // separable Maxwellian M[1, u_w, T_w] = ex[p1] ey[p2]
         for (int q = tid; q < g.nvx + g.nvy; q += blockDim.x) {
-            if (q < g.nvx) { const double d = g.vxmin + q * g.dvx - uwx; ex[q] = exp(-(d * d) / twoTw); }
-            else { const int qq = q - g.nvx; const double d = g.vymin + qq * g.dvy - uwy; ey[qq] = exp(-(d * d) / twoTw); }
+            if (q < g.nvx) {
+                const double d = g.vxmin + q * g.dvx - uwx;
+                axd[q] = d;
+                axs[q] = (WA)d;
+                ex[q] = cm * exp(-(d * d) / twoTw);
+            } else {
+                const int qq = q - g.nvx;
+                const double d = g.vymin + qq * g.dvy - uwy;
+                ayd[qq] = d;
+                ays[qq] = (WA)d;
+                ey[qq] = exp(-(d * d) / twoTw);
+            }
         }
         __syncthreads();
         const long pck = pcell(g, k) * Vec<T>::W;
@@ -1478,15 +1493,14 @@ __global__ void __launch_bounds__(256) k_wall(CvArgs c, BodyParams b, const Body
         int p1 = tid % g.nvx, p2 = tid / g.nvx;
         const int dp1 = blockDim.x % g.nvx, dp2 = blockDim.x / g.nvx;
         for (int p = tid; p < g.nv; p += blockDim.x) {
-            const double ax = g.vxmin + p1 * g.dvx - uwx, ay = g.vymin + p2 * g.dvy - uwy;
-            const double cp = ax * nwx + ay * nwy;
-            const WA cw = (WA)cp, axw = (WA)ax, ayw = (WA)ay;
+            const double cp = axd[p1] * nwx + ayd[p2] * nwy;
+            const WA cw = (WA)cp, axw = axs[p1], ayw = ays[p2];
             if (cp > 0.0) {
                 const WA fv = (WA)f[ebase<T>(g, 0, p) + pck];
                 w8[0].add(cw * fv);
                 w8[5].add(axw * axw * fv); w8[6].add(axw * ayw * fv); w8[7].add(ayw * ayw * fv);
             } else if (cp < 0.0) {
-                const WA m1 = (WA)(cm * ex[p1] * ey[p2]);
+                const WA m1 = (WA)(ex[p1] * ey[p2]);
                 w8[1].add(cw * m1);
                 w8[2].add(axw * axw * m1); w8[3].add(axw * ayw * m1); w8[4].add(ayw * ayw * m1);
             }
@@ -1598,15 +1612,16 @@ __global__ void __launch_bounds__(256, (sizeof(T) == 4) + !SHAK + 1)
     const int gt = threadIdx.x % (32 * kw);          // thread of the split's warps
     for (int item = blockIdx.x; item < n; item += gridDim.x - 1) {
         const int idx = item / items, sp = item % items * nsb + (threadIdx.x >> 5) / kw;
+        // the master's sums are on their way while the record arrives
+        const long m = c.spec_list[idx];
+        T s[4];
+        gather_partials(pin, c.Sin, nc, m, s);
         load_info(info + idx, &I);
         if (!I.ok) { __syncthreads(); continue; }
         const int nm = I.nm;
         int v0, v1;
         split_range(c, sp, W, v0, v1);
         const bool on = sp < c.S;
-        const long m = c.spec_list[idx];
-        T s[4];
-        gather_partials(pin, c.Sin, nc, m, s);
         T rho, ux, uy, tmp;
         if (!primitives<T>(pick<T>(g.dv_f, g.dv), s[0], s[1], s[2], s[3], rho, ux, uy, tmp) && threadIdx.x == 0 && sp == 0)
             atomicExch(&c.err[kErrNonphys], 1);
