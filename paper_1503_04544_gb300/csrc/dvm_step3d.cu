@@ -1000,7 +1000,8 @@ __global__ void __launch_bounds__(256) k_fusion3(Cv3Args c, T *f, T *part)
 // (r - c) (Eq. uwDD).  One block per wall cell: products and compensated sums
 // in the state precision over all velocities, a thread a velocity group (one
 // vector, one pair of divisions for its W velocities) and the 14 sums merged
-// together (64^3 x 20^3: 0.175 -> 0.135 ms a launch), phi and the stress in FP64 by thread 0.  The last block sums the cells in list order into the body
+// together (64^3 x 20^3: 0.175 -> 0.135 ms a launch), phi and the stress in
+// FP64 by thread 0.  The last block sums the cells in list order into the body
 // record and the history.  (phi, u_w, T_w) of each wall cell are left for
 // the control-volume kernel.
 template <typename T>
