@@ -544,11 +544,7 @@ __device__ __forceinline__ void mirrors(const Grid2D &g, int i, int j, I (&m)[4]
 // groups of velocities (31 of a 50 us launch at 32^2 x 16^2).  Eight threads
 // of a warp share a cell: each sums every eighth split, all form the
 // primitives, and the exponentials are dealt out.
-constexpr int kMxBlocks = 4;         // restarts of the Maxwellian's recurrence along a v_x row
 constexpr int kCellThreads = 8;
-
-// Velocities between restarts.
-__device__ __forceinline__ int restart64(int nvx) { return nvx <= 8 * kMxBlocks ? 8 : 16; }
 
 // Sum over the eight threads of a cell (every thread returns it).
 __device__ __forceinline__ double cell_sum(double x)
@@ -558,19 +554,20 @@ __device__ __forceinline__ double cell_sum(double x)
     return x;
 }
 
-// The recurrence's values of a cell into slots [slot][nc]: Q = 2^(-2 c2 dv^2)
-// in slot q, and for every restart velocity v_b the factor A 2^(-c2 (v_b -
-// ux)^2) in slot m + b and R = 2^(-c2 (2 (v_b - ux) dv + dv^2)) in slot r + b.
-__device__ __forceinline__ void put_recurrence(double *cf, long nc, int k, int nvx, double vmin, double dv, double ux,
-                                               double c2, double A, int q, int m, int r)
+// The Maxwellian's v_x factors of a cell into rows [n][nc]: A 2^(-c2 (v - ux)^2)
+// for each of the nvx velocities, 0 in the padding up to n.  M is this factor
+// times the row's factor of the other axes: two exp2 arguments that add up to
+// the one of M, so each value is as exact as its own exp2, tails included, at
+// any spacing dv against sqrt(T) and one FP64 multiplication a velocity.  (A
+// recurrence M(v + dv) = M R, R(v + dv) = R Q from a row's start took two
+// multiplications, 256^2 x 32^2 4.31 ms a launch against 4.14, and lost M
+// where it underflowed at the start of a coarse row.)
+__device__ __forceinline__ void put_factors(double *mx, long nc, int k, int nvx, int n, double vmin, double dv, double ux,
+                                            double c2, double A)
 {
-    const int rec = restart64(nvx), nb = (nvx + rec - 1) / rec;
-    for (int v = k; v <= 2 * nb; v += kCellThreads) {
-        const int b = v >> 1;
-        const double dx = vmin + b * rec * dv - ux;
-        const double x = v == 2 * nb ? 2.0 * dv * dv : (v & 1 ? fma(2.0 * dx, dv, dv * dv) : dx * dx);
-        const double e = exp2(-c2 * x);
-        cf[(long)(v == 2 * nb ? q : (v & 1 ? r : m) + b) * nc] = v < 2 * nb && !(v & 1) ? A * e : e;
+    for (int v = k; v < n; v += kCellThreads) {
+        const double dx = vmin + v * dv - ux;
+        mx[v * nc] = v < nvx ? A * exp2(-c2 * (dx * dx)) : 0.0;
     }
 }
 

@@ -69,7 +69,7 @@ template <typename T> struct BulkArgs {
     const VCoef<T> *vt;       // [nvp]
     const float4 *pt;         // [ngrp][kTabRows] coefficients of a group (k_tables)
     const T *eqp;             // [4][nc] conservative equilibrium parameters, or null (direct moments)
-    const double *cf;         // FP64: per-cell values [C64][nc] (k_cell64)
+    const double *cf;         // FP64: per-cell values [kC64S + nvx][nc] (k_cell64)
     const T *qh;              // [2][nc] heat flux of the control volume at t^n (Shakhov model), used when hin is null
     const T *hin;             // Shakhov: raw heat-flux moments of f^n [S][5][nc] and their reference velocity [2][nc]
     T *hout;                  // Shakhov: the same for f^n+1
@@ -775,28 +775,27 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<T> a, const __g
 
 // ------------------------------------------------------------ FP64 bulk kernel
 // On this part an FP64 operation holds the pipe of an SM's quarter for 64
-// clocks a warp, so this kernel counts FP64 operations and little else: 33 a
+// clocks a warp, so this kernel counts FP64 operations and little else: 32 a
 // velocity pair (f, g) and cell, against 64 of the form it replaced (one cell
 // per thread, every difference from both sides, weights on every face, a
 // limiter whose magnitudes the compiler formed on the FP64 pipe): 7.90 ->
-// 4.31 ms a launch at 256^2 x 32^2, limited fluxes (with k_cell64, 0.14 ms).
+// 4.14 ms a launch at 256^2 x 32^2, limited fluxes (with k_cell64, 0.15 ms).
 //
 // Block = 32 x 8 cells, four warps of 32 cells in x and two rows.  A thread
 // takes its two cells in upwind order of v_y: they share the face between
 // them, so a pair of cells costs four y differences and three y limiter
 // values instead of six and four.  Warps whose cells all have the limiter on
-// every face use no face weights.  The Maxwellian times dt/tau along a v_x row
-// is the recurrence M(v + dv) = M R, R(v + dv) = R Q, restarted every 8
-// velocities (16 from 33 per axis on) from the cell's v_x factor in shared
-// memory times the row's v_y factor (one exp2 per row and cell); relative
-// error below 30 ulp (130).  A group whose v_y changes sign between its two
-// velocities (odd nvx) takes each velocity's neighbours on its own side.
+// every face use no face weights.  The Maxwellian times dt/tau is the cell's
+// v_x factor (put_factors; read a group ahead, without which a launch of few
+// groups waits for it: 36.3 -> 37.4 us a step at 32^2 x 16^2) times the row's
+// v_y factor (one exp2 per row and cell).  A group whose v_y changes sign
+// between its two velocities (odd nvx) takes each velocity's neighbours on its
+// own side.
 constexpr int kRows64 = 4;            // warps of a block
 constexpr int kZ64 = 2;               // rows of a thread
 constexpr int kStages64 = 3;
 static_assert(kRows64 * kZ64 == kRows, "the tile of the state's tensor maps");
-enum C64 { kUy = 0, kC2, kRel, kGf, kQm, kMb, kRb = kMb + kMxBlocks, kC64 = kRb + kMxBlocks,
-           kKqx = kC64, kKqy, kUx, kIT, kC64S };
+enum C64 { kUy = 0, kC2, kRel, kGf, kC64, kKqx = kC64, kKqy, kUx, kIT, kC64S };
 
 template <bool SHAK> constexpr size_t bulk64_smem()
 {
@@ -813,7 +812,8 @@ __device__ __forceinline__ uint32_t branch_code(double m, double b)
 }
 
 // The per-cell values of k_bulk64 for the plain cells (dvm_device.cuh): the
-// slots of C64.  Block = 16 cells x kCellThreads.
+// slots of C64, then the v_x factors from slot kC64S on.  Block = 16 cells x
+// kCellThreads.
 template <bool SHAK> __global__ void __launch_bounds__(128) k_cell64(BulkArgs<double> a, double *cf)
 {
     const Grid2D &g = a.g;
@@ -840,7 +840,7 @@ template <bool SHAK> __global__ void __launch_bounds__(128) k_cell64(BulkArgs<do
     }
     const double iT = 1.0 / tmp, c2 = (0.5 * kLog2e) * iT;
     double *const o = cf + cell;
-    put_recurrence(o, nc, k, g.nvx, g.vxmin, g.dvx, ux, c2, r * rho * (0.5 / kPi) * iT, kQm, kMb, kRb);
+    put_factors(o + kC64S * nc, nc, k, g.nvx, g.nvx, g.vxmin, g.dvx, ux, c2, r * rho * (0.5 / kPi) * iT);
     if (k == kCellThreads - 1) {
         o[kUy * nc] = uy;
         o[kC2 * nc] = c2;
@@ -875,7 +875,6 @@ __global__ void __launch_bounds__(32 * kRows64, SHAK ? 2 : 3)
     const int gps = (g.ngrp + a.S - 1) / a.S;
     const int g0 = split * gps, g1 = min(g0 + gps, g.ngrp);
     const int ngr = max(g1 - g0, 0);
-    const int rec = restart64(g.nvx);
     const auto load_group = [&](int n) {
         mbar_expect_tx(&full[n % NST], kStageBytes);
         tma_load_3d(ring + (n % NST) * (kStageBytes / 16), &tmap, &full[n % NST], i0 * 2, j0, (g0 + n) * 2);
@@ -889,11 +888,13 @@ __global__ void __launch_bounds__(32 * kRows64, SHAK ? 2 : 3)
         if (ngr > 0) load_group(0);
     }
     uint32_t word = 0, fullm = 0;   // bit t: cell t plain, 4 + t: to be zeroed, 8 + 4 t: its face mask
+    const double *fac[ZC];          // v_x factors of the cells (of cell 0 outside the grid)
 #pragma unroll
     for (int t = 0; t < ZC; ++t) {
         const int j = jt + t;
         const bool in = i < g.nx && j < g.ny;
         const long cell = (long)j * g.nx + i;
+        fac[t] = a.cf + kC64S * nc + (in ? cell : 0);
         const uint8_t fl = in ? a.flags[cell] : 0;
         double *const cz = coef + t * NT;       // slot k of the cell: cz[k * ZC * NT]
         if (fl & kPlain) {
@@ -935,12 +936,21 @@ __global__ void __launch_bounds__(32 * kRows64, SHAK ? 2 : 3)
     for (int t = 0; t < ZC; ++t)
 #pragma unroll
         for (int m = 0; m < 4; ++m) q[t][m] = 0;
-    double Mr[ZC], Rr[ZC], Er[ZC], kyr[ZC], d4r[ZC];   // recurrence; the row's factor and Shakhov terms
+    double Er[ZC], kyr[ZC], d4r[ZC];        // the row's factor and Shakhov terms
 #pragma unroll
-    for (int t = 0; t < ZC; ++t) Mr[t] = Rr[t] = Er[t] = kyr[t] = d4r[t] = 0;
+    for (int t = 0; t < ZC; ++t) Er[t] = kyr[t] = d4r[t] = 0;
     const double2 *const pt = reinterpret_cast<const double2 *>(a.pt);
     uint32_t bad = 0;
-    int p1 = (g0 * 2) % g.nvx;
+    int p1 = (g0 * 2) % g.nvx, p1n = p1 + 1 < g.nvx ? p1 + 1 : 0;   // v_x indices of the group's velocities
+    double fx[ZC][2];                       // their factors, read a group ahead
+    const auto load_factors = [&] {
+#pragma unroll
+        for (int t = 0; t < ZC; ++t) {
+            fx[t][0] = __ldg(fac[t] + p1 * nc);
+            fx[t][1] = __ldg(fac[t] + p1n * nc);
+        }
+    };
+    if (busy) load_factors();
     bool first = true;
     for (int it = 0; it < ngr; ++it) {
         if (tid == 0 && it + 1 < ngr) {
@@ -949,8 +959,8 @@ __global__ void __launch_bounds__(32 * kRows64, SHAK ? 2 : 3)
                 mbar_wait_or(smem_u32(&empty[(it + 1) % NST]), (uint32_t)(((it + 1) / NST - 1) & 1), bad);
             load_group(it + 1);
         }
-        mbar_wait_or(smem_u32(&full[it % NST]), (uint32_t)((it / NST) & 1), bad);
         const int grp = g0 + it;
+        mbar_wait_or(smem_u32(&full[it % NST]), (uint32_t)((it / NST) & 1), bad);
         if (busy) {
             const double2 *const tile = ring + (it % NST) * (kStageBytes / 16) + cb;
             double nnux[2], nnuy[2], kx[2], ky[2], vx[2], vy[2], ke[2];
@@ -969,25 +979,16 @@ __global__ void __launch_bounds__(32 * kRows64, SHAK ? 2 : 3)
 #pragma unroll
             for (int e = 0; e < 2; ++e) {
                 const bool pad = grp * 2 + e >= g.nv;
-                if ((p1 % rec == 0 || first) && !pad) {
-                    const int b = p1 / rec;
+                if ((e ? p1n : p1) == 0 || first) {
 #pragma unroll
                     for (int t = 0; t < ZC; ++t) {
                         const double *const cz = coef + t * NT;
-                        if (p1 == 0 || first) {
-                            const double dy = vy[e] - cz[kUy * ZC * NT], c2 = cz[kC2 * ZC * NT];
-                            Er[t] = exp2(-c2 * dy * dy);
-                            if constexpr (SHAK) {
-                                // k c.q = kqx dx + kqy dy, |c|^2/T - 4 = dx^2/T + (dy^2/T - 4)
-                                kyr[t] = cz[kKqy * ZC * NT] * dy;
-                                d4r[t] = fma(dy * cz[kIT * ZC * NT], dy, -4.0);
-                            }
-                        }
-                        Mr[t] = cz[(kMb + b) * ZC * NT] * Er[t];
-                        Rr[t] = cz[(kRb + b) * ZC * NT];
-                        for (int k = b * rec; k < p1; ++k) {          // a split that starts inside a row
-                            Mr[t] *= Rr[t];
-                            Rr[t] *= cz[kQm * ZC * NT];
+                        const double dy = vy[e] - cz[kUy * ZC * NT], c2 = cz[kC2 * ZC * NT];
+                        Er[t] = exp2(-c2 * dy * dy);
+                        if constexpr (SHAK) {
+                            // k c.q = kqx dx + kqy dy, |c|^2/T - 4 = dx^2/T + (dy^2/T - 4)
+                            kyr[t] = cz[kKqy * ZC * NT] * dy;
+                            d4r[t] = fma(dy * cz[kIT * ZC * NT], dy, -4.0);
                         }
                     }
                     first = false;
@@ -995,7 +996,7 @@ __global__ void __launch_bounds__(32 * kRows64, SHAK ? 2 : 3)
 #pragma unroll
                 for (int t = 0; t < ZC; ++t) {
                     const double *const cz = coef + t * NT;
-                    fe[t][e] = pad ? 0.0 : Mr[t];
+                    fe[t][e] = pad ? 0.0 : fx[t][e] * Er[t];
                     if constexpr (SHAK) {
                         const double dx = vx[e] - cz[kUx * ZC * NT];
                         const double mk = fe[t][e] * fma(cz[kKqx * ZC * NT], dx, kyr[t]);
@@ -1004,11 +1005,11 @@ __global__ void __launch_bounds__(32 * kRows64, SHAK ? 2 : 3)
                     } else {
                         ge[t][e] = fe[t][e];
                     }
-                    Mr[t] *= Rr[t];
-                    Rr[t] *= cz[kQm * ZC * NT];
                 }
-                if (++p1 == g.nvx) p1 = 0;
             }
+            p1 = p1n + 1 < g.nvx ? p1n + 1 : 0;
+            p1n = p1 + 1 < g.nvx ? p1 + 1 : 0;
+            load_factors();
             // the row differences beyond the warp's ends, one lane each: the two
             // of row t, component comp, velocity e in lanes 2 (e + 2 comp + 4 t)
             // and the next: D(32), and D(-1) (v_x >= 0) or D(33)
@@ -2560,7 +2561,7 @@ size_t vcoef_bytes(int prec) { return prec == DVM_FP32 ? sizeof(VCoef<float>) : 
 
 size_t cvinfo_bytes() { return sizeof(CvInfo); }
 
-size_t cf64_bytes2d(const dvm_ctx *c) { return sizeof(double) * kC64S * (size_t)c->nc; }
+size_t cf64_bytes2d(const dvm_ctx *c) { return sizeof(double) * (kC64S + c->nvx) * (size_t)c->nc; }
 
 cudaError_t members2d(dvm_ctx *c, bool moving)
 {

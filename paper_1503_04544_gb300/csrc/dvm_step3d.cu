@@ -143,7 +143,7 @@ template <typename T> struct Bulk3Args {
     const VX3<T> *vxt;        // [nvxp]
     const VYZ3<T> *vyz;       // [nvy * nvz]
     const T *eqp;             // [5][nc] conservative equilibrium parameters, or null (direct moments)
-    const double *cf;         // FP64: per-cell values [kMxCount][nc] (k_cell64_3)
+    const double *cf;         // FP64: per-cell values [kMxCount + nvxp][nc] (k_cell64_3)
     const T *qh;              // [3][nc] heat flux of the control volume at t^n (Shakhov model)
     T pr1;                    // 1 - Pr (Shakhov model)
     int *err;
@@ -167,8 +167,8 @@ template <bool SHAK> __host__ __device__ constexpr int ring3() { return SHAK?5:k
 
 // Per-cell values of the bulk kernel in shared memory.  FP32: c0, c1, c2, r
 // (one vector), uy, uz, and the Shakhov model's k q.  FP64: the values of
-// MxSlot for the Maxwellian's recurrence along v_x.
-enum MxSlot { kMxUy = 0, kMxUz, kMxC2, kMxRel, kMxQ, kMxM, kMxR = kMxM + kMxBlocks, kMxCount = kMxR + kMxBlocks };
+// MxSlot.
+enum MxSlot { kMxUy = 0, kMxUz, kMxC2, kMxRel, kMxCount };
 template <typename T, bool SHAK> __host__ __device__ constexpr int ncoef3()
 {
     return sizeof(T) == 8 ? kMxCount : (SHAK ? 9 : 6);
@@ -203,7 +203,8 @@ __device__ __forceinline__ float unit_lane(F2 x, int l) { float a, b; f2_get(x, 
 __device__ __forceinline__ double unit_lane(double x, int) { return x; }
 
 // The per-cell values of the FP64 bulk kernel for the plain cells
-// (dvm_device.cuh): the slots of MxSlot.  Block = 16 cells x kCellThreads.
+// (dvm_device.cuh): the slots of MxSlot, then the v_x factors.  Block = 16
+// cells x kCellThreads.
 __global__ void __launch_bounds__(128) k_cell64_3(Bulk3Args<double> a, double *cf)
 {
     const Grid3D &g = a.g;
@@ -231,7 +232,7 @@ __global__ void __launch_bounds__(128) k_cell64_3(Bulk3Args<double> a, double *c
     }
     const double c2 = (0.5 * kLog2e) / tmp;
     double *const o = cf + cell;
-    put_recurrence(o, nc, k, g.nvx, g.vxmin, g.dvx, ux, c2, r * rho * norm3(tmp), kMxQ, kMxM, kMxR);
+    put_factors(o + kMxCount * nc, nc, k, g.nvx, g.nvxp, g.vxmin, g.dvx, ux, c2, r * rho * norm3(tmp));
     if (k == kCellThreads - 1) {
         o[kMxUy * nc] = uy;
         o[kMxUz * nc] = uz;
@@ -266,15 +267,13 @@ __global__ void __launch_bounds__(128) k_cell64_3(Bulk3Args<double> a, double *c
 // v_x F and v_x^2 F over the row and forms the five moments once per row,
 // into compensated sums in shared memory.
 //
-// FP64: the Maxwellian along the row by the recurrence M(v + dv) = M R,
-// R(v + dv) = R Q, restarted every 8 velocities (16 from 33 velocities per
-// axis on) from per-cell values of the v_x factor, times the row's factor of
-// v_y and v_z (one exp2 a row): two FP64 multiplications a velocity instead of
-// an exp2.  Relative error below 30 ulp (130 for 33 and more velocities).
+// FP64: the Maxwellian is the cell's v_x factor (put_factors; read for the
+// whole column before the group's planes) times the row's factor of v_y and
+// v_z (one exp2 a row): one FP64 multiplication a velocity instead of an exp2.
 //
 // FP32 is bound by issue slots (70 warp instructions a velocity and 32 cells,
 // 24 of them on the half-rate ALU pipe) and by waits for planes; FP64 by the
-// FP64 pipe (two lanes a clock; 26 operations a velocity).  The form before
+// FP64 pipe (two lanes a clock; 25 operations a velocity).  The form before
 // this one (a thread per column in fixed z order, both z faces' planes read,
 // exp2 per velocity, velocity by velocity moments) took, a launch: FP32 64^3 x
 // 20^3 9.72 ms, now 7.2; 96^3 x 20^3 30.6, now 23.4; Shakhov 45 x 50 x 37 x
@@ -330,8 +329,6 @@ __global__ void __launch_bounds__(32 * warps3<T>(), 1)
         mbar_expect_tx(&full[slot], (uint32_t)(px * (a.ty + 4) * 16));
         tma_load_4d(ring + slot * PC, &tmap, &full[slot], i0 * W, j0, grp >= gpos ? z0 + o : z0 + ZC + 3 - o, grp);
     };
-    // velocities between restarts of the FP64 recurrence
-    const int rec = restart64(g.nvx);
 
     if (tid == 0) {
         for (int st = 0; st < RING; ++st) {
@@ -421,6 +418,9 @@ __global__ void __launch_bounds__(32 * warps3<T>(), 1)
     *cellw = word;
     __syncthreads();
 
+    // FP64: v_x factors of the column's first cell (of cell 0 of its plane
+    // outside the grid)
+    const double *const mx0 = F64 ? a.cf + kMxCount * nc + (long)z0 * g.nx * g.ny + (inij ? j * g.nx + i : 0) : nullptr;
     const int c0 = (ly + 2) * px + lx + 2;
     const int sz = (g.nx + 4) * (g.ny + 4);
     const int pc0 = inij ? nbr3(g, i, j, z0) : 0;
@@ -490,7 +490,7 @@ __global__ void __launch_bounds__(32 * warps3<T>(), 1)
     for (int t = 0; t < ZC; ++t) S0[t] = S1[t] = S2[t] = T(0);
     T cg[ZC];                       // FP32: the row's constant of the exponent
     T kyz[ZC], l5[ZC];              // Shakhov: the row's part of k c.q; 2 log2(A)/log2(e) - 5
-    T Mr[ZC], Rr[ZC], Er[ZC];       // FP64: recurrence, and the row's factor of v_y and v_z
+    T Er[ZC];                       // FP64: the row's factor of v_y and v_z
     VYZ3<T> cyz{};
     uint32_t keepo = 0, fullo = 0;  // cells to store / without face weights, in upwind order
     bool pz = true;
@@ -514,13 +514,6 @@ __global__ void __launch_bounds__(32 * warps3<T>(), 1)
                 if constexpr (F64) {
                     const T dy = cyz.vy - cz[kMxUy * NT], dz = cyz.vz - cz[kMxUz * NT];
                     Er[s] = exp2(-cz[kMxC2 * NT] * (dy * dy + dz * dz));
-                    const int b = xg * W / rec;
-                    Mr[s] = cz[(kMxM + b) * NT] * Er[s];
-                    Rr[s] = cz[(kMxR + b) * NT];
-                    for (int q = b * rec; q < xg * W; ++q) {   // a split that starts inside a row
-                        Mr[s] *= Rr[s];
-                        Rr[s] *= cz[kMxQ * NT];
-                    }
                 } else {
                     const float4 cv = *reinterpret_cast<const float4 *>(coef + (t * NT + tid) * 4);
                     const T dy = cyz.vy - cz[0], dz = cyz.vz - cz[NT];
@@ -533,12 +526,15 @@ __global__ void __launch_bounds__(32 * warps3<T>(), 1)
                 }
             }
             fresh = false;
-        } else if (F64 && xg * W % rec == 0) {
+        }
+        // FP64: the v_x factors of the column's cells, in upwind order
+        T fx[F64 ? ZC : 1][W];
+        if constexpr (F64) {
 #pragma unroll
             for (int s = 0; s < ZC; ++s) {
-                const T *const cz = cq + (pz ? s : ZC - 1 - s) * NCQ * NT + tid;
-                Mr[s] = cz[(kMxM + xg * W / rec) * NT] * Er[s];
-                Rr[s] = cz[(kMxR + xg * W / rec) * NT];
+                const double *const m = mx0 + min(pz ? s : ZC - 1 - s, g.nz - 1 - z0) * (long)(g.nx * g.ny) + xg * W * nc;
+#pragma unroll
+                for (int e = 0; e < W; ++e) fx[s][e] = __ldg(m + e * nc);
             }
         }
         // the rows of the x flux are read again for every cell (below)
@@ -592,15 +588,9 @@ __global__ void __launch_bounds__(32 * warps3<T>(), 1)
             ld_units(vtab + 4 * xg + 2, nnux);
             ld_units(vtab + 4 * xg + 3, kx);
             if constexpr (F64) {
-                const T *const cz = cq + t * NCQ * NT + tid;
-                const T Q = cz[kMxQ * NT];
-                r = cz[kMxRel * NT];
+                r = cq[(t * NCQ + kMxRel) * NT + tid];
 #pragma unroll
-                for (int e = 0; e < W; ++e) {
-                    feq[e] = xg * W + e < g.nvx ? Mr[s] : T(0);
-                    Mr[s] *= Rr[s];
-                    Rr[s] *= Q;
-                }
+                for (int e = 0; e < W; ++e) feq[e] = fx[s][e] * Er[s];
             } else {
                 const float4 cv = *reinterpret_cast<const float4 *>(coef + (t * NT + tid) * 4);
                 r = cv.w;
@@ -2014,7 +2004,7 @@ size_t vtab3_bytes(const dvm_ctx *c) { return (size_t)c->nvxp * 2 * c->elem + (s
 
 size_t cvinfo3_bytes() { return sizeof(CvInfo3); }
 
-size_t cf64_bytes3d(const dvm_ctx *c) { return sizeof(double) * kMxCount * (size_t)c->nc; }
+size_t cf64_bytes3d(const dvm_ctx *c) { return sizeof(double) * (kMxCount + c->nvxp) * (size_t)c->nc; }
 
 cudaError_t members3d(dvm_ctx *c)
 {
