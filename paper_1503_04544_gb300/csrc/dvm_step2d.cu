@@ -594,24 +594,14 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<T> a, const __g
                     F2 fq[2], fg[2];
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
-                        {
-                            F2 X;
-                            float x0, x1;
-                            if constexpr (MUSCL || SHAK) {
-                                // log2 M = el0 - 2 c2 |v|^2/2 + e1x vx + e1y vy
-                                X = fma2(NC2, P.ke[h], EL0);
-                                X = fma2(E1X, P.vx[h], X);
-                                X = fma2(E1Y, P.vy[h], X);
-                                f2_get(X, x0, x1);
-                                fq[h] = f2(ex2_fast(x0), ex2_fast(x1));
-                            } else {
-                                // M = A 2^(-c2 |v - u|^2): the first-order form
-                                // is bound by memory and has room for it
-                                const F2 DX = sub2(P.vx[h], f2(ux)), DY = sub2(P.vy[h], f2(uy));
-                                X = mul2(fma2(DY, DY, mul2(DX, DX)), f2(-c2));
-                                f2_get(X, x0, x1);
-                                fq[h] = mul2(f2(A), f2(ex2_fast(x0), ex2_fast(x1)));
-                            }
+                        float x0, x1;
+                        if constexpr (MUSCL) {
+                            // log2 M = el0 - 2 c2 |v|^2/2 + e1x vx + e1y vy
+                            F2 X = fma2(NC2, P.ke[h], EL0);
+                            X = fma2(E1X, P.vx[h], X);
+                            X = fma2(E1Y, P.vy[h], X);
+                            f2_get(X, x0, x1);
+                            fq[h] = f2(ex2_fast(x0), ex2_fast(x1));
                             if constexpr (SHAK) {
                                 // |c|^2/T - 4 = 2 (log2 A - log2 M) / log2 e - 4,
                                 // k c.q = kqx vx + kqy vy - (kqx ux + kqy uy);
@@ -622,6 +612,22 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<T> a, const __g
                                 const F2 MK = mul2(fq[h], KCQ);
                                 fq[h] = fma2(MK, D4, fq[h]);
                                 fg[h] = mul2(f2(gfac), fma2(MK, f2(2.f), fq[h]));
+                            }
+                        } else {
+                            // M = A 2^(-c2 |v - u|^2), subnormal factors too: the
+                            // first-order form is bound by memory and has room
+                            // for exp2f and for the terms from v - u, which
+                            // keep their digits at any u
+                            const F2 DX = sub2(P.vx[h], f2(ux)), DY = sub2(P.vy[h], f2(uy));
+                            const F2 D2 = fma2(DY, DY, mul2(DX, DX));
+                            f2_get(mul2(D2, f2(-c2)), x0, x1);
+                            fq[h] = mul2(f2(A), f2(dexp2(x0), dexp2(x1)));
+                            if constexpr (SHAK) {
+                                // f_S = M (1 + k c.q (|c|^2/T - 4)) and g_S =
+                                // T/2 M (1 + k c.q (|c|^2/T - 2))
+                                const F2 KCQ = fma2(f2(kqx), DX, mul2(f2(kqy), DY));
+                                fg[h] = mul2(mul2(f2(gfac), fq[h]), fma2(KCQ, fma2(D2, f2(iT), f2(-2.f)), f2(1.f)));
+                                fq[h] = mul2(fq[h], fma2(KCQ, fma2(D2, f2(iT), f2(-4.f)), f2(1.f)));
                             }
                         }
                     }
