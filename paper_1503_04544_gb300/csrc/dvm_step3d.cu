@@ -151,6 +151,7 @@ template <typename T> struct Bulk3Args {
 
 constexpr int kZc3 = 4;                           // z-planes per block column
 constexpr int kPlanes3 = kZc3 + 3;                // planes of a column: two upwind, the cells, one downwind
+constexpr int kFold3 = 8;                         // groups of the longest plain FP32 moment sum
 
 // Warps of the bulk kernel's block.  FP32: 16, the most that leave a thread
 // 128 registers.  FP64: 8 (shared memory of the per-cell data; the kernel is
@@ -264,7 +265,8 @@ __global__ void __launch_bounds__(128) k_cell64_3(Bulk3Args<double> a, double *c
 // as fast: one slow warp holds up its whole block at the ring.
 //
 // Moments: v_y and v_z are uniform in a row of groups, so a cell sums F,
-// v_x F and v_x^2 F over the row and forms the five moments once per row,
+// v_x F and v_x^2 F over the row and forms the five moments once per row (in
+// FP32 once per 32 velocities of a longer one, so that no plain sum is longer),
 // into compensated sums in shared memory.
 //
 // FP64: the Maxwellian is the cell's v_x factor (put_factors; read for the
@@ -729,8 +731,9 @@ __global__ void __launch_bounds__(32 * warps3<T>(), 1)
             release(gi, s + 2);
         }
         release(gi, ZC + 2);
-        // the row's moments into the compensated sums
-        if (++xg == g.nxg || gi + 1 == ngr) {
+        // the row's moments into the compensated sums, FP32 after 32
+        // velocities at the latest
+        if (++xg == g.nxg || gi + 1 == ngr || (!F64 && xg % kFold3 == 0)) {
             const T vyz2 = cyz.vy * cyz.vy + cyz.vz * cyz.vz;
 #pragma unroll
             for (int s = 0; s < ZC; ++s) {
