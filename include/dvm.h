@@ -192,7 +192,9 @@ int dvm_init_maxwellian(dvm_ctx *ctx, const double *rho, const double *ux,
                         const double *uy, const double *uz, const double *T);
 
 /* Copy a full state in or out.  bytes must equal ncell*ncomp*nv*elem.
- * on_device = 0: host pointer; 1: device pointer.  Errors: DVM_ERR_ARG. */
+ * on_device = 0: host pointer; 1: device pointer (an array on the context's
+ * device is read or written in place).  Errors: DVM_ERR_ARG (size; a device
+ * allocation that ends before the state does). */
 int dvm_set_state(dvm_ctx *ctx, const void *f, size_t bytes, int on_device);
 int dvm_get_state(dvm_ctx *ctx, void *f, size_t bytes, int on_device);
 

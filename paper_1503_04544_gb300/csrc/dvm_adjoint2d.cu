@@ -1931,8 +1931,9 @@ int drag_adjoint_t(dvm_ctx *c, int nsteps, int K, double *J, double *gTw, double
     }
     // the public-layout staging buffer of a seed or a lambda^0 that the
     // layout kernels cannot use in place
-    const bool seed_direct = seed && seed_dev && direct_access(c, seed);
-    const bool lam0_direct = lam0 && lam0_dev && direct_access(c, lam0);
+    const size_t pubb = c->state_elems * c->elem;
+    const bool seed_direct = seed && seed_dev && array_access(c, seed, pubb) == ArrayAccess::kDirect;
+    const bool lam0_direct = lam0 && lam0_dev && array_access(c, lam0, pubb) == ArrayAccess::kDirect;
     if (((seed && !seed_direct) || (lam0 && !lam0_direct)) && !c->d_pub)
         AC(cudaMalloc(&c->d_pub, c->state_elems * c->elem));
     if (seed) {

@@ -724,12 +724,20 @@ static int ensure_pub(dvm_ctx *c)
 // A device array on this context's device is converted in place; a host array
 // (or one a kernel here cannot read) passes through the staging buffer.
 
+static int short_array(const char *what)
+{
+    set_error(std::string(what) + ": the device array ends before the state does");
+    return DVM_ERR_ARG;
+}
+
 int dvm_set_state(dvm_ctx *c, const void *f, size_t bytes, int on_device)
 {
     if (!c || !f) { set_error("null"); return DVM_ERR_ARG; }
     if (split_step_open(c, "dvm_set_state")) return DVM_ERR_STATE;
     if (bytes != c->state_elems * c->elem) { set_error("state size mismatch"); return DVM_ERR_ARG; }
-    if (on_device && direct_access(c, f)) {
+    const ArrayAccess acc = on_device ? array_access(c, f, bytes) : ArrayAccess::kStaged;
+    if (acc == ArrayAccess::kShort) return short_array("dvm_set_state");
+    if (acc == ArrayAccess::kDirect) {
         CK(pack_state(c, f, c->f[c->cur]));
     } else {
         int rc = ensure_pub(c);
@@ -752,7 +760,9 @@ int dvm_get_state(dvm_ctx *c, void *f, size_t bytes, int on_device)
 {
     if (!c || !f) { set_error("null"); return DVM_ERR_ARG; }
     if (bytes != c->state_elems * c->elem) { set_error("state size mismatch"); return DVM_ERR_ARG; }
-    if (on_device && direct_access(c, f)) {
+    const ArrayAccess acc = on_device ? array_access(c, f, bytes) : ArrayAccess::kStaged;
+    if (acc == ArrayAccess::kShort) return short_array("dvm_get_state");
+    if (acc == ArrayAccess::kDirect) {
         CK(unpack_state(c, c->f[c->cur], f));
     } else {
         int rc = ensure_pub(c);
@@ -1526,6 +1536,10 @@ int dvm_adjoint(dvm_ctx *c, int nsteps, int checkpoint_every, int with_drag, con
     if (!with_drag && !seed) { set_error("dvm_adjoint: no objective (with_drag = 0 and no seed)"); return DVM_ERR_ARG; }
     int rc = adjoint_checks(c, nsteps, checkpoint_every);
     if (rc != DVM_OK) return rc;
+    const size_t bytes = c->state_elems * c->elem;
+    if (seed && seed_on_device && array_access(c, seed, bytes) == ArrayAccess::kShort) return short_array("dvm_adjoint: seed");
+    if (lambda0 && lambda0_on_device && array_access(c, lambda0, bytes) == ArrayAccess::kShort)
+        return short_array("dvm_adjoint: lambda0");
     double *gbc[4] = {gbc0, gbc1, gbc2, gbc3};
     rc = drag_adjoint2d(c, nsteps, checkpoint_every, J, gTw, gbc, gprim0, nullptr, nullptr, with_drag ? 1 : 0, seed,
                         seed_on_device, lambda0, lambda0_on_device);

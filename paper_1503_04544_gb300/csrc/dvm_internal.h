@@ -239,7 +239,8 @@ cudaError_t ghost2d(dvm_ctx *c, int side, const double *d_prim, int nside);
 cudaError_t pack_state(dvm_ctx *c, const void *pub, void *dev);      // public -> device
 cudaError_t unpack_state(dvm_ctx *c, const void *dev, void *pub);    // device -> public
 cudaError_t add_state(dvm_ctx *c, const void *pub, void *dev);       // dev += public
-bool direct_access(const dvm_ctx *c, const void *p);                 // a caller's array usable in place
+enum class ArrayAccess { kDirect, kStaged, kShort };                 // in place, by a copy, or too short
+ArrayAccess array_access(const dvm_ctx *c, const void *p, size_t bytes);   // of a caller's device array
 cudaError_t zero_solid2d(dvm_ctx *c);                            // both state buffers
 cudaError_t halo2d(dvm_ctx *c, int buf);                         // periodic / zero-gradient padding
 cudaError_t members2d(dvm_ctx *c, bool moving);                  // control-volume records

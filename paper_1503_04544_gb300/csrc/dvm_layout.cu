@@ -10,6 +10,8 @@
 // device side.  One element per thread, as before, touched 16 bytes of a
 // 32-byte sector in another slab with every fourth thread: 2D, 256^2 x 32^2
 // FP32 (0.54 GB each way) 469 us, 3D, 64^3 x 20^3 FP32 10.8 ms.
+#include <cudaTypedefs.h>
+
 #include "dvm_device.cuh"
 
 namespace dvm {
@@ -122,6 +124,17 @@ __global__ void __launch_bounds__(kLayThreads) k_layout(LayArgs a, T *pub, T *de
     }
 }
 
+// A function of the driver, or null.
+template <typename F> F driver_entry(const char *name, unsigned version)
+{
+    cudaDriverEntryPointQueryResult q;
+    void *fn = nullptr;
+    const cudaError_t e = cudaGetDriverEntryPointByVersion(name, &fn, version, cudaEnableDefault, &q);
+    if (e == cudaSuccess && q == cudaDriverEntryPointSuccess) return reinterpret_cast<F>(fn);
+    cudaGetLastError();
+    return nullptr;
+}
+
 template <typename T, LayMode MODE>
 cudaError_t layout_t(dvm_ctx *c, T *pub, T *dev)
 {
@@ -166,19 +179,46 @@ cudaError_t add_state(dvm_ctx *c, const void *pub, void *dev)
     return layout_t<double, kAddToDevice>(c, (double *)const_cast<void *>(pub), (double *)dev);
 }
 
-// Whether a kernel on this context's device may use the caller's array in
-// place: memory of this device, whole elements.  Anything else (another
-// device's memory, an odd address) goes through the staging buffer.
-bool direct_access(const dvm_ctx *c, const void *p)
+// How the kernels here may use a caller's device array of `bytes` bytes.  In
+// place: whole elements, every byte in memory of this context's device.
+// Anything else a copy can read (another device's memory, managed memory, an
+// odd address) goes through the staging buffer.  An array that runs past the
+// end of its allocation, say a tensor of one element expanded, is an error
+// here: a copy of it is refused, a kernel would fault.  In a reserved address
+// range the pieces of memory that are mapped into it are followed to the
+// array's end.
+ArrayAccess array_access(const dvm_ctx *c, const void *p, size_t bytes)
 {
-    if (reinterpret_cast<uintptr_t>(p) % c->elem != 0) return false;
-    cudaPointerAttributes at;
+    static const auto piece = driver_entry<PFN_cuMemGetAddressRange_v3020>("cuMemGetAddressRange", 3020);
+    static const auto attribute = driver_entry<PFN_cuPointerGetAttribute_v4000>("cuPointerGetAttribute", 4000);
     int dev = -1;
-    if (cudaPointerGetAttributes(&at, p) != cudaSuccess || cudaGetDevice(&dev) != cudaSuccess) {
+    if (!attribute || !piece || reinterpret_cast<uintptr_t>(p) % c->elem != 0 || cudaGetDevice(&dev) != cudaSuccess) {
+        cudaGetLastError();
+        return ArrayAccess::kStaged;
+    }
+    const auto on_device = [dev](CUdeviceptr at) {
+        cudaPointerAttributes attr;
+        if (cudaPointerGetAttributes(&attr, reinterpret_cast<const void *>(at)) == cudaSuccess)
+            return attr.type == cudaMemoryTypeDevice && attr.device == dev;
         cudaGetLastError();
         return false;
+    };
+    CUdeviceptr at = reinterpret_cast<CUdeviceptr>(p), start = 0;
+    const CUdeviceptr end = at + bytes;
+    size_t size = 0;
+    if (!on_device(at) || piece(&start, &size, at) != CUDA_SUCCESS) return ArrayAccess::kStaged;
+    if (end <= start + size) return ArrayAccess::kDirect;
+    at = start + size;
+    if (attribute(&start, CU_POINTER_ATTRIBUTE_RANGE_START_ADDR, reinterpret_cast<CUdeviceptr>(p)) != CUDA_SUCCESS ||
+        attribute(&size, CU_POINTER_ATTRIBUTE_RANGE_SIZE, reinterpret_cast<CUdeviceptr>(p)) != CUDA_SUCCESS)
+        return ArrayAccess::kStaged;
+    if (end > start + size) return ArrayAccess::kShort;
+    while (at < end) {
+        if (piece(&start, &size, at) != CUDA_SUCCESS || start + size <= at) return ArrayAccess::kShort;
+        if (!on_device(at)) return ArrayAccess::kStaged;
+        at = start + size;
     }
-    return at.type == cudaMemoryTypeDevice && at.device == dev;
+    return ArrayAccess::kDirect;
 }
 
 }  // namespace dvm
