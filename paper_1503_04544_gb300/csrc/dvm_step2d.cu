@@ -1359,14 +1359,16 @@ __global__ void __launch_bounds__(256) k_fusion(CvArgs c, T *f, T *part)
         load_info(info + item / c.S, &I);
         int v0, v1;
         split_range(c, sp, Vec<T>::W, v0, v1);
-        const double rS = 1.0 / I.Sn;    // a division per value was most of the FP64 work
+        // FP32 multiplies by 1 / S, whose rounding is far below its own (a
+        // division per value was most of the FP64 work); FP64 divides
+        const double rS = 1.0 / I.Sn;
         Acc<T> a[4];
         for (int comp = 0; comp < 2; ++comp)
             for (int p = v0 + threadIdx.x; p < v1; p += blockDim.x) {
                 const long base = ebase<T>(g, comp, p);
                 double acc = 0;
                 for (int q = 0; q < nm; ++q) acc += I.mem[q].sb * (double)f[base + I.mem[q].pc * Vec<T>::W];
-                const T fcv = (T)(acc * rS);
+                const T fcv = (T)(sizeof(T) == 4 ? acc * rS : acc / I.Sn);
                 for (int q = 0; q < nm; ++q) {
                     f[base + I.mem[q].pc * Vec<T>::W] = fcv;
                     for (int t = 0; t < 4; ++t)
