@@ -541,16 +541,20 @@ __device__ __forceinline__ void mirrors(const Grid2D &g, int i, int j, I (&m)[4]
 // k_cell64_3) for all velocity splits: an FP64 operation holds the pipe for 64
 // clocks a warp, and some 400 of them per cell (the sums of the splits, the
 // primitives, the exponentials) in every split's prologue were worth six
-// groups of velocities (31 of a 50 us launch at 32^2 x 16^2).  Eight threads
-// of a warp share a cell: each sums every eighth split, all form the
-// primitives, and the exponentials are dealt out.
+// groups of velocities (31 of a 50 us launch at 32^2 x 16^2).  CT threads of a
+// warp share a cell: each sums every CT-th split, all form the primitives, and
+// the exponentials are dealt out.  CT is 8, and 16 while the blocks that this
+// makes have an SM each (32^2 x 16^2, one exponential a thread: 721 us a pass
+// of 20 steps against 732 with 8; on more cells the primitives formed by twice
+// as many threads would cost more).
 constexpr int kCellThreads = 8;
+constexpr long kCellsFor16 = 152 * 128 / 16;
 
-// Sum over the eight threads of a cell (every thread returns it).
-__device__ __forceinline__ double cell_sum(double x)
+// Sum over the threads of a cell (every thread returns it).
+template <int CT> __device__ __forceinline__ double cell_sum(double x)
 {
 #pragma unroll
-    for (int o = kCellThreads / 2; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
+    for (int o = CT / 2; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
     return x;
 }
 
@@ -562,10 +566,11 @@ __device__ __forceinline__ double cell_sum(double x)
 // recurrence M(v + dv) = M R, R(v + dv) = R Q from a row's start took two
 // multiplications, 256^2 x 32^2 4.31 ms a launch against 4.14, and lost M
 // where it underflowed at the start of a coarse row.)
+template <int CT>
 __device__ __forceinline__ void put_factors(double *mx, long nc, int k, int nvx, int n, double vmin, double dv, double ux,
                                             double c2, double A)
 {
-    for (int v = k; v < n; v += kCellThreads) {
+    for (int v = k; v < n; v += CT) {
         const double dx = vmin + v * dv - ux;
         mx[v * nc] = v < nvx ? A * exp2(-c2 * (dx * dx)) : 0.0;
     }

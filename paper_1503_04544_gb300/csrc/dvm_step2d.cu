@@ -800,6 +800,7 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<T> a, const __g
 constexpr int kRows64 = 4;            // warps of a block
 constexpr int kZ64 = 2;               // rows of a thread
 constexpr int kStages64 = 3;
+constexpr int kFold64 = 8;            // groups of a moment sum before it joins the total
 static_assert(kRows64 * kZ64 == kRows, "the tile of the state's tensor maps");
 enum C64 { kUy = 0, kC2, kRel, kGf, kC64, kKqx = kC64, kKqy, kUx, kIT, kC64S };
 
@@ -818,23 +819,23 @@ __device__ __forceinline__ uint32_t branch_code(double m, double b)
 }
 
 // The per-cell values of k_bulk64 for the plain cells (dvm_device.cuh): the
-// slots of C64, then the v_x factors from slot kC64S on.  Block = 16 cells x
-// kCellThreads.
-template <bool SHAK> __global__ void __launch_bounds__(128) k_cell64(BulkArgs<double> a, double *cf)
+// slots of C64, then the v_x factors from slot kC64S on.  Block = 128 / CT cells
+// x CT threads.
+template <bool SHAK, int CT> __global__ void __launch_bounds__(128) k_cell64(BulkArgs<double> a, double *cf)
 {
     const Grid2D &g = a.g;
     const long nc = (long)g.nx * g.ny;
-    const long cell = (long)blockIdx.x * (128 / kCellThreads) + threadIdx.x / kCellThreads;
-    const int k = threadIdx.x % kCellThreads;
+    const long cell = (long)blockIdx.x * (128 / CT) + threadIdx.x / CT;
+    const int k = threadIdx.x % CT;
     const bool plain = cell < nc && (a.flags[cell] & kPlain);
     double s[4] = {0, 0, 0, 0};
     if (plain)
 #pragma unroll 4
-        for (int q = k; q < a.Sin; q += kCellThreads)
+        for (int q = k; q < a.Sin; q += CT)
 #pragma unroll
             for (int m = 0; m < 4; ++m) s[m] += a.pin[((long)q * 4 + m) * nc + cell];
 #pragma unroll
-    for (int m = 0; m < 4; ++m) s[m] = cell_sum(s[m]);
+    for (int m = 0; m < 4; ++m) s[m] = cell_sum<CT>(s[m]);
     if (!plain) return;
     double rho, ux, uy, tmp;
     if (!primitives<double>(g.dv, s[0], s[1], s[2], s[3], rho, ux, uy, tmp) && k == 0) atomicExch(&a.err[kErrNonphys], 1);
@@ -846,8 +847,8 @@ template <bool SHAK> __global__ void __launch_bounds__(128) k_cell64(BulkArgs<do
     }
     const double iT = 1.0 / tmp, c2 = (0.5 * kLog2e) * iT;
     double *const o = cf + cell;
-    put_factors(o + kC64S * nc, nc, k, g.nvx, g.nvx, g.vxmin, g.dvx, ux, c2, r * rho * (0.5 / kPi) * iT);
-    if (k == kCellThreads - 1) {
+    put_factors<CT>(o + kC64S * nc, nc, k, g.nvx, g.nvx, g.vxmin, g.dvx, ux, c2, r * rho * (0.5 / kPi) * iT);
+    if (k == CT - 1) {
         o[kUy * nc] = uy;
         o[kC2 * nc] = c2;
         o[kRel * nc] = r;
@@ -937,7 +938,10 @@ __global__ void __launch_bounds__(32 * kRows64, SHAK ? 2 : 3)
             if (j == g.ny - 1 && g.bc[3] == DVM_BC_ZEROGRAD) { vst<double>(d + pitch, o); vst<double>(d + 2 * pitch, o); }
         }
     };
-    double q[ZC][4];                        // moment sums of the thread's cells (physical order)
+    // moment sums of the thread's cells, over kFold64 groups, then onto the
+    // thread's values in pout, so that a sum of many velocities is one of short
+    // ones
+    double q[ZC][4];
 #pragma unroll
     for (int t = 0; t < ZC; ++t)
 #pragma unroll
@@ -958,7 +962,21 @@ __global__ void __launch_bounds__(32 * kRows64, SHAK ? 2 : 3)
     };
     if (busy) load_factors();
     bool first = true;
-    for (int it = 0; it < ngr; ++it) {
+    // the sums after the groups before n
+    const auto put_sums = [&](int n) {
+#pragma unroll
+        for (int t = 0; t < ZC; ++t) {
+            if (!(((word >> t) | (word >> (4 + t))) & 1u)) continue;
+            double *const s = a.pout + (long)split * 4 * nc + (long)(jt + t) * g.nx + i;
+#pragma unroll
+            for (int m = 0; m < 4; ++m) {
+                s[m * nc] = n <= kFold64 ? q[t][m] : s[m * nc] + q[t][m];
+                q[t][m] = 0;
+            }
+        }
+    };
+    for (int c0 = 0; c0 < ngr; c0 += kFold64, put_sums(c0))      // chunks of groups
+    for (int it = c0; it < min(c0 + kFold64, ngr); ++it) {
         if (tid == 0 && it + 1 < ngr) {
             // the next group into the slot that group it - 2 left
             if (it + 1 >= NST)
@@ -1161,13 +1179,7 @@ __global__ void __launch_bounds__(32 * kRows64, SHAK ? 2 : 3)
         mbar_arrive_if(smem_u32(&empty[it % NST]), tx == 0);
     }
     if (bad) atomicExch(&a.err[kErrTimeout], 1);
-#pragma unroll
-    for (int t = 0; t < ZC; ++t) {
-        if (!(((word >> t) | (word >> (4 + t))) & 1u)) continue;
-        const long cell = (long)(jt + t) * g.nx + i;
-#pragma unroll
-        for (int m = 0; m < 4; ++m) a.pout[((long)split * 4 + m) * nc + cell] = q[t][m];
-    }
+    if (ngr == 0) put_sums(0);
 }
 
 // ------------------------------------------------------------ control volumes
@@ -2248,8 +2260,10 @@ cudaError_t launch_bulk(dvm_ctx *c, const BulkArgs<T> &a)
     using K = BulkKernel<MUSCL, REC, SHAK>;
     constexpr size_t smem = sizeof(T) == 4 ? K::smem32 : K::smem64;
     if constexpr (sizeof(T) == 8) {
-        constexpr int cells = 128 / kCellThreads;
-        k_cell64<SHAK><<<(unsigned)((c->nc + cells - 1) / cells), 128, 0, c->stream>>>(a, c->cf64);
+        if (c->nc <= kCellsFor16)
+            k_cell64<SHAK, 16><<<nblk(c->nc, 128 / 16), 128, 0, c->stream>>>(a, c->cf64);
+        else
+            k_cell64<SHAK, kCellThreads><<<nblk(c->nc, 128 / kCellThreads), 128, 0, c->stream>>>(a, c->cf64);
         c->launches += 1;
     }
     const auto kernel = [] {

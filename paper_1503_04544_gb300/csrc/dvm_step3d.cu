@@ -151,7 +151,7 @@ template <typename T> struct Bulk3Args {
 
 constexpr int kZc3 = 4;                           // z-planes per block column
 constexpr int kPlanes3 = kZc3 + 3;                // planes of a column: two upwind, the cells, one downwind
-constexpr int kFold3 = 8;                         // groups of the longest plain FP32 moment sum
+constexpr int kFold3 = 8;                         // groups of the longest plain moment sum
 
 // Warps of the bulk kernel's block.  FP32: 16, the most that leave a thread
 // 128 registers.  FP64: 8 (shared memory of the per-cell data; the kernel is
@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(128) k_cell64_3(Bulk3Args<double> a, double *c
 #pragma unroll
             for (int m = 0; m < 5; ++m) s[m] += a.pin[((long)q * 5 + m) * nc + cell];
 #pragma unroll
-    for (int m = 0; m < 5; ++m) s[m] = cell_sum(s[m]);
+    for (int m = 0; m < 5; ++m) s[m] = cell_sum<kCellThreads>(s[m]);
     if (!plain) return;
     double rho, ux, uy, uz, tmp;
     if (!primitives3<double>(g.dv, s, rho, ux, uy, uz, tmp) && k == 0) atomicExch(&a.err[kErrNonphys], 1);
@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(128) k_cell64_3(Bulk3Args<double> a, double *c
     }
     const double c2 = (0.5 * kLog2e) / tmp;
     double *const o = cf + cell;
-    put_factors(o + kMxCount * nc, nc, k, g.nvx, g.nvxp, g.vxmin, g.dvx, ux, c2, r * rho * norm3(tmp));
+    put_factors<kCellThreads>(o + kMxCount * nc, nc, k, g.nvx, g.nvxp, g.vxmin, g.dvx, ux, c2, r * rho * norm3(tmp));
     if (k == kCellThreads - 1) {
         o[kMxUy * nc] = uy;
         o[kMxUz * nc] = uz;
@@ -265,9 +265,9 @@ __global__ void __launch_bounds__(128) k_cell64_3(Bulk3Args<double> a, double *c
 // as fast: one slow warp holds up its whole block at the ring.
 //
 // Moments: v_y and v_z are uniform in a row of groups, so a cell sums F,
-// v_x F and v_x^2 F over the row and forms the five moments once per row (in
-// FP32 once per 32 velocities of a longer one, so that no plain sum is longer),
-// into compensated sums in shared memory.
+// v_x F and v_x^2 F over the row and forms the five moments once per row (once
+// per eight groups of a longer one, so that no plain sum is longer), into sums
+// in shared memory, compensated in FP32.
 //
 // FP64: the Maxwellian is the cell's v_x factor (put_factors; read for the
 // whole column before the group's planes) times the row's factor of v_y and
@@ -731,9 +731,8 @@ __global__ void __launch_bounds__(32 * warps3<T>(), 1)
             release(gi, s + 2);
         }
         release(gi, ZC + 2);
-        // the row's moments into the compensated sums, FP32 after 32
-        // velocities at the latest
-        if (++xg == g.nxg || gi + 1 == ngr || (!F64 && xg % kFold3 == 0)) {
+        // the row's moments into the sums, after kFold3 groups at the latest
+        if (++xg == g.nxg || gi + 1 == ngr || xg % kFold3 == 0) {
             const T vyz2 = cyz.vy * cyz.vy + cyz.vz * cyz.vz;
 #pragma unroll
             for (int s = 0; s < ZC; ++s) {
