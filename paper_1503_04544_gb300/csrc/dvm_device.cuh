@@ -209,24 +209,10 @@ __device__ __forceinline__ double minmod3(double a, double b)
     return (ia ^ ib) < 0 ? 0.0 : __longlong_as_double(r);
 }
 
-// The two limiter values of one axis that share the difference a: the
-// downwind face minmod(b, a) and the upwind face minmod(a, c) (exact: each
-// is one of its arguments or zero).
-__device__ __forceinline__ void minmod_pair(float b, float a, float c, float &mo, float &mi)
-{
-    // magnitudes (see minmod_mag_pair); both values carry the sign of a
-    mo = xorsign(fmaxf(min_xorsign_abs(b, a), 0.f), a);
-    mi = xorsign(fmaxf(min_xorsign_abs(a, c), 0.f), a);
-}
-__device__ __forceinline__ void minmod_pair(double b, double a, double c, double &mo, double &mi)
-{
-    mo = minmod3(b, a);
-    mi = minmod3(a, c);
-}
-
-// Magnitudes of the two limiter values of minmod_pair: |minmod(b, a)| =
-// max(min_xorsign_abs(b, a), 0) and |minmod(a, c)| likewise.  Both limiter
-// values, where not zero, have the sign of a.
+// Magnitudes of the two limiter values of one axis that share the difference
+// a, the downwind face's |minmod(b, a)| = max(min_xorsign_abs(b, a), 0) and the
+// upwind face's |minmod(a, c)| likewise.  Both limiter values, where not zero,
+// have the sign of a.
 __device__ __forceinline__ void minmod_mag_pair(float b, float a, float c, float &mo, float &mi)
 {
     mo = fmaxf(min_xorsign_abs(b, a), 0.f);

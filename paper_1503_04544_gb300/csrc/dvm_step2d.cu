@@ -88,88 +88,53 @@ constexpr int kStageBytes = 2 * kTileY * kTileX * 16;     // both components of 
 // discrete adjoint): 1 when minmod returned its first argument a (the
 // downwind difference), 2 when it returned the second b (the upwind
 // difference; also on a tie), 0 when it returned 0 or the face is first order.
-template <typename T>
-__device__ __forceinline__ uint32_t branch_bits(T m, T a, T b, T w)
+__device__ __forceinline__ uint32_t branch_bits(float m, float a, float b, float w)
 {
-    return (w == T(0) || m == T(0)) ? 0u : (m == b ? 2u : (m == a ? 1u : 0u));
+    return (w == 0.f || m == 0.f) ? 0u : (m == b ? 2u : (m == a ? 1u : 0u));
 }
 
 // Update of one component of one velocity group for the thread's cell from
 // the shared-memory tile (Eq. ExSchemeDD on a full gas cell, fluxes of Eq.
-// FluxDD in difference form with the limited reconstruction), moment sums.
-// c0 is the tile index of the cell; ux1/uy1 the tile offsets of one cell step
-// towards the upwind side along x/y (sign-uniform groups), else per element.
-// With REC the branches of the two downwind faces are or-ed into bw at bit
-// ((COMP * 2 + axis) * W + e) * 2.
-template <typename T, bool MUSCL, int COMP, bool UNIFORM, bool REC>
-__device__ __forceinline__ void bulk_tile(const typename Vec<T>::type *t, int c0, int ux1, int uy1,
-                                          const T (&vx)[Vec<T>::W], const T (&vy)[Vec<T>::W],
-                                          const T (&nux)[Vec<T>::W], const T (&nuy)[Vec<T>::W],
-                                          const T (&feq)[Vec<T>::W], T wxm, T wxp, T wym, T wyp, T r,
-                                          T (&out)[Vec<T>::W], T &q0, T &q1, T &q2, T &q3, uint32_t &bw)
+// FluxDD in difference form with the limited reconstruction), moment sums; for
+// the groups whose v_x or v_y changes sign, velocity by velocity.  c0 is the
+// tile index of the cell.  With REC the branches of the two downwind faces are
+// or-ed into bw at bit ((COMP * 2 + axis) * 4 + e) * 2.
+template <bool MUSCL, int COMP, bool REC>
+__device__ __forceinline__ void bulk_tile(const float4 *t, int c0, const float (&vx)[4], const float (&vy)[4],
+                                          const float (&nux)[4], const float (&nuy)[4], const float (&feq)[4], float wxm,
+                                          float wxp, float wym, float wyp, float r, float (&out)[4], float &q0, float &q1,
+                                          float &q2, float &q3, uint32_t &bw)
 {
-    constexpr int W = Vec<T>::W;
-    T f[W];
-    sld<T>(t + c0, f);
-    if (UNIFORM) {
-        T u1[W], w1[W], d1[W], u2[W], e1[W], w2[W];
-        sld<T>(t + c0 - ux1, u1);
-        sld<T>(t + c0 - uy1, w1);
-        if (MUSCL) {
-            sld<T>(t + c0 + ux1, d1);
-            sld<T>(t + c0 - 2 * ux1, u2);
-            sld<T>(t + c0 + uy1, e1);
-            sld<T>(t + c0 - 2 * uy1, w2);
-        }
-        const bool px = ux1 > 0, py = uy1 > 0;
-        const T cxo = px ? wxp : wxm, cxi = px ? wxm : wxp;
-        const T cyo = py ? wyp : wym, cyi = py ? wym : wyp;
+    constexpr int W = 4;
+    float f[W], xm[W], xp[W], ym[W], yp[W], xm2[W], xp2[W], ym2[W], yp2[W];
+    sld<float>(t + c0, f);
+    sld<float>(t + c0 - 1, xm); sld<float>(t + c0 + 1, xp);
+    sld<float>(t + c0 - kTileX, ym); sld<float>(t + c0 + kTileX, yp);
+    if (MUSCL) {
+        sld<float>(t + c0 - 2, xm2); sld<float>(t + c0 + 2, xp2);
+        sld<float>(t + c0 - 2 * kTileX, ym2); sld<float>(t + c0 + 2 * kTileX, yp2);
+    }
 #pragma unroll
-        for (int e = 0; e < W; ++e) {
-            const T ax = f[e] - u1[e], ay = f[e] - w1[e];
-            T dfx = ax, dfy = ay;
-            if (MUSCL) {
-                const T bx = d1[e] - f[e], by = e1[e] - f[e], cx = u1[e] - u2[e], cy = w1[e] - w2[e];
-                const T mxo = minmod3(bx, ax), myo = minmod3(by, ay), mxi = minmod3(ax, cx), myi = minmod3(ay, cy);
-                dfx += (T(1) - nux[e]) * (cxo * mxo - cxi * mxi);
-                dfy += (T(1) - nuy[e]) * (cyo * myo - cyi * myi);
-                if (REC) {
-                    bw |= branch_bits(mxo, bx, ax, cxo) << (((COMP * 2 + 0) * W + e) * 2);
-                    bw |= branch_bits(myo, by, ay, cyo) << (((COMP * 2 + 1) * W + e) * 2);
-                }
-            }
-            out[e] = f[e] - nux[e] * dfx - nuy[e] * dfy + r * (feq[e] - f[e]);
-        }
-    } else {
-        T xm[W], xp[W], ym[W], yp[W], xm2[W], xp2[W], ym2[W], yp2[W];
-        sld<T>(t + c0 - 1, xm); sld<T>(t + c0 + 1, xp);
-        sld<T>(t + c0 - kTileX, ym); sld<T>(t + c0 + kTileX, yp);
+    for (int e = 0; e < W; ++e) {
+        const bool px = vx[e] >= 0.f, py = vy[e] >= 0.f;
+        const float u1 = px ? xm[e] : xp[e], w1 = py ? ym[e] : yp[e];
+        const float ax = f[e] - u1, ay = f[e] - w1;
+        float dfx = ax, dfy = ay;
         if (MUSCL) {
-            sld<T>(t + c0 - 2, xm2); sld<T>(t + c0 + 2, xp2);
-            sld<T>(t + c0 - 2 * kTileX, ym2); sld<T>(t + c0 + 2 * kTileX, yp2);
-        }
-#pragma unroll
-        for (int e = 0; e < W; ++e) {
-            const bool px = vx[e] >= T(0), py = vy[e] >= T(0);
-            const T u1 = px ? xm[e] : xp[e], w1 = py ? ym[e] : yp[e];
-            const T ax = f[e] - u1, ay = f[e] - w1;
-            T dfx = ax, dfy = ay;
-            if (MUSCL) {
-                const T d1 = px ? xp[e] : xm[e], u2 = px ? xm2[e] : xp2[e];
-                const T e1 = py ? yp[e] : ym[e], w2 = py ? ym2[e] : yp2[e];
-                const T cxo = px ? wxp : wxm, cxi = px ? wxm : wxp;
-                const T cyo = py ? wyp : wym, cyi = py ? wym : wyp;
-                const T bx = d1 - f[e], by = e1 - f[e], cx = u1 - u2, cy = w1 - w2;
-                const T mxo = minmod3(bx, ax), myo = minmod3(by, ay), mxi = minmod3(ax, cx), myi = minmod3(ay, cy);
-                dfx += (T(1) - nux[e]) * (cxo * mxo - cxi * mxi);
-                dfy += (T(1) - nuy[e]) * (cyo * myo - cyi * myi);
-                if (REC) {
-                    bw |= branch_bits(mxo, bx, ax, cxo) << (((COMP * 2 + 0) * W + e) * 2);
-                    bw |= branch_bits(myo, by, ay, cyo) << (((COMP * 2 + 1) * W + e) * 2);
-                }
+            const float d1 = px ? xp[e] : xm[e], u2 = px ? xm2[e] : xp2[e];
+            const float e1 = py ? yp[e] : ym[e], w2 = py ? ym2[e] : yp2[e];
+            const float cxo = px ? wxp : wxm, cxi = px ? wxm : wxp;
+            const float cyo = py ? wyp : wym, cyi = py ? wym : wyp;
+            const float bx = d1 - f[e], by = e1 - f[e], cx = u1 - u2, cy = w1 - w2;
+            const float mxo = minmod3(bx, ax), myo = minmod3(by, ay), mxi = minmod3(ax, cx), myi = minmod3(ay, cy);
+            dfx += (1.f - nux[e]) * (cxo * mxo - cxi * mxi);
+            dfy += (1.f - nuy[e]) * (cyo * myo - cyi * myi);
+            if (REC) {
+                bw |= branch_bits(mxo, bx, ax, cxo) << (((COMP * 2 + 0) * W + e) * 2);
+                bw |= branch_bits(myo, by, ay, cyo) << (((COMP * 2 + 1) * W + e) * 2);
             }
-            out[e] = f[e] - nux[e] * dfx - nuy[e] * dfy + r * (feq[e] - f[e]);
         }
+        out[e] = f[e] - nux[e] * dfx - nuy[e] * dfy + r * (feq[e] - f[e]);
     }
 #pragma unroll
     for (int e = 0; e < W; ++e) {
@@ -177,7 +142,7 @@ __device__ __forceinline__ void bulk_tile(const typename Vec<T>::type *t, int c0
             q0 += out[e];
             q1 += vx[e] * out[e];
             q2 += vy[e] * out[e];
-            q3 += T(0.5) * (vx[e] * vx[e] + vy[e] * vy[e]) * out[e];
+            q3 += 0.5f * (vx[e] * vx[e] + vy[e] * vy[e]) * out[e];
         } else {
             q3 += out[e];
         }
@@ -291,8 +256,7 @@ __device__ __forceinline__ void bulk_tile_up_x2(const float4 *t, int c0, int ux1
 }
 
 // Adds the two lanes of each packed moment sum to q0..q3 and clears them.
-template <typename T>
-__device__ __forceinline__ void fold_pairs(F2 (&Q)[4], T &q0, T &q1, T &q2, T &q3)
+__device__ __forceinline__ void fold_pairs(F2 (&Q)[4], float &q0, float &q1, float &q2, float &q3)
 {
     float a, b;
     f2_get(Q[0], a, b); q0 += a + b;
@@ -419,20 +383,15 @@ __device__ __forceinline__ void store_cell(typename Vec<T>::type *slab, int pc, 
 // (|c|^2/T - 2)], k = (1 - Pr) / (5 rho T^2), with the heat flux q of the
 // cell at t^n: from the raw moments of f^n that the previous step left in
 // hin (shifted to the cell's velocity, see hmom_x2), or from k_heatflux when
-// hin is null.  The FP32 variant leaves the raw moments of f^{n+1} about the
-// origin in hout for the next step.
-template <typename T, bool MUSCL, bool REC, bool SHAK>
-__global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<T> a, const __grid_constant__ CUtensorMap tmap)
+// hin is null.  It leaves the raw moments of f^{n+1} about the origin in hout
+// for the next step.  (The FP64 kernel does not: bound by the FP64 pipe, it
+// loses less by one more read of f^n in k_heatflux than by these sums.)
+template <bool MUSCL, bool REC, bool SHAK>
+__global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<float> a, const __grid_constant__ CUtensorMap tmap)
 {
-    constexpr int W = Vec<T>::W;
-    // FP32 only (FP64: k_bulk64).  The Shakhov variant leaves raw heat-flux
-    // moments of the new state; an FP64 step is bound by the FP64 pipe, where
-    // one more read of f^n by k_heatflux costs less than these sums.
-    static_assert(sizeof(T) == 4, "the FP32 bulk kernel");
-    constexpr bool HRAW = SHAK;
-    using V = typename Vec<T>::type;
+    constexpr int W = 4;
     extern __shared__ __align__(128) unsigned char smem[];
-    V *ring = reinterpret_cast<V *>(smem);
+    float4 *ring = reinterpret_cast<float4 *>(smem);
     const float4 *const tab = reinterpret_cast<const float4 *>(smem + kStages * kStageBytes);   // [kStages][kTabRows]
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + kStages * (kStageBytes + kTabBytes));
     uint64_t *empty = full + kStages;
@@ -450,7 +409,7 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<T> a, const __g
     const int ngr = max(g1 - g0, 0);
     const uint8_t fl = inside ? a.flags[cell] : 0;
     const bool plain = (fl & kPlain) != 0, zero = (fl & kZero) != 0;
-    V *fout = reinterpret_cast<V *>(a.fout);
+    float4 *fout = reinterpret_cast<float4 *>(a.fout);
 
     // tile and coefficients of group n of the split into its stage
     const auto load_group = [&](int n) {
@@ -469,64 +428,64 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<T> a, const __g
     }
 
     // equilibrium of the cell at t^n
-    T A = 0, c2 = 0, r = 0, gfac = 0, ux = 0, uy = 0, el0 = 0, e1x = 0, e1y = 0;
-    T kqx = 0, kqy = 0, iT = 0, l2a4 = 0, nkuq = 0;  // Shakhov: k q_x, k q_y, 1/T, 2 log2(A)/log2(e) - 4, -k u.q
+    float A = 0, c2 = 0, r = 0, gfac = 0, ux = 0, uy = 0, el0 = 0, e1x = 0, e1y = 0;
+    float kqx = 0, kqy = 0, iT = 0, l2a4 = 0, nkuq = 0;  // Shakhov: k q_x, k q_y, 1/T, 2 log2(A)/log2(e) - 4, -k u.q
     if (plain) {
-        T s[4];
+        float s[4];
         gather_partials(a.pin, a.Sin, nc, cell, s);
-        T rho, tmp;
-        if (!primitives<T>(pick<T>(g.dv_f, g.dv), s[0], s[1], s[2], s[3], rho, ux, uy, tmp))
+        float rho, tmp;
+        if (!primitives<float>(g.dv_f, s[0], s[1], s[2], s[3], rho, ux, uy, tmp))
             atomicExch(&a.err[kErrNonphys], 1);
-        r = pick<T>(g.dt_tau0_f, g.dt_tau0) * rho;
+        r = g.dt_tau0_f * rho;
         if (a.eqp) {
             // conservative equilibrium (Sec. 3.1): tau from the direct
             // density, the Maxwellian from the Newton parameters
             rho = a.eqp[cell]; ux = a.eqp[nc + cell]; uy = a.eqp[2 * nc + cell]; tmp = a.eqp[3 * nc + cell];
         }
-        A = rho / (T(2.0 * kPi) * tmp);
-        c2 = T(kLog2e) / (T(2) * tmp);
-        gfac = tmp / T(2);
+        A = rho / (float(2.0 * kPi) * tmp);
+        c2 = float(kLog2e) / (2.f * tmp);
+        gfac = tmp / 2.f;
         if constexpr (SHAK) {
-            T qx = 0, qy = 0;
-            if (HRAW && a.hin) {
+            float qx = 0, qy = 0;
+            if (a.hin) {
                 // heat flux at t^n from the raw moments of f^n that the
                 // previous step wrote, about their reference velocity u_r
                 // (the origin, or the control volume's velocity at t^{n-1}
                 // for cells that k_special wrote): w = u - u_r and
                 // E' = sum (|v - u_r|^2/2 f + g)
-                Acc<T> h[5];
+                Acc<float> h[5];
                 for (int sp = 0; sp < a.S; ++sp)
 #pragma unroll
-                    for (int m = 0; m < 5; ++m) h[m].merge(a.hin[((long)sp * 5 + m) * nc + cell], T(0));
+                    for (int m = 0; m < 5; ++m) h[m].merge(a.hin[((long)sp * 5 + m) * nc + cell], 0.f);
                 const long ur = (long)a.S * 5 * nc + cell;
-                const T urx = a.hin[ur], ury = a.hin[ur + nc];
-                const T wx = ux - urx, wy = uy - ury;
-                const T e1 = s[3] - urx * s[1] - ury * s[2] + T(0.5) * (urx * urx + ury * ury) * s[0];
-                const T rw2 = s[0] * (wx * wx + wy * wy);
-                const T dv = pick<T>(g.dv_f, g.dv);
+                const float urx = a.hin[ur], ury = a.hin[ur + nc];
+                const float wx = ux - urx, wy = uy - ury;
+                const float e1 = s[3] - urx * s[1] - ury * s[2] + 0.5f * (urx * urx + ury * ury) * s[0];
+                const float rw2 = s[0] * (wx * wx + wy * wy);
+                const float dv = g.dv_f;
                 qx = dv * (h[0].value() - wx * h[2].value() - wy * h[3].value() - wx * e1 + wx * rw2);
                 qy = dv * (h[1].value() - wx * h[3].value() - wy * h[4].value() - wy * e1 + wy * rw2);
             } else {
                 qx = a.qh[cell];
                 qy = a.qh[nc + cell];
             }
-            const T k = a.pr1 / (T(5) * rho * tmp * tmp);
+            const float k = a.pr1 / (5.f * rho * tmp * tmp);
             kqx = k * qx;
             kqy = k * qy;
-            iT = T(1) / tmp;
-            l2a4 = T(2.0 / kLog2e) * log2(A) - T(4);
+            iT = 1.f / tmp;
+            l2a4 = float(2.0 / kLog2e) * log2(A) - 4.f;
             nkuq = -(kqx * ux + kqy * uy);
         }
         // log2 M(v) = el0 + e1x vx + e1y vy - c2 |v|^2 (packed path)
         el0 = log2(A) - c2 * (ux * ux + uy * uy);
-        e1x = T(2) * c2 * ux;
-        e1y = T(2) * c2 * uy;
+        e1x = 2.f * c2 * ux;
+        e1y = 2.f * c2 * uy;
     }
     const int mask = fl >> kMaskShift;
     // limiter weights of the faces x-, x+, y-, y+ (1/2 where the limited
     // reconstruction is allowed, 0 where the flux falls back to first order)
-    const T wxm = (mask & 1) ? T(0.5) : T(0), wxp = (mask & 2) ? T(0.5) : T(0);
-    const T wym = (mask & 4) ? T(0.5) : T(0), wyp = (mask & 8) ? T(0.5) : T(0);
+    const float wxm = (mask & 1) ? 0.5f : 0.f, wxp = (mask & 2) ? 0.5f : 0.f;
+    const float wym = (mask & 4) ? 0.5f : 0.f, wyp = (mask & 8) ? 0.5f : 0.f;
     const int c0 = (ty + 2) * kTileX + tx + 2;
     int mir[4];               // padded indices fit in 32 bits (checked at context creation)
     mirrors(g, i, j, mir);
@@ -538,8 +497,8 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<T> a, const __g
     {
         EL0 = f2(el0); E1X = f2(e1x); E1Y = f2(e1y); NC2 = f2(-2.f * c2);
     }
-    Acc<T> m0, m1, m2, m3;
-    T q0 = 0, q1 = 0, q2 = 0, q3 = 0;
+    Acc<float> m0, m1, m2, m3;
+    float q0 = 0, q1 = 0, q2 = 0, q3 = 0;
     F2 Qp[4];                 // per-lane sums of the packed FP32 path
 #pragma unroll
     for (int m = 0; m < 4; ++m) Qp[m] = f2(0.f);
@@ -550,7 +509,7 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<T> a, const __g
 #pragma unroll
     for (int m = 0; m < 5; ++m) Hp[m] = f2(0.f);
     float *sacc = reinterpret_cast<float *>(smem + kStages * (kStageBytes + kTabBytes) + 2 * kStages * sizeof(uint64_t));
-    if constexpr (HRAW) {
+    if constexpr (SHAK) {
 #pragma unroll
         for (int m = 0; m < 2 * kSaccRows; ++m) sacc[m * 32 * kRows + tid] = 0;
     }
@@ -564,18 +523,18 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<T> a, const __g
             load_group(k);
         }
         if (!mbar_wait(&full[st], (uint32_t)((it / kStages) & 1))) atomicExch(&a.err[kErrTimeout], 1);
-        const V *tile = ring + (long)st * (kStageBytes / 16);
-        V *o0 = fout + (long)q * 2 * g.slab;
+        const float4 *tile = ring + (long)st * (kStageBytes / 16);
+        float4 *o0 = fout + (long)q * 2 * g.slab;
         if (plain) {
             const ulonglong2 *const pt = reinterpret_cast<const ulonglong2 *>(tab + st * kTabRows);
             const int2 sg = *reinterpret_cast<const int2 *>(pt + 7);
             const int sx = sg.x, sy = sg.y;
-            T vx[W], vy[W], nux[W], nuy[W], feq[W], out[W];
+            float vx[W], vy[W], nux[W], nuy[W], feq[W], out[W];
             uint32_t bw = 0;
             // the FP32 Shakhov variant keeps every moment sum in the per-lane
             // pairs: the scalar path's sums of this group go there at its end
-            T t0 = 0, t1 = 0, t2 = 0, t3 = 0;
-            T &p0 = sel<HRAW>(t0, q0), &p1 = sel<HRAW>(t1, q1), &p2 = sel<HRAW>(t2, q2), &p3 = sel<HRAW>(t3, q3);
+            float t0 = 0, t1 = 0, t2 = 0, t3 = 0;
+            float &p0 = sel<SHAK>(t0, q0), &p1 = sel<SHAK>(t1, q1), &p2 = sel<SHAK>(t2, q2), &p3 = sel<SHAK>(t3, q3);
             {
                 if (sx != 0 && sy != 0) {
                     // packed FP32 path of the sign-uniform groups, coefficients
@@ -636,7 +595,7 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<T> a, const __g
                         bulk_tile_x2<0, REC>(tile, c0, ux1, uy1, P, fq, wxm, wxp, wym, wyp, r2, out, Qp, bw);
                     else
                         bulk_tile_up_x2<0>(tile, c0, ux1, uy1, P, fq, r2, out, Qp);
-                    store_cell<T>(o0, pc, mir, anymir, out);
+                    store_cell<float>(o0, pc, mir, anymir, out);
                     if constexpr (SHAK) {
                         hmom_x2<0>(f2(out[0], out[1]), P.vx[0], P.vy[0], P.ke[0], Hp);
                         hmom_x2<0>(f2(out[2], out[3]), P.vx[1], P.vy[1], P.ke[1], Hp);
@@ -652,7 +611,7 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<T> a, const __g
                                              Qp, bw);
                     else
                         bulk_tile_up_x2<1>(tile + kTileY * kTileX, c0, ux1, uy1, P, fq, r2, out, Qp);
-                    store_cell<T>(o0 + g.slab, pc, mir, anymir, out);
+                    store_cell<float>(o0 + g.slab, pc, mir, anymir, out);
                     if constexpr (SHAK) {
                         hmom_x2<1>(f2(out[0], out[1]), P.vx[0], P.vy[0], P.ke[0], Hp);
                         hmom_x2<1>(f2(out[2], out[3]), P.vx[1], P.vy[1], P.ke[1], Hp);
@@ -662,55 +621,39 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<T> a, const __g
             }
 #pragma unroll
             for (int e = 0; e < W; ++e) {
-                const VCoef<T> vc = ld_coef(a.vt + q * W + e);
+                const VCoef<float> vc = ld_coef(a.vt + q * W + e);
                 vx[e] = vc.vx; vy[e] = vc.vy; nux[e] = vc.nux; nuy[e] = vc.nuy;
             }
 #pragma unroll
             for (int e = 0; e < W; ++e) {
-                const T dx = vx[e] - ux, dy = vy[e] - uy;
+                const float dx = vx[e] - ux, dy = vy[e] - uy;
                 feq[e] = A * dexp2(-(dx * dx + dy * dy) * c2);
             }
             // Shakhov: the equilibria of f and g (the BGK g equilibrium T/2 M
             // is formed in place after the f update)
-            T feqg[W];
+            float feqg[W];
             if constexpr (SHAK) {
 #pragma unroll
                 for (int e = 0; e < W; ++e) {
-                    const T dx = vx[e] - ux, dy = vy[e] - uy;
-                    const T kcq = kqx * dx + kqy * dy, d2 = (dx * dx + dy * dy) * iT;
-                    feqg[e] = gfac * feq[e] * fma(kcq, d2 - T(2), T(1));
-                    feq[e] *= fma(kcq, d2 - T(4), T(1));
+                    const float dx = vx[e] - ux, dy = vy[e] - uy;
+                    const float kcq = kqx * dx + kqy * dy, d2 = (dx * dx + dy * dy) * iT;
+                    feqg[e] = gfac * feq[e] * fma(kcq, d2 - 2.f, 1.f);
+                    feq[e] *= fma(kcq, d2 - 4.f, 1.f);
                 }
             }
-            if (sx != 0 && sy != 0) {
-                const int ux1 = sx > 0 ? 1 : -1, uy1 = sy > 0 ? kTileX : -kTileX;
-                bulk_tile<T, MUSCL, 0, true, REC>(tile, c0, ux1, uy1, vx, vy, nux, nuy, feq, wxm, wxp, wym, wyp, r,
-                                                  out, p0, p1, p2, p3, bw);
-                store_cell<T>(o0, pc, mir, anymir, out);
-                if constexpr (HRAW) hmom_group<0>(out, vx, vy, Hp);
-                if constexpr (!SHAK) {
-#pragma unroll
-                    for (int e = 0; e < W; ++e) feqg[e] = feq[e] * gfac;
-                }
-                bulk_tile<T, MUSCL, 1, true, REC>(tile + kTileY * kTileX, c0, ux1, uy1, vx, vy, nux, nuy, feqg, wxm,
-                                                  wxp, wym, wyp, r, out, p0, p1, p2, p3, bw);
-                store_cell<T>(o0 + g.slab, pc, mir, anymir, out);
-                if constexpr (HRAW) hmom_group<1>(out, vx, vy, Hp);
+            bulk_tile<MUSCL, 0, REC>(tile, c0, vx, vy, nux, nuy, feq, wxm, wxp, wym, wyp, r, out, p0, p1, p2, p3, bw);
+            store_cell<float>(o0, pc, mir, anymir, out);
+            if constexpr (SHAK) {
+                hmom_group<0>(out, vx, vy, Hp);
             } else {
-                bulk_tile<T, MUSCL, 0, false, REC>(tile, c0, 1, kTileX, vx, vy, nux, nuy, feq, wxm, wxp, wym, wyp, r,
-                                                   out, p0, p1, p2, p3, bw);
-                store_cell<T>(o0, pc, mir, anymir, out);
-                if constexpr (HRAW) hmom_group<0>(out, vx, vy, Hp);
-                if constexpr (!SHAK) {
 #pragma unroll
-                    for (int e = 0; e < W; ++e) feqg[e] = feq[e] * gfac;
-                }
-                bulk_tile<T, MUSCL, 1, false, REC>(tile + kTileY * kTileX, c0, 1, kTileX, vx, vy, nux, nuy, feqg,
-                                                   wxm, wxp, wym, wyp, r, out, p0, p1, p2, p3, bw);
-                store_cell<T>(o0 + g.slab, pc, mir, anymir, out);
-                if constexpr (HRAW) hmom_group<1>(out, vx, vy, Hp);
+                for (int e = 0; e < W; ++e) feqg[e] = feq[e] * gfac;
             }
-            if constexpr (HRAW) {
+            bulk_tile<MUSCL, 1, REC>(tile + kTileY * kTileX, c0, vx, vy, nux, nuy, feqg, wxm, wxp, wym, wyp, r, out, p0, p1,
+                                     p2, p3, bw);
+            store_cell<float>(o0 + g.slab, pc, mir, anymir, out);
+            if constexpr (SHAK) hmom_group<1>(out, vx, vy, Hp);
+            if constexpr (SHAK) {
                 Qp[0] = add2(Qp[0], f2(t0, 0.f)); Qp[1] = add2(Qp[1], f2(t1, 0.f));
                 Qp[2] = add2(Qp[2], f2(t2, 0.f)); Qp[3] = add2(Qp[3], f2(t3, 0.f));
             }
@@ -718,8 +661,8 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<T> a, const __g
             if (REC) a.bits[(long)q * a.bslab + (long)(j + 2) * a.bpitch + i + 2] = bw;
             // fold the plain sums of 8 groups (16 in the FP32 Shakhov variant)
             // into the compensated sums
-            if (++fold == (HRAW ? 16 : 8)) {
-                if constexpr (HRAW) {
+            if (++fold == (SHAK ? 16 : 8)) {
+                if constexpr (SHAK) {
                     fold_lanes<4>(Qp, 0, sacc, tid);
                     fold_lanes<5>(Hp, 4, sacc, tid);
                 } else {
@@ -730,11 +673,11 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<T> a, const __g
                 fold = 0;
             }
         } else if (zero) {
-            T z[W];
+            float z[W];
 #pragma unroll
             for (int e = 0; e < W; ++e) z[e] = 0;
-            store_cell<T>(o0, pc, mir, anymir, z);
-            store_cell<T>(o0 + g.slab, pc, mir, anymir, z);
+            store_cell<float>(o0, pc, mir, anymir, z);
+            store_cell<float>(o0 + g.slab, pc, mir, anymir, z);
         }
         __syncwarp();
         if (tx == 0) mbar_arrive(&empty[st]);
@@ -745,7 +688,7 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<T> a, const __g
         for (int k = max(ngr - kStages, 0); k < ngr; ++k) mbar_wait(&full[k % kStages], (uint32_t)((k / kStages) & 1));
     }
     if (plain) {
-        if constexpr (HRAW) {
+        if constexpr (SHAK) {
             fold_lanes<4>(Qp, 0, sacc, tid);
             fold_lanes<5>(Hp, 4, sacc, tid);
 #pragma unroll
@@ -768,7 +711,7 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<T> a, const __g
     } else if (zero) {
 #pragma unroll
         for (int m = 0; m < 4; ++m) a.pout[((long)split * 4 + m) * nc + cell] = 0;
-        if constexpr (HRAW) {
+        if constexpr (SHAK) {
 #pragma unroll
             for (int m = 0; m < 5; ++m) a.hout[((long)split * 5 + m) * nc + cell] = 0;
             if (split == 0) {
@@ -2247,7 +2190,7 @@ inline int nblk(long n, int b) { return (int)((n + b - 1) / b); }
 
 // The bulk kernel of a precision, its threads and shared memory.
 template <bool MUSCL, bool REC, bool SHAK> struct BulkKernel {
-    static constexpr auto kernel32 = k_bulk<float, MUSCL, REC, SHAK>;
+    static constexpr auto kernel32 = k_bulk<MUSCL, REC, SHAK>;
     static constexpr auto kernel64 = k_bulk64<MUSCL, REC, SHAK>;
     static constexpr size_t smem32 = (size_t)kStages * (kStageBytes + kTabBytes) + 2 * kStages * sizeof(uint64_t) +
                                      (SHAK ? kSaccBytes : 0);
