@@ -550,7 +550,7 @@ template <int CT> __device__ __forceinline__ double cell_sum(double x)
 // the one of M, so each value is as exact as its own exp2, tails included, at
 // any spacing dv against sqrt(T) and one FP64 multiplication a velocity.  (A
 // recurrence M(v + dv) = M R, R(v + dv) = R Q from a row's start took two
-// multiplications, 256^2 x 32^2 4.31 ms a launch against 4.14, and lost M
+// multiplications, 256^2 x 32^2 4.31 ms a launch against 4.19, and lost M
 // where it underflowed at the start of a coarse row.)
 template <int CT>
 __device__ __forceinline__ void put_factors(double *mx, long nc, int k, int nvx, int n, double vmin, double dv, double ux,

@@ -724,11 +724,11 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<float> a, const
 
 // ------------------------------------------------------------ FP64 bulk kernel
 // On this part an FP64 operation holds the pipe of an SM's quarter for 64
-// clocks a warp, so this kernel counts FP64 operations and little else: 32 a
-// velocity pair (f, g) and cell, against 64 of the form it replaced (one cell
+// clocks a warp, so this kernel counts FP64 operations and little else: 33 a
+// velocity pair (f, g) and cell, against 62 of the form it replaced (one cell
 // per thread, every difference from both sides, weights on every face, a
 // limiter whose magnitudes the compiler formed on the FP64 pipe): 7.90 ->
-// 4.14 ms a launch at 256^2 x 32^2, limited fluxes (with k_cell64, 0.15 ms).
+// 4.19 ms a launch at 256^2 x 32^2, limited fluxes (with k_cell64, 0.15 ms).
 //
 // Block = 32 x 8 cells, four warps of 32 cells in x and two rows.  A thread
 // takes its two cells in upwind order of v_y: they share the face between

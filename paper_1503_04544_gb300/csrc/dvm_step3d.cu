@@ -17,11 +17,12 @@
 // last block sums them in list order), k_bulk3 (every gas cell that is a
 // control volume on its own), k_special3 (cut and merged control volumes).
 // k_bulk3 assigns one thread to a column of cells along z; a warp covers 32
-// consecutive cells along x, so the velocity of a group (hence the upwind
-// side along y and z) is uniform across the warp.  The velocity groups are
-// split over blockIdx.z; each block streams the planes of its column through
-// shared memory with TMA, writes the new state and accumulates the moments of
-// the new state for the next step.
+// consecutive cells of the block's tile, row after row (a row may end inside a
+// warp), at the velocities of one group, so the upwind side along y and z is
+// uniform across the warp.  The velocity groups are split over blockIdx.z;
+// each block streams the planes of its column through shared memory with TMA,
+// writes the new state and accumulates the moments of the new state for the
+// next step.
 #include <cudaTypedefs.h>
 
 #include <cstdio>
@@ -273,13 +274,15 @@ __global__ void __launch_bounds__(128) k_cell64_3(Bulk3Args<double> a, double *c
 // whole column before the group's planes) times the row's factor of v_y and
 // v_z (one exp2 a row): one FP64 multiplication a velocity instead of an exp2.
 //
-// FP32 is bound by issue slots (70 warp instructions a velocity and 32 cells,
-// 24 of them on the half-rate ALU pipe) and by waits for planes; FP64 by the
-// FP64 pipe (two lanes a clock; 25 operations a velocity).  The form before
-// this one (a thread per column in fixed z order, both z faces' planes read,
-// exp2 per velocity, velocity by velocity moments) took, a launch: FP32 64^3 x
-// 20^3 9.72 ms, now 7.2; 96^3 x 20^3 30.6, now 23.4; Shakhov 45 x 50 x 37 x
-// (14, 15, 13) 2.13, now 1.53; FP64 40^3 x 12^3 20.8, now 7.7.
+// FP32 is bound by issue slots (64^3 x 12^3: 77 warp instructions a velocity
+// and 32 cells, 27 of them on the half-rate ALU pipe) and by waits for planes;
+// FP64 by the FP64 pipe (two lanes a clock; 29 operations a velocity with its
+// share of the row's, at 12 velocities a row).  The form before this one (a
+// thread per column in fixed z order, both z faces' planes read, exp2 per
+// velocity, velocity by velocity moments) took, a launch: FP32 64^3 x 20^3
+// 9.72 ms, now 7.3; 96^3 x 20^3 30.6, now 23.4; Shakhov 45 x 50 x 37 x (14, 15,
+// 13) 2.13, now 1.67; FP64 40^3 x 12^3 20.8, now 7.4 (7.7 with a recurrence
+// for the Maxwellian).
 //
 // With SHAK (the Shakhov model, FP32) the cells relax towards F_S = M [1 +
 // k c.q (|c|^2/T - 5)], k = (1 - Pr) / (5 rho T^2), with the heat flux q of
@@ -1934,12 +1937,11 @@ cudaError_t split_relax3d_t(dvm_ctx *c, const double *xbuf)
 // grid with the least work: a tile takes the time of its warps (in fours,
 // one per SM sub-partition) and of about six more (latencies that few warps do
 // not cover), weighted with a fifth of the halo it re-reads and a little for
-// short rows; what fits a ring
-// slot.  64^2 cells: 32 x 16.  FP32, 45 x 50 cells: 45 x 11, 1.53 ms a launch
-// (37 planes, 14 x 15 x 13 velocities, Shakhov) against 1.82 with 16 x 32 and
-// 2.66 with 5 x 50 (as few lanes outside the grid, but 8 warps an SM).  FP64,
-// 40^2: 40 x 6, 7.7 ms (40 planes, 12^3) against 9.4 with 16 x 16 and 12.1
-// with 32 x 8.
+// short rows; what fits a ring slot.  64^2 cells: 32 x 16.  FP32, 45 x 50
+// cells: 45 x 11, 1.53 ms a launch within a step (37 planes, 14 x 15 x 13
+// velocities, Shakhov) against 1.82 with 16 x 32 and 2.66 with 5 x 50 (as few
+// lanes outside the grid, but 8 warps an SM).  FP64, 40^2: 40 x 6, 7.7 ms (40
+// planes, 12^3, at the time) against 9.4 with 16 x 16 and 12.1 with 32 x 8.
 void tile3d(const dvm_ctx *c, int *tx, int *ty)
 {
     const int threads = 32 * (c->prec == DVM_FP32 ? warps3<float>() : warps3<double>());
