@@ -724,7 +724,7 @@ __global__ void __launch_bounds__(32 * kRows, 2) k_bulk(BulkArgs<float> a, const
 
 // ------------------------------------------------------------ FP64 bulk kernel
 // On this part an FP64 operation holds the pipe of an SM's quarter for 64
-// clocks a warp, so this kernel counts FP64 operations and little else: 33 a
+// clocks a warp, so this kernel counts FP64 operations and little else: 32 a
 // velocity pair (f, g) and cell, against 62 of the form it replaced (one cell
 // per thread, every difference from both sides, weights on every face, a
 // limiter whose magnitudes the compiler formed on the FP64 pipe): 7.90 ->
